@@ -105,7 +105,10 @@ typedef enum { LBW_EQ_CURVILINEAR = 0, LBW_EQ_MOMENT_MATCHING = 1, LBW_EQ_HERMIT
  * from the closed-form metric in the arithmetic type (FP32 or FP64), by the producer warp's
  * lanes; only single lattices (not ensembles) with FP32 or FP64 storage on the tile kernel
  * (q2 extent a multiple of 64, non-periodic q1) accept it.  AUTO takes the table, the faster of
- * the two on the benchmark lattices (measured: 472 against 966 us per torus step). */
+ * the two on the benchmark lattices (measured: 472 against 966 us per torus step), and advances
+ * lattices that the SMs hold (up to 620,000 nodes; FP64, and 16-bit storage on the tile kernel:
+ * 300,000) many steps per launch, with the table rows kept in shared memory; TABLE and ANALYTIC
+ * always launch once per step. */
 typedef enum { LBW_GEOM_AUTO = 0, LBW_GEOM_TABLE = 1, LBW_GEOM_ANALYTIC = 2 } lbw_geom_mode;
 
 /* A Gaussian pulse P0 = amp exp(-|X - x|^2 / (2 sigma^2)) in the embedding distance. */
@@ -134,7 +137,7 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
 lbw_status lbw_init(lbw_grid* g, const lbw_pulse* host_pulses, int32_t n_pulses);
 
 /* Advance n_steps >= 0 time steps (one fused stream + collide launch per step, captured in
- * CUDA graphs).  Asynchronous on the grid's stream; registered probes record P after each
+ * CUDA graphs; small lattices many steps per cooperative launch, see lbw_geom_mode).  Asynchronous on the grid's stream; registered probes record P after each
  * step's streaming.  Every device wait inside a step is bounded: if one runs out, the kernel
  * raises a flag instead of hanging, and the next call that synchronises (lbw_probe_read,
  * lbw_spectrum, lbw_get_field, lbw_get_populations) returns LBW_ETIMEOUT until lbw_init. */
@@ -146,8 +149,8 @@ lbw_status lbw_step(lbw_grid* g, int64_t n_steps);
  * amp sin(omega t): kind 0 imposes P = amp sin(omega t) (f = f^eq(sqrt(g) P, 0)), kind 1
  * imposes J'_z (the q3 component of J') = amp sin(omega t) and keeps the node's rho.
  * omega in rad / step.  n = 0 removes the sources.  LBW_EINVAL for nodes outside the lattice
- * or kind not 0 / 1.  Without sources a step is a single kernel launch; with sources a small
- * second launch per step applies them. */
+ * or kind not 0 / 1.  Where a step is a launch of its own, a small second launch applies the
+ * sources. */
 lbw_status lbw_source(lbw_grid* g, const int32_t* host_q, int32_t n, int32_t kind, double amp,
                       double omega);
 
@@ -231,7 +234,9 @@ void lbw_destroy(lbw_grid* g);
  * Ensembles: many independent lattices of uneven sizes (each a full instance of the scheme
  * above with its own geometry and probes) advanced together.  One time step of the whole
  * ensemble is one launch of a persistent kernel over a (member, tile, q3 segment) work list;
- * steps are captured in CUDA graphs.  A member's results agree with the same lattice run
+ * steps are captured in CUDA graphs.  Ensembles of small members advance many steps per
+ * cooperative launch instead, in turns of as many members as the SMs hold, until the caller
+ * sets a launch shape or the autotuner finds one faster.  A member's results agree with the same lattice run
  * alone to the rounding of its storage (the kernels may sum in another order).
  * ---------------------------------------------------------------------------------------- */
 typedef struct lbw_batch lbw_batch; /* opaque, library-owned */

@@ -21,6 +21,7 @@
 
 #include "lbw_internal.h"
 #include "lbw_march.cuh"
+#include "lbw_resident.h"
 #include "lbw_tma.cuh"
 
 namespace lbw {
@@ -1014,6 +1015,7 @@ struct lbw_batch {
   bool tma = false;              // padded members on the TMA-staged kernel
   bool rowk = false;             // ... and every member fits a full-row tile (shape.by == 0)
   void* maps = nullptr;          // device: per member tensor maps (buffer 0, buffer 1, table)
+  Resident* res = nullptr;       // small members: many steps per launch (nullptr: a launch per step)
   // harmonic sources of all members (offsets from the buffer base), applied after each step
   int nsrc = 0, src_kind = 0;
   double src_amp = 0.0;
@@ -1036,35 +1038,14 @@ void drop_graphs(lbw_batch* b) {
 
 template <typename S>
 void fill_args(lbw_batch* b, int m, int src, StepArgs<S>& a) {
-  using R = typename Store<S>::R;
-  const Grid& g = b->views[m];
-  std::memset(&a, 0, sizeof(a));
-  a.fin = reinterpret_cast<const S*>(g.f[src]);
-  a.fout = reinterpret_cast<S*>(g.f[1 - src]);
-  a.tab = reinterpret_cast<const R*>(g.table);
-  a.n1 = g.d.n[0]; a.n2 = g.d.n[1]; a.n3 = g.d.n[2];
+  a = step_args<S>(b->views[m], src);
   a.lz = b->shape.lz;
-  a.nn = g.nn;
-  for (int k = 0; k < 6; ++k) a.bc[k] = g.d.bc[k];
-  a.damping = (R)g.d.damping;
-  a.cs2 = (R)g.d.cs2;
-  a.two_w0 = (R)(2.0 * g.w0);
-  for (int i = 0; i < 7; ++i) {
-    const double w = i == 0 ? g.w0 : g.w1;
-    a.w[i] = (R)w;
-    a.inv_w[i] = (R)(1.0 / w);
-  }
-  a.s2lo = g.d.bc[2] == LBW_BC_ANTIBOUNCE ? R(-1) : R(1);
-  a.s2hi = g.d.bc[3] == LBW_BC_ANTIBOUNCE ? R(-1) : R(1);
   a.nprobe = b->nprobe;
   a.probe_q = b->probe_q ? b->probe_q + (size_t)m * b->nprobe * 3 : nullptr;
   a.series = b->series ? b->series + (size_t)m * b->nprobe * b->cap : nullptr;
   a.cap = b->cap;
   a.counters = b->counters;
   a.nblocks = 0;
-  a.pitch = g.pitch ? g.pitch : g.d.n[1];
-  a.col0 = g.col0;
-  a.ps = pop_stride(&g);
 }
 
 template <typename S>
@@ -1298,9 +1279,23 @@ lbw_status ensure_graph(lbw_batch* b, int start, int len) {
   return LBW_OK;
 }
 
+// `n` time steps on the resident kernel
+cudaError_t run_resident(lbw_batch* b, int n) {
+  const ResState rs{{b->f[0], b->f[1]}, b->cur, b->counters, nullptr, b->nprobe, b->cap,
+                    static_cast<const SourceEntry*>(b->src), b->src_kind, b->src_amp, b->stream};
+  const cudaError_t e = resident_run(b->res, nullptr, b->members[0], rs, n);
+  if (e == cudaSuccess) b->cur ^= n & 1;
+  return e;
+}
+
 lbw_status advance(lbw_batch* b, int64_t n_steps) {
   const int chain = 64;
   int64_t left = n_steps;
+  while (b->res && left > 0) {
+    const int n = (int)std::min<int64_t>(left, kResChunk);
+    LBW_CUDA(run_resident(b, n));
+    left -= n;
+  }
   if (left >= chain) {
     for (int start = 0; start < 2; ++start) {
       lbw_status st = ensure_graph(b, start, chain);
@@ -1470,6 +1465,16 @@ lbw_status lbw_batch_create(const lbw_grid_desc* descs, int32_t n, void* stream,
   }
   lbw_status st = refresh(b);
   if (st != LBW_OK) return cleanup(st);
+  // Small members run many steps per launch, in turns of what the SMs hold: always ahead of the
+  // register-pipelined kernel (41 pipes of 10,000 FP32 nodes: 120 -> 11.7 us per step of all, 175:
+  // 470 -> 44.5) and of the FP64 tiles (1.3e6 nodes: 231 -> 137), of FP32 tiles up to one turn
+  // (0.62e6 nodes: 19.3 -> 17.2; 1.3e6: 25.5 against 36.2), of 16-bit tiles up to half of one.
+  std::vector<const Grid*> lattices;
+  for (const Grid& g : b->views) lattices.push_back(&g);
+  const bool wide = b->prec == LBW_F64 || b->prec == LBW_F32;
+  st = resident_create(lattices.data(), n, b->prec, b->tma,
+                       !b->tma || b->prec == LBW_F64 ? 1LL << 40 : (wide ? 640000 : 300000), b->stream, &b->res);
+  if (st != LBW_OK) return cleanup(st);
   LBW_CUDA(cudaStreamSynchronize(b->stream));
   *out = b;
   return LBW_OK;
@@ -1487,6 +1492,7 @@ void lbw_batch_destroy(lbw_batch* b) {
   if (b->items) cudaFreeAsync(b->items, b->stream);
   if (b->maps) cudaFreeAsync(b->maps, b->stream);
   if (b->src) cudaFreeAsync(b->src, b->stream);
+  resident_destroy(b->res, b->stream);
   if (b->probe_q) cudaFreeAsync(b->probe_q, b->stream);
   if (b->series) cudaFreeAsync(b->series, b->stream);
   cudaStreamSynchronize(b->stream);
@@ -1603,7 +1609,7 @@ lbw_status lbw_batch_source(lbw_batch* b, const int32_t* host_q, int32_t per_mem
     b->src_kind = kind;
     b->src_amp = amp;
   }
-  return LBW_OK;
+  return b->res ? resident_sources(b->res, host_q, per_member, b->stream) : LBW_OK;
 }
 
 lbw_status lbw_batch_step(lbw_batch* b, int64_t n_steps) {
@@ -1709,13 +1715,14 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
   if (trial_steps < 1 || trial_steps > 1000) return fail(LBW_EINVAL, "1 <= trial_steps <= 1000");
   const std::string sig = signature(b);
   std::string line;
-  bool cached = false;
+  bool cached = false, resident = false;
   Shape best = b->shape;
   if (cache_path) {  // JSON lines: {"signature": "...", "by": 8, "lz": 32, "cps": 2, "ms": ...}
     std::ifstream in(cache_path);
     while (in && std::getline(in, line)) {
       if (line.find("\"" + sig + "\"") == std::string::npos) continue;
       Shape s;
+      resident = line.find("\"resident\": 1") != std::string::npos;
       if (sscanf(line.c_str() + line.find("\"by\""), "\"by\": %d, \"lz\": %d, \"cps\": %d", &s.by, &s.lz,
                  &s.cps) == 3) {
         best = s;
@@ -1723,6 +1730,7 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
       }
     }
   }
+  const Shape start = b->shape;
   double best_ms = -1.0;
   std::ostringstream rep;
   if (!cached) {
@@ -1764,21 +1772,44 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
             best = b->shape;
           }
         }
+    if (b->res) {  // against the kernel that small members start with
+      b->shape = start;
+      lbw_status st = refresh(b);
+      if (st != LBW_OK) return st;
+      LBW_CUDA(run_resident(b, 2));  // warm-up
+      LBW_CUDA(cudaEventRecord(e0, b->stream));
+      for (int s = 0; s < trial_steps; s += kResChunk) LBW_CUDA(run_resident(b, std::min(kResChunk, trial_steps - s)));
+      LBW_CUDA(cudaEventRecord(e1, b->stream));
+      LBW_CUDA(cudaEventSynchronize(e1));
+      float ms = 0.f;
+      LBW_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+      ms /= trial_steps;
+      rep << "resident ms=" << ms << "\n";
+      resident = ms < best_ms;
+      if (resident) {
+        best_ms = ms;
+        best = start;
+      }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (cache_path) {
       std::ofstream o(cache_path, std::ios::app);
       o << "{\"signature\": \"" << sig << "\", \"by\": " << best.by << ", \"lz\": " << best.lz
-        << ", \"cps\": " << best.cps << ", \"ms\": " << best_ms << "}\n";
+        << ", \"cps\": " << best.cps << ", \"ms\": " << best_ms << (resident ? ", \"resident\": 1" : "") << "}\n";
     }
   }
   b->shape = best;
+  if (!resident) {
+    resident_destroy(b->res, b->stream);
+    b->res = nullptr;
+  }
   lbw_status st = refresh(b);
   if (st != LBW_OK) return st;
   // trial steps ran on the ensemble's buffers: callers tune before lbw_batch_init
   LBW_CUDA(cudaMemsetAsync(b->counters, 0, 4 * sizeof(unsigned long long), b->stream));
   LBW_CUDA(cudaStreamSynchronize(b->stream));
-  rep << (cached ? "cached " : "chosen ") << "by=" << best.by << " lz=" << best.lz << " cps=" << best.cps
+  rep << (cached ? "cached " : "chosen ") << (resident ? "resident " : "") << "by=" << best.by << " lz=" << best.lz << " cps=" << best.cps
       << " signature=" << sig << "\n";
   if (report && report_cap > 0) {
     const std::string r = rep.str();
@@ -1798,6 +1829,10 @@ lbw_status lbw_batch_set_shape(lbw_batch* b, int32_t tile_rows, int32_t seg_plan
   if (ctas_per_sm < 1 || ctas_per_sm > std::max(1, cps_max) || (b->tma && cps_max == 0))
     return fail(LBW_EINVAL, "ctas_per_sm must be in [1, what the kernel keeps resident]");
   const Shape old = b->shape;
+  // a shape chosen by the caller is one of the tiled kernels'
+  const bool was_resident = b->res != nullptr;
+  resident_destroy(b->res, b->stream);
+  b->res = nullptr;
   b->shape = Shape{tile_rows, seg_planes, ctas_per_sm};
   lbw_status st = refresh(b);
   if (st != LBW_OK) {
@@ -1805,7 +1840,7 @@ lbw_status lbw_batch_set_shape(lbw_batch* b, int32_t tile_rows, int32_t seg_plan
     refresh(b);
     return st;
   }
-  if (b->tma && old.by == 0 && tile_rows != 0) {  // the 64-column kernel reads ghost columns
+  if (b->tma && (old.by == 0 || was_resident) && tile_rows != 0) {  // the 64-column kernel reads ghost columns
     for (int m = 0; m < b->n; ++m) {
       const Grid& g = b->views[m];
       const long long rows = 7LL * g.d.n[0] * g.d.n[2];

@@ -28,6 +28,8 @@ enum TableSlot {
 
 constexpr int kMaxProbes = 64;
 
+struct Resident;  // plan of the multi-step kernel (lbw_resident.h)
+
 struct Grid {
   lbw_grid_desc d;
   cudaStream_t stream = nullptr;
@@ -61,6 +63,7 @@ struct Grid {
   double src_amp = 0.0;
   alignas(64) unsigned char tmaps[5 * 128];  // tensor maps: f[0] main/halo, f[1] main/halo, table
   dim3 grid_dim;
+  Resident* res = nullptr;  // small lattices: many steps per launch (nullptr: a launch per step)
   // captured step chains, one per parity of the starting buffer
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   int graph_len = 0;

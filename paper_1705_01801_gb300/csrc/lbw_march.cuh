@@ -170,6 +170,86 @@ struct StepArgs {
   GeomArgs<R> geo;  // closed-form geometry (used by the tile kernel in the analytic mode)
 };
 
+// Launch arguments of a lattice whose buffer `src` holds the current state.
+template <typename S>
+StepArgs<S> step_args(const Grid& lattice, int src) {
+  using R = typename Store<S>::R;
+  const Grid* g = &lattice;
+  StepArgs<S> a;
+  a.fin = reinterpret_cast<const S*>(g->f[src]);
+  a.fout = reinterpret_cast<S*>(g->f[1 - src]);
+  a.tab = reinterpret_cast<const R*>(g->table);
+  a.n1 = g->d.n[0]; a.n2 = g->d.n[1]; a.n3 = g->d.n[2];
+  a.lz = g->lz;
+  a.nn = g->nn;
+  for (int k = 0; k < 6; ++k) a.bc[k] = g->d.bc[k];
+  a.damping = (R)g->d.damping;
+  double eq_e, eq_two0;
+  equilibrium_coefs(g->d, &eq_e, &eq_two0);
+  a.cs2 = (R)eq_e;  // cs^2 for the paper's method; the Cartesian equilibria change it
+  a.two_w0 = (R)eq_two0;
+  for (int i = 0; i < 7; ++i) {
+    double w = i == 0 ? g->w0 : g->w1;
+    a.w[i] = (R)w;
+    a.inv_w[i] = (R)(1.0 / w);
+  }
+  a.s2lo = g->d.bc[2] == LBW_BC_ANTIBOUNCE ? R(-1) : R(1);
+  a.s2hi = g->d.bc[3] == LBW_BC_ANTIBOUNCE ? R(-1) : R(1);
+  a.nprobe = g->nprobe;
+  a.probe_q = g->probe_q;
+  a.series = g->series;
+  a.cap = g->cap;
+  a.counters = g->counters;
+  a.nblocks = g->grid_dim.x * g->grid_dim.y * g->grid_dim.z;
+  a.pitch = g->pitch ? g->pitch : g->d.n[1];
+  a.col0 = g->col0;
+  a.ps = pop_stride(g);
+  a.geo.kind = g->d.kind;
+  a.geo.profile = g->d.horn_profile;
+  a.geo.x0r = (R)g->d.x0[0];
+  a.geo.x0w = (R)g->d.x0[2];
+  a.geo.h0 = (R)g->d.h[0];
+  a.geo.h1 = (R)g->d.h[1];
+  a.geo.h2 = (R)g->d.h[2];
+  a.geo.g0 = (R)g->d.geom[0];
+  a.geo.g1 = (R)g->d.geom[1];
+  a.geo.g2 = (R)g->d.geom[2];
+  a.geo.c2 = (R)(g->d.c * g->d.c);
+  a.geo.cs2 = (R)g->d.cs2;
+  return a;
+}
+
+// Reading of the paper's sources (ring, plate and point sources of Sec. IV impose P, or J'_z
+// for the plate, as C sin(omega t)): after step t the source node's post-collision
+// populations are replaced by the equilibrium carrying the imposed value v = C sin(omega t);
+// kind 0: f_i = f_i^eq(sqrt(g) v, 0); kind 1: f_i = f_i^eq(rho, (0, 0, sqrt(g) v)) with the
+// node's own rho.  16-bit formats store f_i / w_i.
+template <typename S>
+__device__ __forceinline__ void impose_source(S* base, const SourceEntry& s, int kind, double v) {
+  const double cs2 = s.cs2;
+  const double w0 = 1.0 - 3.0 * cs2, w1 = 0.5 * cs2;
+  S* f = base + s.off;
+  double rho = 0.0, j3 = 0.0;
+  if (kind == 0) {
+    rho = s.sg * v;
+  } else {
+    for (int i = 0; i < 7; ++i) {
+      double x = (double)Store<S>::ld_smem(f + (long long)i * s.ps);
+      if (Store<S>::kScaled) x *= (i == 0 ? w0 : w1);
+      rho += x;
+    }
+    j3 = s.sg * v;
+  }
+  for (int i = 0; i < 7; ++i) {
+    const double xi3 = i == 5 ? 1.0 : (i == 6 ? -1.0 : 0.0);
+    double val = i == 0 ? w0 * rho : w1 * (rho + xi3 * j3 / cs2);
+    if (Store<S>::kScaled) val /= (i == 0 ? w0 : w1);
+    const typename Store<S>::R r = (typename Store<S>::R)val;
+    Store<S>::st(f + (long long)i * s.ps, r);
+    if (s.ghost != 0) Store<S>::st(f + (long long)i * s.ps + s.ghost, r);
+  }
+}
+
 __device__ __forceinline__ long long node(int q1, int q2, int q3, int n1, int n2) {
   return ((long long)q3 * n1 + q1) * n2 + q2;
 }

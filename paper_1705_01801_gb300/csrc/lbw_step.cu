@@ -810,53 +810,6 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
   }
 }
 
-template <typename S>
-StepArgs<S> make_args(Grid* g, int src) {
-  using R = typename Store<S>::R;
-  StepArgs<S> a;
-  a.fin = reinterpret_cast<const S*>(g->f[src]);
-  a.fout = reinterpret_cast<S*>(g->f[1 - src]);
-  a.tab = reinterpret_cast<const R*>(g->table);
-  a.n1 = g->d.n[0]; a.n2 = g->d.n[1]; a.n3 = g->d.n[2];
-  a.lz = g->lz;
-  a.nn = g->nn;
-  for (int k = 0; k < 6; ++k) a.bc[k] = g->d.bc[k];
-  a.damping = (R)g->d.damping;
-  double eq_e, eq_two0;
-  equilibrium_coefs(g->d, &eq_e, &eq_two0);
-  a.cs2 = (R)eq_e;  // cs^2 for the paper's method; the Cartesian equilibria change it
-  a.two_w0 = (R)eq_two0;
-  for (int i = 0; i < 7; ++i) {
-    double w = i == 0 ? g->w0 : g->w1;
-    a.w[i] = (R)w;
-    a.inv_w[i] = (R)(1.0 / w);
-  }
-  a.s2lo = g->d.bc[2] == LBW_BC_ANTIBOUNCE ? R(-1) : R(1);
-  a.s2hi = g->d.bc[3] == LBW_BC_ANTIBOUNCE ? R(-1) : R(1);
-  a.nprobe = g->nprobe;
-  a.probe_q = g->probe_q;
-  a.series = g->series;
-  a.cap = g->cap;
-  a.counters = g->counters;
-  a.nblocks = g->grid_dim.x * g->grid_dim.y * g->grid_dim.z;
-  a.pitch = g->pitch ? g->pitch : g->d.n[1];
-  a.col0 = g->col0;
-  a.ps = pop_stride(g);
-  a.geo.kind = g->d.kind;
-  a.geo.profile = g->d.horn_profile;
-  a.geo.x0r = (R)g->d.x0[0];
-  a.geo.x0w = (R)g->d.x0[2];
-  a.geo.h0 = (R)g->d.h[0];
-  a.geo.h1 = (R)g->d.h[1];
-  a.geo.h2 = (R)g->d.h[2];
-  a.geo.g0 = (R)g->d.geom[0];
-  a.geo.g1 = (R)g->d.geom[1];
-  a.geo.g2 = (R)g->d.geom[2];
-  a.geo.c2 = (R)(g->d.c * g->d.c);
-  a.geo.cs2 = (R)g->d.cs2;
-  return a;
-}
-
 template <typename S, int BY, int NPT, bool ANA>
 constexpr size_t tma_smem_bytes() {
   using R = typename Store<S>::R;
@@ -891,7 +844,7 @@ auto tma_dispatch(int by, int npt, bool ana, F&& f) {
 template <typename S>
 cudaError_t launch_step_t(Grid* g, int src) {
   using R = typename Store<S>::R;
-  StepArgs<S> a = make_args<S>(g, src);
+  StepArgs<S> a = step_args<S>(*g, src);
   if (g->tma_by > 0) {
     const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(g->tmaps);
     // consecutive steps overlap launch and prologue with the previous step's tail
@@ -1130,47 +1083,20 @@ cudaError_t launch_init_t(Grid* g, const double* d_pulses, int npulse) {
       g->d.n[2], rho0);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  StepArgs<S> a = make_args<S>(g, 1 - g->cur);  // fout = current buffer
+  StepArgs<S> a = step_args<S>(*g, 1 - g->cur);  // fout = current buffer
   init_f_kernel<S><<<blocks, threads, 0, g->stream>>>(a, rho0);
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- harmonic sources -------
 
-// Reading of the paper's sources (ring, plate and point sources of Sec. IV impose P, or J'_z
-// for the plate, as C sin(omega t)): after step t the source node's post-collision
-// populations are replaced by the equilibrium carrying the imposed value; kind 0:
-// f_i = f_i^eq(sqrt(g) C sin(omega t), 0); kind 1: f_i = f_i^eq(rho, (0, 0, sqrt(g) C sin(omega t)))
-// with the node's own rho.  16-bit formats store f_i / w_i.
 template <typename S>
 __global__ void source_kernel(S* __restrict__ base, const SourceEntry* __restrict__ e, int n, int kind,
                               double amp, const unsigned long long* __restrict__ counters) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const SourceEntry s = e[k];
-  const double cs2 = s.cs2;
-  const double w0 = 1.0 - 3.0 * cs2, w1 = 0.5 * cs2;
-  const double v = amp * sin(s.omega * (double)counters[0]);
-  S* f = base + s.off;
-  double rho = 0.0, j3 = 0.0;
-  if (kind == 0) {
-    rho = s.sg * v;
-  } else {
-    for (int i = 0; i < 7; ++i) {
-      double x = (double)Store<S>::ld(f + (long long)i * s.ps);
-      if (Store<S>::kScaled) x *= (i == 0 ? w0 : w1);
-      rho += x;
-    }
-    j3 = s.sg * v;
-  }
-  for (int i = 0; i < 7; ++i) {
-    const double xi3 = i == 5 ? 1.0 : (i == 6 ? -1.0 : 0.0);
-    double val = i == 0 ? w0 * rho : w1 * (rho + xi3 * j3 / cs2);
-    if (Store<S>::kScaled) val /= (i == 0 ? w0 : w1);
-    const typename Store<S>::R r = (typename Store<S>::R)val;
-    Store<S>::st(f + (long long)i * s.ps, r);
-    if (s.ghost != 0) Store<S>::st(f + (long long)i * s.ps + s.ghost, r);
-  }
+  impose_source(base, s, kind, amp * sin(s.omega * (double)counters[0]));
 }
 
 // ---------------------------------------------------------------- read-out ---------------
