@@ -167,7 +167,7 @@ lbw_status lbw_probe_read(lbw_grid* g, double* host_out, int64_t cap_per_probe,
  * (probe = -1), computed on the device: mean removed, Hann window, zero padding to the
  * smallest power of two >= 4 T, |DFT|^2, the k strongest local maxima above 1e-3 of the
  * largest (sorted by frequency), each refined by a parabola through log-power and 40
- * golden-section steps on the windowed DTFT over +-1 bin.  host_freq / host_amp receive up
+ * golden-section steps on the windowed DTFT over +-1 bin (evaluated from its moments).  host_freq / host_amp receive up
  * to k values (rad/step, amplitude 2 |X| / sum w); *n_found how many.  LBW_EUNSTABLE (and no
  * peaks) when the series holds a non-finite value; the same holds for every spectrum call. */
 lbw_status lbw_spectrum(lbw_grid* g, int32_t probe, int32_t k, double* host_freq,
@@ -192,7 +192,7 @@ lbw_status lbw_spectrum_series(const double* host_x, int64_t T, int32_t n_series
  *  - dev_x: T doubles in device memory owned by the caller (one series, 4 <= T <= 16384;
  *    larger T is rejected with LBW_EINVAL).  host_freq / host_amp: room for k values;
  *    *host_n_found: how many.  k in [1, 64].
- *  - All workspace lives in one fixed device array of about 2.6 MB inside the library, which
+ *  - All workspace lives in one fixed device array of about 2 MB inside the library, which
  *    every GPU that loads the library holds until the process exits.  No call here allocates
  *    or frees device memory.
  *  - The array's device address is looked up (cudaGetSymbolAddress) by the first call in each

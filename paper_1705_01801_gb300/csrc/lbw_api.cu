@@ -568,8 +568,8 @@ lbw_status lbw_spectrum(lbw_grid* g, int32_t probe, int32_t k, double* host_freq
   if (st != LBW_OK) return st;
   if (rec < 4) return fail(LBW_ESTATE, "fewer than 4 recorded samples");
   const double* base = g->series + (probe >= 0 ? (size_t)probe * g->cap : 0);
-  return spectrum_device(base, (int64_t)rec, probe >= 0 ? 1 : g->nprobe, (int32_t)g->cap,
-                         probe < 0, k, g->stream, host_freq, host_amp, n_found);
+  return spectrum_device(base, (int64_t)rec, 1, 0, probe >= 0 ? 1 : g->nprobe, g->cap, k, g->stream, host_freq,
+                         host_amp, n_found);
 }
 
 lbw_status lbw_spectrum_lowest(lbw_grid* g, int32_t probe, int32_t k, double rel_power,
@@ -583,8 +583,8 @@ lbw_status lbw_spectrum_lowest(lbw_grid* g, int32_t probe, int32_t k, double rel
   if (st != LBW_OK) return st;
   if (rec < 4) return fail(LBW_ESTATE, "fewer than 4 recorded samples");
   const double* base = g->series + (probe >= 0 ? (size_t)probe * g->cap : 0);
-  return spectrum_device(base, (int64_t)rec, probe >= 0 ? 1 : g->nprobe, (int32_t)g->cap,
-                         probe < 0, k, g->stream, host_freq, host_amp, n_found, true, rel_power);
+  return spectrum_device(base, (int64_t)rec, 1, 0, probe >= 0 ? 1 : g->nprobe, g->cap, k, g->stream, host_freq,
+                         host_amp, n_found, true, rel_power);
 }
 
 lbw_status lbw_spectrum_series(const double* host_x, int64_t T, int32_t n_series, int32_t k,
@@ -602,10 +602,7 @@ lbw_status lbw_spectrum_series(const double* host_x, int64_t T, int32_t n_series
     cudaFreeAsync(d_x, s);
     return cuda_fail(e, "spectrum upload");
   }
-  lbw_status st = LBW_OK;
-  for (int j = 0; j < n_series && st == LBW_OK; ++j)
-    st = spectrum_device(d_x + (size_t)j * T, T, 1, (int32_t)T, false, k, s, host_freq + (size_t)j * k,
-                         host_amp + (size_t)j * k, host_n_found + j);
+  const lbw_status st = spectrum_device(d_x, T, n_series, T, 1, T, k, s, host_freq, host_amp, host_n_found);
   cudaFreeAsync(d_x, s);
   cudaStreamSynchronize(s);
   return st;

@@ -1665,13 +1665,8 @@ lbw_status lbw_batch_spectrum(lbw_batch* b, int32_t k, double* host_freq, double
   lbw_status st0 = batch_counters(b, &rec);
   if (st0 != LBW_OK) return st0;
   if (rec < 4) return fail(LBW_ESTATE, "fewer than 4 recorded samples");
-  for (int m = 0; m < b->n; ++m) {
-    lbw_status st = spectrum_device(b->series + (size_t)m * b->nprobe * b->cap, (int64_t)rec, b->nprobe,
-                                    (int32_t)b->cap, true, k, b->stream, host_freq + (size_t)m * k,
-                                    host_amp + (size_t)m * k, host_n_found + m);
-    if (st != LBW_OK) return st;
-  }
-  return LBW_OK;
+  return spectrum_device(b->series, (int64_t)rec, b->n, b->nprobe * b->cap, b->nprobe, b->cap, k, b->stream, host_freq,
+                         host_amp, host_n_found);
 }
 
 lbw_status lbw_batch_spectrum_lowest(lbw_batch* b, int32_t k, double rel_power, double* host_freq,
@@ -1684,13 +1679,8 @@ lbw_status lbw_batch_spectrum_lowest(lbw_batch* b, int32_t k, double rel_power, 
   lbw_status st0 = batch_counters(b, &rec);
   if (st0 != LBW_OK) return st0;
   if (rec < 4) return fail(LBW_ESTATE, "fewer than 4 recorded samples");
-  for (int m = 0; m < b->n; ++m) {
-    lbw_status st = spectrum_device(b->series + (size_t)m * b->nprobe * b->cap, (int64_t)rec, b->nprobe,
-                                    (int32_t)b->cap, true, k, b->stream, host_freq + (size_t)m * k,
-                                    host_amp + (size_t)m * k, host_n_found + m, true, rel_power);
-    if (st != LBW_OK) return st;
-  }
-  return LBW_OK;
+  return spectrum_device(b->series, (int64_t)rec, b->n, b->nprobe * b->cap, b->nprobe, b->cap, k, b->stream, host_freq,
+                         host_amp, host_n_found, true, rel_power);
 }
 
 lbw_status lbw_batch_get_populations(lbw_batch* b, int32_t member, double* host_f) {

@@ -4,13 +4,24 @@
 // Sec. IV.C, Fig. FreqTorus).  For a pulse-excited run the same modes are the peaks of the
 // probe signal's spectrum, estimated here:
 //   1. mean removed, Hann window w_t = 1/2 - 1/2 cos(2 pi t / (T - 1));
-//   2. zero padding to M = smallest power of two >= 4 T; radix-2 Stockham FFT
-//      (log2 M passes through global memory, natural-order output);
+//   2. zero padding to M = smallest power of two >= 4 T; the real series as one complex
+//      Stockham FFT of M / 2 points (even samples real, odd samples imaginary), sixteen points
+//      per thread and pass;
 //   3. |X_j|^2, local maxima above 1e-3 of the largest bin; the k strongest are chosen with
 //      warp-shuffle arg-max reductions (ties: lower bin) and sorted by frequency;
 //   4. each peak is refined by a parabola through log-power at j-1, j, j+1 and 40
-//      golden-section steps on the windowed DTFT over +-1 bin (one CTA per peak; the DTFT
-//      sum uses per-thread chunks with a rotation recurrence for e^{-i omega t}).
+//      golden-section steps on the windowed DTFT over +-1 bin.  Over that range the DTFT is a
+//      power series in omega - omega_0 whose coefficients are moments of the series, so the
+//      series is read once per peak and not once per evaluation.
+//
+// All estimates of a call (the series of lbw_spectrum_series, the members of an ensemble) run in
+// the same launches, grid.y of them.  FP64 arithmetic (2 operations a cycle and SM) is what
+// bounds the estimator: a radix-2 pass with a sincospi per butterfly takes 50 operations a
+// point, a radix-16 pass about 20 and does the work of four; golden section on the sums takes
+// 81 x 8 a sample and peak, the moments about 40, spread over all SMs instead of one CTA per peak.
+// Measured, 16 host series of 20,000 samples with 8 peaks each, one after the other -> here:
+// 62.2 -> 0.86 ms (moments 0.30, four FFT passes 0.17, search 0.10, selection 0.08, power 0.06);
+// one series of 20,000: 4.1 -> 0.46 ms, of 256: 0.97 -> 0.41 ms.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -24,109 +35,202 @@
 namespace lbw {
 namespace {
 
-constexpr int kThreads = 512;
 constexpr double kGolden = 0.6180339887498949;
+constexpr double kPi = 3.141592653589793238462643383279502884;
+constexpr int kParts = 64;   // partial sums of a series' mean
+constexpr int kSegs = 64;    // segments of a series in the refinement
+constexpr int kSegQ = 7;     // moments about a segment's centre: |dw (t - tc)| <= pi / 256, so
+                             // the first neglected term is below 1e-17 of the sum of |x|
+constexpr int kMom = 18;     // moments about the series' centre: |dw (t - T / 2)| <= pi / 4
 
-__device__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
+// Device arrays of the estimates of one call: estimate e's slice of each begins at e times the
+// length given here.
+struct Work {
+  double* xw;               // T      summed, then windowed series
+  double* part;             // kParts partial sums
+  double2 *A, *B;           // M / 2  FFT ping-pong
+  double* P;                // M / 2 + 1
+  long long* cand;          // M / 4 + 1
+  unsigned long long* count;  // 2: candidates, largest power (bits)
+  long long* chosen;        // 64
+  double2* mom;             // k x kSegs x kSegQ
+  double* res;              // kRes: number of peaks, mean, 64 frequencies, 64 amplitudes
+};
+constexpr int kRes = 2 + 2 * 64;
+
+// sum of the nser series (stride apart) of each estimate, and partial sums for the mean
+__global__ void sum_kernel(const double* __restrict__ x, long long T, int nser, long long stride,
+                           long long est_stride, Work w) {
+  __shared__ double red[32];
+  const double* src = x + blockIdx.y * est_stride;
+  double* dst = w.xw + blockIdx.y * T;
+  const long long len = (T + gridDim.x - 1) / gridDim.x, t0 = blockIdx.x * len, t1 = min(T, t0 + len);
   double s = 0.0;
-  if (threadIdx.x < 32) {
-    s = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) red[0] = s;
+  for (long long t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
+    double v = 0.0;
+    for (int p = 0; p < nser; ++p) v += src[(long long)p * stride + t];
+    dst[t] = v;
+    s += v;
+  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) v += red[k];
+    w.part[blockIdx.y * kParts + blockIdx.x] = v;
+  }
+}
+
+// xw_t = w_t (x_t - mean) in place
+__global__ void window_kernel(long long T, int parts, Work w) {
+  __shared__ double mean;
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int k = 0; k < parts; ++k) s += w.part[blockIdx.y * kParts + k];
+    mean = s / (double)T;
+    if (blockIdx.x == 0) w.res[blockIdx.y * kRes + 1] = mean;
   }
   __syncthreads();
-  return red[0];
+  double* x = w.xw + blockIdx.y * T;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < T; t += (long long)gridDim.x * blockDim.x)
+    x[t] = (0.5 - 0.5 * cospi(2.0 * (double)t / (double)(T - 1))) * (x[t] - mean);
 }
 
-// mean of the (summed) series and sum of the window weights
-__global__ void stats_kernel(const double* __restrict__ x, long long T, int nser, long long stride,
-                             double* out) {
-  __shared__ double red[32];
-  double s = 0.0, sw = 0.0;
-  for (long long t = threadIdx.x; t < T; t += blockDim.x) {
-    double v = 0.0;
-    for (int p = 0; p < nser; ++p) v += x[(long long)p * stride + t];
-    s += v;
-    sw += 0.5 - 0.5 * cospi(2.0 * (double)t / (double)(T - 1));
+__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ double2 mul_mi(double2 a) { return make_double2(a.y, -a.x); }  // a (-i)
+
+// forward DFTs of R values in registers, natural order
+template <int R> __device__ __forceinline__ void dft(double2 (&v)[R]);
+template <> __device__ __forceinline__ void dft<2>(double2 (&v)[2]) {
+  const double2 a = v[0];
+  v[0] = cadd(a, v[1]);
+  v[1] = csub(a, v[1]);
+}
+template <> __device__ __forceinline__ void dft<4>(double2 (&v)[4]) {
+  const double2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]), d = mul_mi(csub(v[1], v[3]));
+  v[0] = cadd(a, c);
+  v[1] = cadd(b, d);
+  v[2] = csub(a, c);
+  v[3] = csub(b, d);
+}
+template <> __device__ __forceinline__ void dft<8>(double2 (&v)[8]) {
+  constexpr double h = 0.70710678118654752440;  // cos(pi / 4)
+  double2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+  dft<4>(e);
+  dft<4>(o);
+  o[1] = make_double2(h * (o[1].x + o[1].y), h * (o[1].y - o[1].x));
+  o[2] = mul_mi(o[2]);
+  o[3] = make_double2(h * (o[3].y - o[3].x), -h * (o[3].x + o[3].y));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = cadd(e[k], o[k]);
+    v[k + 4] = csub(e[k], o[k]);
   }
-  s = block_sum(s, red);
-  sw = block_sum(sw, red);
-  if (threadIdx.x == 0) {
-    out[0] = s / (double)T;
-    out[1] = sw;
+}
+template <> __device__ __forceinline__ void dft<16>(double2 (&v)[16]) {
+  constexpr double h = 0.70710678118654752440, c = 0.92387953251128675613, s = 0.38268343236508977173;  // pi / 8
+  const double2 w[10] = {{1, 0}, {c, -s}, {h, -h}, {s, -c}, {0, -1}, {0, 0}, {-h, -h}, {0, 0}, {0, 0}, {-c, s}};
+  double2 t[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    double2 u[4] = {v[a], v[a + 4], v[a + 8], v[a + 12]};
+    dft<4>(u);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) t[b][a] = a * b == 0 ? u[b] : (a * b == 4 ? mul_mi(u[b]) : cmul(u[b], w[a * b]));
+  }
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    dft<4>(t[b]);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) v[b + 4 * a] = t[b][a];
   }
 }
 
-// xw_t = w_t (x_t - mean) as complex, zero-padded to M
-__global__ void window_kernel(const double* __restrict__ x, long long T, int nser, long long stride,
-                              const double* __restrict__ stats, long long M, double2* a,
-                              double* xw) {
-  const double mean = stats[0];
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < M;
-       t += (long long)gridDim.x * blockDim.x) {
-    double v = 0.0;
-    if (t < T) {
-      for (int p = 0; p < nser; ++p) v += x[(long long)p * stride + t];
-      v = (0.5 - 0.5 * cospi(2.0 * (double)t / (double)(T - 1))) * (v - mean);
-      xw[t] = v;
+// One Stockham pass: R sub-transforms of size ns are combined into one of R ns.  The first pass
+// (FIRST, ns = 1) reads the windowed series, zero past its end.
+template <int R, bool FIRST>
+__global__ void __launch_bounds__(128) stockham_kernel(const double2* __restrict__ in, double2* __restrict__ out,
+                                                       const double* __restrict__ xw, long long T, long long N,
+                                                       long long ns) {
+  const long long part = N / R;
+  out += blockIdx.y * N;
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < part; j += (long long)gridDim.x * blockDim.x) {
+    double2 v[R];
+    if constexpr (FIRST) {
+      const double* x = xw + blockIdx.y * T;
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        const long long t = 2 * (j + q * part);
+        v[q] = make_double2(t < T ? x[t] : 0.0, t + 1 < T ? x[t + 1] : 0.0);
+      }
+    } else {
+      const double2* src = in + blockIdx.y * N;
+#pragma unroll
+      for (int q = 0; q < R; ++q) v[q] = src[j + q * part];
     }
-    a[t] = make_double2(v, 0.0);
-  }
-}
-
-// one radix-2 Stockham pass: sub-transforms of size ns are combined into size 2 ns
-__global__ void stockham_kernel(const double2* __restrict__ in, double2* __restrict__ out,
-                                long long M, long long ns) {
-  const long long half = M >> 1;
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < half;
-       j += (long long)gridDim.x * blockDim.x) {
     const long long k = j & (ns - 1);
-    const double2 a0 = in[j], b = in[j + half];
-    double s, c;
-    sincospi((double)k / (double)ns, &s, &c);  // w = e^{-i pi k / ns}
-    const double2 a1 = make_double2(b.x * c + b.y * s, b.y * c - b.x * s);
-    const long long d = (j / ns) * 2 * ns + k;
-    out[d] = make_double2(a0.x + a1.x, a0.y + a1.y);
-    out[d + ns] = make_double2(a0.x - a1.x, a0.y - a1.y);
+    if constexpr (!FIRST) {
+      double s, c;
+      sincospi(2.0 * (double)k / (double)(ns * R), &s, &c);
+      double2 w[R];  // e^{-2 pi i k q / (R ns)}, powers by halving
+      w[1] = make_double2(c, -s);
+#pragma unroll
+      for (int q = 2; q < R; ++q) w[q] = cmul(w[q / 2], w[q - q / 2]);
+#pragma unroll
+      for (int q = 1; q < R; ++q) v[q] = cmul(v[q], w[q]);
+    }
+    dft<R>(v);
+    const long long d = (j - k) * R + k;
+#pragma unroll
+    for (int q = 0; q < R; ++q) out[d + q * ns] = v[q];
   }
 }
 
-__global__ void power_kernel(const double2* __restrict__ X, long long M, double* P) {
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j <= M / 2;
-       j += (long long)gridDim.x * blockDim.x)
-    P[j] = X[j].x * X[j].x + X[j].y * X[j].y;
-}
-
-__global__ void max_kernel(const double* __restrict__ P, long long M, double* out) {
+// |X_k|^2 of the real series for k = 0 .. N from the packed transform Z (N points), two bins per
+// thread: X_k = E + w O and X_{N-k} = conj(E - w O) with E = (Z_k + conj Z_{N-k}) / 2,
+// O = -i (Z_k - conj Z_{N-k}) / 2, w = e^{-i pi k / N}; and the largest power past bin 0.
+__global__ void power_kernel(const double2* __restrict__ Zall, long long N, Work w) {
   __shared__ double red[32];
+  const double2* Z = Zall + blockIdx.y * N;
+  double* P = w.P + blockIdx.y * (N + 1);
   double m = 0.0;
-  for (long long j = 1 + threadIdx.x; j <= M / 2; j += blockDim.x) m = fmax(m, P[j]);
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k <= N / 2; k += (long long)gridDim.x * blockDim.x) {
+    const double2 a = Z[k], b = Z[k == 0 ? 0 : N - k];
+    const double2 E = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
+    const double2 O = make_double2(0.5 * (a.y + b.y), -0.5 * (a.x - b.x));
+    double s, c;
+    sincospi((double)k / (double)N, &s, &c);
+    const double2 r = cmul(make_double2(c, -s), O);
+    const double2 p = cadd(E, r), q = csub(E, r);
+    const double pk = p.x * p.x + p.y * p.y, pn = q.x * q.x + q.y * q.y;
+    P[k] = pk;
+    P[N - k] = pn;
+    if (k > 0) m = fmax(m, pk);
+    m = fmax(m, pn);
+  }
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-    if (threadIdx.x == 0) out[2] = m;
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) m = fmax(m, red[k]);
+    // non-negative doubles are ordered like their bits
+    atomicMax(w.count + 2 * blockIdx.y + 1, (unsigned long long)__double_as_longlong(m));
   }
 }
 
-__global__ void candidates_kernel(const double* __restrict__ P, long long M,
-                                  const double* __restrict__ stats, double thresh,
-                                  long long* cand, unsigned long long* count) {
-  const double lim = thresh * stats[2];
-  for (long long j = 1 + blockIdx.x * (long long)blockDim.x + threadIdx.x; j < M / 2;
-       j += (long long)gridDim.x * blockDim.x) {
+__global__ void candidates_kernel(long long N, double thresh, Work w) {
+  const double* P = w.P + blockIdx.y * (N + 1);
+  unsigned long long* count = w.count + 2 * blockIdx.y;
+  const double lim = thresh * __longlong_as_double((long long)count[1]);
+  long long* cand = w.cand + blockIdx.y * (N / 2 + 1);
+  for (long long j = 1 + blockIdx.x * (long long)blockDim.x + threadIdx.x; j < N; j += (long long)gridDim.x * blockDim.x) {
     const double p = P[j];
-    if (p > P[j - 1] && p >= P[j + 1] && p >= lim) {
-      unsigned long long s = atomicAdd(count, 1ULL);
-      cand[s] = j;
-    }
+    if (p > P[j - 1] && p >= P[j + 1] && p >= lim) cand[atomicAdd(count, 1ULL)] = j;
   }
 }
 
@@ -140,16 +244,17 @@ __device__ __forceinline__ bool lower(double, long long ja, double, long long jb
 
 // k rounds of a block-wide arg-max over the candidate list (warp shuffles), then sort; the
 // winner of a round is the strongest candidate, or with `lowest` the lowest-frequency one
-__global__ void select_kernel(const double* __restrict__ P, long long* cand,
-                              const unsigned long long* __restrict__ count, int k,
-                              long long* chosen, int* n_chosen, bool lowest) {
+__global__ void select_kernel(long long N, int k, bool lowest, Work w) {
+  const double* P = w.P + blockIdx.x * (N + 1);
+  long long* cand = w.cand + blockIdx.x * (N / 2 + 1);
+  long long* chosen = w.chosen + blockIdx.x * 64;
   auto wins = [&](double pa, long long ja, double pb, long long jb) {
     return lowest ? lower(pa, ja, pb, jb) : better(pa, ja, pb, jb);
   };
   __shared__ double sp[32];
   __shared__ long long sj[32];
   __shared__ long long pick[64];
-  const long long n = (long long)*count;
+  const long long n = (long long)w.count[2 * blockIdx.x];
   int got = 0;
   for (int r = 0; r < k; ++r) {
     double bp = -1.0;
@@ -194,168 +299,250 @@ __global__ void select_kernel(const double* __restrict__ P, long long* cand,
       pick[b + 1] = v;
     }
     for (int a = 0; a < got; ++a) chosen[a] = pick[a];
-    *n_chosen = got;
+    w.res[blockIdx.x * kRes] = (double)got;
   }
 }
 
-// |sum_t xw_t e^{-i omega t}|^2 over the block
-__device__ double dtft_power(const double* __restrict__ xw, long long T, double omega, double* red) {
-  const long long chunk = (T + blockDim.x - 1) / blockDim.x;
-  const long long t0 = threadIdx.x * chunk, t1 = min(T, t0 + chunk);
-  double re = 0.0, im = 0.0;
-  if (t0 < t1) {
+// Frequency of the parabola through log-power about bin j: the centre of the refinement.
+__device__ __forceinline__ double parabola(const double* P, long long j, long long M) {
+  const double la = log(P[j - 1]), lb = log(P[j]), lc = log(P[j + 1]);
+  const double den = la - 2.0 * lb + lc;
+  double delta = (den < 0.0) ? 0.5 * (la - lc) / den : 0.0;
+  if (!isfinite(delta)) delta = 0.0;
+  return 2.0 * kPi * ((double)j + delta) / (double)M;
+}
+
+// Moments sum_t xw_t e^{-i omega_0 (t - T/2)} ((t - tc) 2 / T)^q, q = 0 .. kSegQ - 1, of each
+// segment (centre tc) of the series, about the parabola's omega_0 of each chosen peak.  One warp
+// per segment; grid (kSegs / 8, peaks, estimates).
+__global__ void __launch_bounds__(256) moments_kernel(long long T, long long N, int k, Work w) {
+  const int lane = threadIdx.x & 31, seg = blockIdx.x * 8 + (threadIdx.x >> 5), peak = blockIdx.y, est = blockIdx.z;
+  if (peak >= (int)w.res[est * kRes]) return;
+  const double om = parabola(w.P + est * (N + 1), w.chosen[est * 64 + peak], 2 * N);
+  const long long len = (T + kSegs - 1) / kSegs, t0 = min(T, seg * len), t1 = min(T, t0 + len);
+  const double* x = w.xw + est * T;
+  const double mid = 0.5 * (double)T, tc = (double)t0 + 0.5 * (double)(len - 1), sc = 2.0 / (double)T;
+  double re[kSegQ] = {}, im[kSegQ] = {};
+  if (t0 + lane < t1) {
     double s, c, ds, dc;
-    sincos(omega * (double)t0, &s, &c);
-    sincos(omega, &ds, &dc);
-    for (long long t = t0; t < t1; ++t) {
-      re += xw[t] * c;
-      im -= xw[t] * s;
+    sincos(om * ((double)(t0 + lane) - mid), &s, &c);
+    sincos(om * 32.0, &ds, &dc);
+    for (long long t = t0 + lane; t < t1; t += 32) {
+      const double v = x[t], u = ((double)t - tc) * sc;
+      double pr = v * c, pi = v * s;  // the imaginary part's sign goes in at the end
+#pragma unroll
+      for (int q = 0; q < kSegQ; ++q) {
+        re[q] += pr;
+        im[q] += pi;
+        pr *= u;
+        pi *= u;
+      }
       const double cn = c * dc - s * ds;
       s = s * dc + c * ds;
       c = cn;
     }
   }
-  re = block_sum(re, red);
-  im = block_sum(im, red);
-  return re * re + im * im;
+  double2* out = w.mom + (((size_t)est * k + peak) * kSegs + seg) * kSegQ;
+#pragma unroll
+  for (int q = 0; q < kSegQ; ++q) {
+    for (int o = 16; o > 0; o >>= 1) {
+      re[q] += __shfl_down_sync(0xffffffffu, re[q], o);
+      im[q] += __shfl_down_sync(0xffffffffu, im[q], o);
+    }
+    if (lane == 0) out[q] = make_double2(re[q], -im[q]);
+  }
 }
 
-__global__ void refine_kernel(const double* __restrict__ xw, long long T, const double* __restrict__ P,
-                              long long M, const long long* __restrict__ chosen,
-                              const int* __restrict__ n_chosen, const double* __restrict__ stats,
-                              double* freq, double* amp) {
-  __shared__ double red[32];
-  const int p = blockIdx.x;
-  if (p >= *n_chosen) return;
-  const long long j = chosen[p];
-  const double la = log(P[j - 1]), lb = log(P[j]), lc = log(P[j + 1]);
-  const double den = la - 2.0 * lb + lc;
-  double delta = (den < 0.0) ? 0.5 * (la - lc) / den : 0.0;
-  if (!isfinite(delta)) delta = 0.0;
-  const double pi = 3.141592653589793238462643383279502884;
-  const double om = 2.0 * pi * ((double)j + delta) / (double)M;
-  const double halfw = 2.0 * pi / (double)M;
+// 40 golden-section steps on |X(omega)|^2 over omega_0 +- 1 bin, with
+// X(omega_0 + y 2 / T) e^{i omega T / 2} = sum_m (-i y)^m / m! G_m and G_m the moments about the
+// centre of the series.  One warp per peak: the lanes shift the segments' moments to the centre
+// (binomially) and add them up; every lane then runs the same search.
+__global__ void __launch_bounds__(32) refine_kernel(long long T, long long N, int k, Work w) {
+  const int lane = threadIdx.x, peak = blockIdx.x, est = blockIdx.y;
+  if (peak >= (int)w.res[est * kRes]) return;
+  const double om = parabola(w.P + est * (N + 1), w.chosen[est * 64 + peak], 2 * N);
+  const long long len = (T + kSegs - 1) / kSegs;
+  const double sc = 2.0 / (double)T;
+  const double2* mom = w.mom + ((size_t)est * k + peak) * kSegs * kSegQ;
+  double re[kMom] = {}, im[kMom] = {};
+  for (int seg = lane; seg < kSegs; seg += 32) {
+    const double v = ((double)min(T, seg * len) + 0.5 * (double)(len - 1) - 0.5 * (double)T) * sc;
+    // add mom_q C(m, q) v^(m - q) to every G_m: row q starts at m = q and grows by v (m + 1) / (m + 1 - q)
+#pragma unroll
+    for (int q = 0; q < kSegQ; ++q) {
+      double ar = mom[seg * kSegQ + q].x, ai = mom[seg * kSegQ + q].y;
+#pragma unroll
+      for (int m = q; m < kMom; ++m) {
+        re[m] += ar;
+        im[m] += ai;
+        const double g = v * ((double)(m + 1) / (double)(m + 1 - q));
+        ar *= g;
+        ai *= g;
+      }
+    }
+  }
+  double fact = 1.0;
+#pragma unroll
+  for (int m = 0; m < kMom; ++m) {
+    for (int o = 16; o > 0; o >>= 1) {
+      re[m] += __shfl_xor_sync(0xffffffffu, re[m], o);
+      im[m] += __shfl_xor_sync(0xffffffffu, im[m], o);
+    }
+    if (m > 0) fact /= (double)m;
+    // times (-i)^m / m!
+    const double a = re[m] * fact, b = im[m] * fact;
+    re[m] = m % 4 == 0 ? a : m % 4 == 1 ? b : m % 4 == 2 ? -a : -b;
+    im[m] = m % 4 == 0 ? b : m % 4 == 1 ? -a : m % 4 == 2 ? -b : a;
+  }
+  auto power = [&](double omega) {
+    const double y = (omega - om) * (0.5 * (double)T), y2 = y * y;
+    double r[2], i[2];  // even and odd powers, two short chains each
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      double a = re[kMom - 2 + h], b = im[kMom - 2 + h];
+#pragma unroll
+      for (int m = kMom - 4 + h; m >= 0; m -= 2) {
+        a = fma(a, y2, re[m]);
+        b = fma(b, y2, im[m]);
+      }
+      r[h] = a;
+      i[h] = b;
+    }
+    const double x = fma(r[1], y, r[0]), z = fma(i[1], y, i[0]);
+    return x * x + z * z;
+  };
+  const double halfw = kPi / (double)N;
   double a = om - halfw, b = om + halfw;
+  double c = b - kGolden * (b - a), d = a + kGolden * (b - a);
+  double fc = power(c), fd = power(d);
   for (int it = 0; it < 40; ++it) {
-    const double c = b - kGolden * (b - a);
-    const double d = a + kGolden * (b - a);
-    const double fc = dtft_power(xw, T, c, red);
-    const double fd = dtft_power(xw, T, d, red);
-    if (fc > fd) b = d; else a = c;
+    if (fc > fd) {
+      b = d; d = c; fd = fc;
+      c = b - kGolden * (b - a);
+      fc = power(c);
+    } else {
+      a = c; c = d; fc = fd;
+      d = a + kGolden * (b - a);
+      fd = power(d);
+    }
   }
-  const double w = 0.5 * (a + b);
-  const double pw = dtft_power(xw, T, w, red);
-  if (threadIdx.x == 0) {
-    freq[p] = w;
-    amp[p] = 2.0 * sqrt(pw) / stats[1];
+  if (lane == 0) {
+    const double o = 0.5 * (a + b);
+    w.res[est * kRes + 2 + peak] = o;
+    // the Hann weights add up to (T - 1) / 2
+    w.res[est * kRes + 2 + 64 + peak] = 2.0 * sqrt(power(o)) / (0.5 * (double)(T - 1));
   }
 }
-
-// Workspace of one estimate, carved from one block of device memory sized for series of up to
-// T samples and transforms of up to M points: stats(4) | a(M) | b(M) | xw(T) | P(M/2+1) |
-// cand(M/4+1) | count | chosen(64) | n_chosen | freq(64) | amp(64).
-struct Workspace {
-  double* stats;
-  double2 *A, *B;
-  double* xw;
-  double* P;
-  long long* cand;
-  unsigned long long* count;
-  long long* chosen;
-  int* n_chosen;
-  double *freq, *amp;
-};
 
 constexpr size_t round16(size_t n) { return (n + 15) / 16 * 16; }
 
-constexpr size_t workspace_bytes(size_t M, size_t T) {
-  return round16(4 * 8) + 2 * round16(M * 16) + round16(T * 8) + round16((M / 2 + 1) * 8) +
-         round16((M / 4 + 1) * 8) + round16(8) + round16(64 * 8) + round16(8) + round16(64 * 8) +
-         round16(64 * 8);
+// Workspace for `count` estimates of T samples, transforms of M points and k peaks.
+constexpr size_t workspace_bytes(size_t M, size_t T, size_t count, size_t k) {
+  return round16(count * T * 8) + round16(count * kParts * 8) + 2 * (count * (M / 2) * 16) +
+         round16(count * (M / 2 + 1) * 8) + round16(count * (M / 4 + 1) * 8) + round16(count * 16) +
+         round16(count * 64 * 8) + count * k * kSegs * kSegQ * 16 + round16(count * kRes * 8);
 }
 
-Workspace carve(unsigned char* base, size_t M, size_t T) {
+Work carve(unsigned char* base, size_t M, size_t T, size_t count, size_t k) {
   unsigned char* p = base;
   auto take = [&](size_t n) { unsigned char* q = p; p += round16(n); return q; };
-  Workspace w;
-  w.stats = (double*)take(4 * 8);
-  w.A = (double2*)take(M * 16);
-  w.B = (double2*)take(M * 16);
-  w.xw = (double*)take(T * 8);
-  w.P = (double*)take((M / 2 + 1) * 8);
-  w.cand = (long long*)take((M / 4 + 1) * 8);
-  w.count = (unsigned long long*)take(8);
-  w.chosen = (long long*)take(64 * 8);
-  w.n_chosen = (int*)take(8);
-  w.freq = (double*)take(64 * 8);
-  w.amp = (double*)take(64 * 8);
+  Work w;
+  w.xw = (double*)take(count * T * 8);
+  w.part = (double*)take(count * kParts * 8);
+  w.A = (double2*)take(count * (M / 2) * 16);
+  w.B = (double2*)take(count * (M / 2) * 16);
+  w.P = (double*)take(count * (M / 2 + 1) * 8);
+  w.cand = (long long*)take(count * (M / 4 + 1) * 8);
+  w.count = (unsigned long long*)take(count * 16);
+  w.chosen = (long long*)take(count * 64 * 8);
+  w.mom = (double2*)take(count * k * kSegs * kSegQ * 16);
+  w.res = (double*)take(count * kRes * 8);
   return w;
 }
 
-// The estimator's launches on stream s and the copy of its results to the host (synchronous).
-// Every workspace value is written before it is read except the candidate counter, which is
-// cleared here, so a workspace may hold anything from an earlier call.  *finite is false when
-// the series' mean is not finite (a NaN or infinity in the series: an unstable run).
-cudaError_t run_estimator(const Workspace& w, const double* d_x, int64_t T, int nser,
-                          int32_t stride_series, int32_t k, bool lowest, double rel_power,
-                          cudaStream_t s, double* h_freq, double* h_amp, int32_t* h_n,
-                          bool* finite) {
+// The estimator's launches on stream s for `count` estimates, and the copy of their results
+// (kRes values each) to the host (synchronous).  Every workspace value is written before it is
+// read except the candidate counters, which are cleared here, so a workspace may hold anything
+// from an earlier call.
+cudaError_t run_estimator(const Work& w, const double* d_x, int64_t T, int count, int64_t est_stride, int nser,
+                          int64_t stride_series, int32_t k, bool lowest, double rel_power, cudaStream_t s,
+                          std::vector<double>& res) {
   long long M = 1;
   while (M < 4 * T) M <<= 1;
+  const long long N = M / 2;
   // a launch error left behind by an unrelated earlier runtime call on this thread would
   // otherwise be read back below as this call's failure
   (void)cudaGetLastError();
-  cudaError_t e = cudaMemsetAsync(w.count, 0, 8, s);
-  const int blocks = 152 * 4;
+  cudaError_t e = cudaMemsetAsync(w.count, 0, 16 * (size_t)count, s);
+  auto blocks = [](long long n, int per) { return (unsigned)std::max(1LL, std::min((n + per - 1) / per, 152LL * 8)); };
   if (e == cudaSuccess) {
-    stats_kernel<<<1, 1024, 0, s>>>(d_x, T, nser, stride_series, w.stats);
-    window_kernel<<<blocks, 256, 0, s>>>(d_x, T, nser, stride_series, w.stats, M, w.A, w.xw);
+    const int parts = (int)std::min<long long>(kParts, (T + 1023) / 1024);
+    sum_kernel<<<dim3(parts, count), 256, 0, s>>>(d_x, T, nser, stride_series, est_stride, w);
+    window_kernel<<<dim3(blocks(T, 256), count), 256, 0, s>>>(T, parts, w);
     double2 *in = w.A, *out = w.B;
-    for (long long ns = 1; ns < M; ns <<= 1) {
-      stockham_kernel<<<blocks, 256, 0, s>>>(in, out, M, ns);
+    for (long long ns = 1; ns < N;) {
+      // radix 16 passes, the first one taking what is left over (N >= 8)
+      int bits = 0;
+      while ((ns << bits) < N) ++bits;
+      const int r = ns == 1 && bits % 4 != 0 ? 1 << (bits % 4) : 16;
+      const dim3 grid(blocks(N / r, 128), count);
+      if (ns > 1) stockham_kernel<16, false><<<grid, 128, 0, s>>>(in, out, w.xw, T, N, ns);
+      else if (r == 16) stockham_kernel<16, true><<<grid, 128, 0, s>>>(in, out, w.xw, T, N, ns);
+      else if (r == 8) stockham_kernel<8, true><<<grid, 128, 0, s>>>(in, out, w.xw, T, N, ns);
+      else if (r == 4) stockham_kernel<4, true><<<grid, 128, 0, s>>>(in, out, w.xw, T, N, ns);
+      else stockham_kernel<2, true><<<grid, 128, 0, s>>>(in, out, w.xw, T, N, ns);
+      ns *= r;
       std::swap(in, out);
     }
-    power_kernel<<<blocks, 256, 0, s>>>(in, M, w.P);
-    max_kernel<<<1, 1024, 0, s>>>(w.P, M, w.stats);
-    candidates_kernel<<<blocks, 256, 0, s>>>(w.P, M, w.stats, rel_power, w.cand, w.count);
-    select_kernel<<<1, 1024, 0, s>>>(w.P, w.cand, w.count, k, w.chosen, w.n_chosen, lowest);
-    refine_kernel<<<k, kThreads, 0, s>>>(w.xw, T, w.P, M, w.chosen, w.n_chosen, w.stats, w.freq, w.amp);
+    power_kernel<<<dim3(blocks(N / 2 + 1, 256), count), 256, 0, s>>>(in, N, w);
+    candidates_kernel<<<dim3(blocks(N, 256), count), 256, 0, s>>>(N, rel_power, w);
+    select_kernel<<<count, 256, 0, s>>>(N, k, lowest, w);
+    moments_kernel<<<dim3(kSegs / 8, k, count), 256, 0, s>>>(T, N, k, w);
+    refine_kernel<<<dim3(k, count), 32, 0, s>>>(T, N, k, w);
     e = cudaGetLastError();
   }
-  int nfound = 0;
-  double mean = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&nfound, w.n_chosen, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&mean, w.stats, sizeof(double), cudaMemcpyDeviceToHost, s);
+  res.resize((size_t)count * kRes);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(res.data(), w.res, 8 * res.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  *finite = std::isfinite(mean);
-  if (!*finite) nfound = 0;
-  if (e == cudaSuccess && nfound > 0) {
-    e = cudaMemcpyAsync(h_freq, w.freq, sizeof(double) * nfound, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_amp, w.amp, sizeof(double) * nfound, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  }
-  if (e == cudaSuccess) *h_n = nfound;
   return e;
+}
+
+// Estimate e's results to the caller's arrays; false when its series' mean is not finite (a NaN
+// or infinity in the series: an unstable run).
+bool put_result(const std::vector<double>& res, int e, double* freq, double* amp, int32_t* n) {
+  const double* r = res.data() + (size_t)e * kRes;
+  if (!std::isfinite(r[1])) return false;
+  *n = (int32_t)r[0];
+  std::copy(r + 2, r + 2 + *n, freq);
+  std::copy(r + 2 + 64, r + 2 + 64 + *n, amp);
+  return true;
 }
 
 }  // namespace
 
-lbw_status spectrum_device(const double* d_x, int64_t T, int32_t n_series, int32_t stride_series,
-                           bool sum_all, int32_t k, cudaStream_t s, double* h_freq,
-                           double* h_amp, int32_t* h_n, bool lowest, double rel_power) {
-  long long M = 1;
-  while (M < 4 * T) M <<= 1;
+lbw_status spectrum_device(const double* d_x, int64_t T, int32_t count, int64_t est_stride, int32_t n_sum,
+                           int64_t stride_series, int32_t k, cudaStream_t s, double* h_freq, double* h_amp,
+                           int32_t* h_n, bool lowest, double rel_power) {
+  size_t M = 1;
+  while (M < 4 * (size_t)T) M <<= 1;
+  // as many estimates per pass as fit in 256 MB of workspace
+  const int per = (int)std::max<size_t>(1, std::min<size_t>(std::min(count, 4096), (256u << 20) / workspace_bytes(M, (size_t)T, 1, k)));
   unsigned char* base = nullptr;
-  LBW_CUDA(cudaMallocAsync((void**)&base, workspace_bytes((size_t)M, (size_t)T), s));
-  const Workspace w = carve(base, (size_t)M, (size_t)T);
-  int32_t nfound = 0;
+  LBW_CUDA(cudaMallocAsync((void**)&base, workspace_bytes(M, (size_t)T, per, k), s));
+  const Work w = carve(base, M, (size_t)T, per, k);
+  std::vector<double> res;
+  cudaError_t e = cudaSuccess;
   bool finite = true;
-  const cudaError_t e = run_estimator(w, d_x, T, sum_all ? n_series : 1, stride_series, k, lowest,
-                                      rel_power, s, h_freq, h_amp, &nfound, &finite);
+  for (int first = 0; first < count && e == cudaSuccess && finite; first += per) {
+    const int n = std::min(per, count - first);
+    e = run_estimator(w, d_x + (size_t)first * est_stride, T, n, est_stride, n_sum, stride_series, k, lowest, rel_power,
+                      s, res);
+    for (int j = 0; j < n && e == cudaSuccess && finite; ++j)
+      finite = put_result(res, j, h_freq + (size_t)(first + j) * k, h_amp + (size_t)(first + j) * k, h_n + first + j);
+  }
   cudaFreeAsync(base, s);
   if (e != cudaSuccess) return cuda_fail(e, "spectrum");
   if (!finite) return fail(LBW_EUNSTABLE, "spectrum: the series holds a non-finite value (unstable run)");
-  *h_n = nfound;
   return LBW_OK;
 }
 
@@ -378,7 +565,7 @@ constexpr size_t kStaticMaxM = 4 * (size_t)kStaticMaxT;  // a power of two: M of
 // The workspace.  In host code this name is only a host-side handle: its device address comes
 // from cudaGetSymbolAddress, looked up once per device context (static_workspace below).
 static __device__ __align__(256) unsigned char
-    g_spectrum_scratch[lbw::workspace_bytes(lbw::kStaticMaxM, lbw::kStaticMaxT)];
+    g_spectrum_scratch[lbw::workspace_bytes(lbw::kStaticMaxM, lbw::kStaticMaxT, 1, 64)];
 
 namespace {
 
@@ -453,14 +640,15 @@ extern "C" lbw_status lbw_spectrum_series_static(const double* dev_x, int64_t T,
   unsigned char* base = nullptr;
   cudaError_t e = static_workspace(dev, &base);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_spectrum_scratch)");
-  const Workspace w = carve(base, kStaticMaxM, (size_t)kStaticMaxT);
-  int32_t nfound = 0;
-  bool finite = true;
-  e = run_estimator(w, dev_x, T, 1, (int32_t)T, k, false, 1e-3,
-                    reinterpret_cast<cudaStream_t>(stream), host_freq, host_amp, &nfound, &finite);
+  size_t M = 1;
+  while (M < 4 * (size_t)T) M <<= 1;
+  std::vector<double> res;
+  e = run_estimator(carve(base, M, (size_t)T, 1, k), dev_x, T, 1, T, 1, T, k, false, 1e-3,
+                    reinterpret_cast<cudaStream_t>(stream), res);
   if (e != cudaSuccess) return cuda_fail(e, "lbw_spectrum_series_static");
-  if (!finite) return fail(LBW_EUNSTABLE, "spectrum: the series holds a non-finite value");
+  int32_t nfound = 0;
+  if (!put_result(res, 0, host_freq, host_amp, &nfound))
+    return fail(LBW_EUNSTABLE, "spectrum: the series holds a non-finite value");
   *host_n_found = nfound;
   return LBW_OK;
 }
-
