@@ -344,7 +344,9 @@ lbw_status lbw_mlp_grad(lbw_mlp* q, const float* host_x, const float* host_t, in
 lbw_status lbw_mlp_adam_step(lbw_mlp* q, const float* host_grad, float lr);
 /* n_steps Adam steps on minibatches of `batch` rows of the n samples: step s uses rows
  * host_order[s * batch .. s * batch + batch - 1] (the caller draws the order).  host_loss
- * (may be NULL) receives the minibatch loss before each step. */
+ * (may be NULL) receives the minibatch loss before each step.  Hidden widths that are multiples of
+ * 4 up to 512 with at most 64 inputs, 16 outputs and 512 rows train in one cooperative launch per
+ * 1024 steps, whose bounded waits return LBW_ETIMEOUT when one runs out. */
 lbw_status lbw_mlp_train(lbw_mlp* q, const float* host_x, const float* host_t, int32_t n,
                          const int32_t* host_order, int32_t n_steps, int32_t batch, float lr, float* host_loss);
 void lbw_mlp_destroy(lbw_mlp* q);
