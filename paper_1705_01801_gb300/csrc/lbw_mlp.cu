@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "lbw_internal.h"
+#include "lbw_mlp_forward.cuh"
 
 namespace lbw {
 namespace {
@@ -554,9 +555,19 @@ struct lbw_mlp {
   float *p2 = nullptr, *xch = nullptr;
   size_t xch_size = 0;
   unsigned* sync = nullptr;
+  // inference in one launch: transposed weights in FP32 / BF16 (valid since the last change of the
+  // parameters) and the rows' inputs and outputs
+  float* wt = nullptr;
+  __nv_bfloat16* wtb = nullptr;
+  bool wt_valid = false, wtb_valid = false;
+  float* io = nullptr;
+  size_t io_size = 0;
 };
 
 namespace {
+
+// the rounded and transposed copies of the weights are stale
+void params_changed(lbw_mlp* q) { q->pb_valid = q->wt_valid = q->wtb_valid = false; }
 
 void free_work(lbw_mlp* q) {
   for (float* a : q->act)
@@ -622,6 +633,64 @@ void backward(lbw_mlp* q, int rows) {
       std::swap(q->delta, q->delta2);
     }
   }
+}
+
+template <typename WB, int RB>
+cudaError_t launch_forward(lbw_mlp* q, const FwdArgs& a, const WB* wt) {
+  const size_t smem = fwd_smem<RB>(a.dims, a.depth);
+  const cudaError_t e =
+      cudaFuncSetAttribute(forward_kernel<WB, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  forward_kernel<WB, RB><<<(a.n + RB - 1) / RB, kFwdThreads, smem, q->stream>>>(a, wt);
+  return cudaGetLastError();
+}
+
+bool fits_forward(const lbw_mlp* q) {
+  for (int w : q->dims)
+    if (w > kFwdMaxWidth) return false;
+  return q->depth <= kFwdMaxDepth;
+}
+
+// n rows through the network in one launch, host to host; WB the weights' storage.
+template <typename WB>
+lbw_status forward_fused(lbw_mlp* q, const float* host_x, int n, float* host_y, WB*& wt, bool& valid) {
+  FwdArgs a{};
+  a.depth = q->depth;
+  a.n = n;
+  a.bias = q->p;
+  size_t at = 0;
+  for (int l = 0; l <= q->depth; ++l) a.dims[l] = q->dims[l];
+  for (int l = 0; l < q->depth; ++l) {
+    a.woff[l] = (unsigned)at;
+    a.boff[l] = (unsigned)q->boff[l];
+    at += (size_t)a.dims[l] * fwd_pad(a.dims[l + 1]);
+  }
+  if (!wt) LBW_CUDA(cudaMallocAsync((void**)&wt, sizeof(WB) * at, q->stream));
+  const size_t nx = (size_t)n * q->in, ny = (size_t)n * q->out;
+  if (nx + ny > q->io_size) {
+    if (q->io) cudaFreeAsync(q->io, q->stream);
+    q->io = nullptr;
+    q->io_size = 0;
+    LBW_CUDA(cudaMallocAsync((void**)&q->io, sizeof(float) * (nx + ny), q->stream));
+    q->io_size = nx + ny;
+  }
+  a.x = q->io;
+  a.y = q->io + nx;
+  LBW_CUDA(cudaMemcpyAsync(q->io, host_x, sizeof(float) * nx, cudaMemcpyHostToDevice, q->stream));
+  if (!valid) {
+    for (int l = 0; l < q->depth; ++l)
+      pack_kernel<WB><<<dim3((a.dims[l] + 31) / 32, fwd_pad(a.dims[l + 1]) / 32), dim3(32, 8), 0, q->stream>>>(
+          q->p + q->woff[l], a.dims[l], a.dims[l + 1], wt + a.woff[l]);
+    valid = true;
+  }
+  // rows per CTA: more rows share a read of the weights, fewer fill the SMs
+  const cudaError_t e = n <= 4 * 152 ? launch_forward<WB, 4>(q, a, wt)
+                        : n <= 8 * 2 * 152 ? launch_forward<WB, 8>(q, a, wt)
+                        : n <= 16 * 4 * 152 ? launch_forward<WB, 16>(q, a, wt) : launch_forward<WB, 32>(q, a, wt);
+  if (e != cudaSuccess) return cuda_fail(e, "mlp forward");
+  LBW_CUDA(cudaMemcpyAsync(host_y, a.y, sizeof(float) * ny, cudaMemcpyDeviceToHost, q->stream));
+  LBW_CUDA(cudaStreamSynchronize(q->stream));
+  return LBW_OK;
 }
 
 // Launch shape of train_kernel.
@@ -811,7 +880,8 @@ void lbw_mlp_destroy(lbw_mlp* q) {
   if (!q) return;
   free_work(q);
   if (q->sync) cudaFreeAsync(q->sync, q->stream);
-  float* bufs[] = {q->p, q->g, q->m1, q->m2, q->data_x, q->data_t, q->p2, q->xch};
+  if (q->wtb) cudaFreeAsync(q->wtb, q->stream);
+  float* bufs[] = {q->p, q->g, q->m1, q->m2, q->data_x, q->data_t, q->p2, q->xch, q->wt, q->io};
   for (float* b : bufs)
     if (b) cudaFreeAsync(b, q->stream);
   if (q->pb) cudaFreeAsync(q->pb, q->stream);
@@ -840,12 +910,13 @@ lbw_status lbw_mlp_set_params(lbw_mlp* q, const float* host_params) {
   LBW_CUDA(cudaMemsetAsync(q->m2, 0, sizeof(float) * q->nparam, q->stream));
   LBW_CUDA(cudaStreamSynchronize(q->stream));
   q->adam_t = 0;
-  q->pb_valid = false;
+  params_changed(q);
   return LBW_OK;
 }
 
 lbw_status lbw_mlp_forward(lbw_mlp* q, const float* host_x, int32_t n, float* host_y) {
   if (!q || !host_x || !host_y || n < 1) return fail(LBW_EINVAL, "bad argument");
+  if (fits_forward(q)) return forward_fused<float>(q, host_x, n, host_y, q->wt, q->wt_valid);
   lbw_status st = ensure_work(q, n);
   if (st != LBW_OK) return st;
   LBW_CUDA(cudaMemcpyAsync(q->act[0], host_x, sizeof(float) * n * q->in, cudaMemcpyHostToDevice, q->stream));
@@ -858,6 +929,7 @@ lbw_status lbw_mlp_forward(lbw_mlp* q, const float* host_x, int32_t n, float* ho
 
 lbw_status lbw_mlp_predict_bf16(lbw_mlp* q, const float* host_x, int32_t n, float* host_y) {
   if (!q || !host_x || !host_y || n < 1) return fail(LBW_EINVAL, "bad argument");
+  if (fits_forward(q)) return forward_fused<__nv_bfloat16>(q, host_x, n, host_y, q->wtb, q->wtb_valid);
   lbw_status st = ensure_work(q, n);
   if (st != LBW_OK) return st;
   if (!q->pb_valid) {
@@ -899,7 +971,7 @@ lbw_status lbw_mlp_adam_step(lbw_mlp* q, const float* host_grad, float lr) {
                                                (float)(1.0 - std::pow(0.999, (double)q->adam_t)));
   LBW_CUDA(cudaGetLastError());
   LBW_CUDA(cudaStreamSynchronize(q->stream));
-  q->pb_valid = false;
+  params_changed(q);
   return LBW_OK;
 }
 
@@ -947,7 +1019,7 @@ lbw_status lbw_mlp_train(lbw_mlp* q, const float* host_x, const float* host_t, i
     cudaFreeAsync(d_order, q->stream);
     cudaFreeAsync(d_curve, q->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(q->stream);
-    q->pb_valid = false;
+    params_changed(q);
     if (st != LBW_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "mlp train");
     if (err) return fail(LBW_ETIMEOUT, "a training step's bounded wait ran out; the parameters are undefined until "
@@ -973,7 +1045,7 @@ lbw_status lbw_mlp_train(lbw_mlp* q, const float* host_x, const float* host_t, i
   cudaFreeAsync(d_curve, q->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(q->stream);
   if (e != cudaSuccess) return cuda_fail(e, "mlp train");
-  q->pb_valid = false;
+  params_changed(q);
   return LBW_OK;
 }
 
