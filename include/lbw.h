@@ -243,8 +243,8 @@ typedef struct lbw_batch lbw_batch; /* opaque, library-owned */
 
 /* n members (1..65536), all with the same prec; each descriptor is validated as in
  * lbw_create_grid.  Populations start at zero.  The initial launch shape is full-row tiles
- * with 16-plane segments where every member fits one (see lbw_batch_tune), else 7-row tiles
- * of 64 columns, else the register-pipelined kernel's default. */
+ * where every member fits one (see lbw_batch_tune), else 7-row tiles of 64 columns, with the
+ * segment length that fills the SMs most evenly, else the register-pipelined kernel's default. */
 lbw_status lbw_batch_create(const lbw_grid_desc* descs, int32_t n, void* stream, lbw_batch** out);
 
 /* Initial state at rest for every member: host_counts[m] pulses for member m, taken in order

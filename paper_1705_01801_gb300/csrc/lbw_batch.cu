@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <fstream>
+#include <functional>
 #include <sstream>
 #include <string>
 #include <vector>
@@ -31,10 +32,16 @@ using namespace dev;
 
 constexpr int kBatchBX = 32;  // q2 columns per tile (one warp per tile row)
 
+// One work item: planes z0 .. z1 - 1 of the tile at (x0, y0) of a member (`by` interior rows of a
+// full-row tile, unused by the other kernels).
+struct __align__(16) BatchItem {
+  int member, x0, y0, z0, z1, by, pad[2];
+};
+
 template <typename S>
 __global__ void __launch_bounds__(512) batch_step_kernel(const StepArgs<S>* __restrict__ members,
-                                                         const int4* __restrict__ items, int n_items,
-                                                         int lz, unsigned long long* counters,
+                                                         const BatchItem* __restrict__ items,
+                                                         int n_items, unsigned long long* counters,
                                                          int nprobe, long long cap) {
   using R = typename Store<S>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -44,8 +51,8 @@ __global__ void __launch_bounds__(512) batch_step_kernel(const StepArgs<S>* __re
   __shared__ unsigned long long t_sample;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x, nthr = blockDim.x * blockDim.y;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-    const int4 item = items[it];  // member, x0, y0, z0
-    const unsigned* src = reinterpret_cast<const unsigned*>(members + item.x);
+    const BatchItem item = items[it];
+    const unsigned* src = reinterpret_cast<const unsigned*>(members + item.member);
     unsigned* dst = reinterpret_cast<unsigned*>(&A);
     for (int k = tid; k < (int)(sizeof(StepArgs<S>) / 4); k += nthr) dst[k] = src[k];
     if (tid == 0) {
@@ -53,9 +60,8 @@ __global__ void __launch_bounds__(512) batch_step_kernel(const StepArgs<S>* __re
       t_sample = counters[1];
     }
     __syncthreads();
-    const int z1 = min(item.w + lz, A.n3);
-    scan_probes(A, item.y, item.z, item.w, z1, probe_list, &probe_cnt);
-    march_tile(A, item.y, item.z, item.w, z1, reinterpret_cast<R*>(smem_raw), probe_list, probe_cnt,
+    scan_probes(A, item.x0, item.y0, item.z0, item.z1, probe_list, &probe_cnt);
+    march_tile(A, item.x0, item.y0, item.z0, item.z1, reinterpret_cast<R*>(smem_raw), probe_list, probe_cnt,
                t_sample);
     __syncthreads();  // shared memory is reused by the next item
   }
@@ -101,7 +107,7 @@ __device__ __forceinline__ void mbar_inval(unsigned bar) {
 template <typename S, int BY>
 __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
     const StepArgs<S>* __restrict__ members, const CUtensorMap* __restrict__ maps, int src,
-    const int4* __restrict__ items, int n_items, int lz, unsigned long long* counters, int nprobe,
+    const BatchItem* __restrict__ items, int n_items, unsigned long long* counters, int nprobe,
     long long cap) {
   using R = typename Store<S>::R;
   using L = BatchTmaLayout<S, BY>;
@@ -138,6 +144,10 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
   const unsigned SL = OFF + 128, RHO = SL + NB * SLOTB, TAB = RHO + RHOB;
   auto full_at = [&](int k) { return sbase + OFF + 8u * k; };
   auto empty_at = [&](int k) { return sbase + OFF + 8u * (NB + k); };
+  // programmatic dependent launch, as in step_tma_kernel: the next step's CTAs may be scheduled while
+  // this one drains, and nothing of the previous step is touched before it has completed
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   if (tid == 0) {
     abort_flag = 0;
     t_sample = counters[1];
@@ -147,9 +157,9 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
 
   bool fresh = true;
   for (int it = next_it; it < n_items;) {
-    const int4 item = items[it];  // member, x0 (data column), y0 (may be -1), z0
+    const BatchItem item = items[it];  // x0: data column, y0 may be -1
     {
-      const unsigned* from = reinterpret_cast<const unsigned*>(members + item.x);
+      const unsigned* from = reinterpret_cast<const unsigned*>(members + item.member);
       unsigned* to = reinterpret_cast<unsigned*>(&A);
       for (int k = tid; k < (int)(sizeof(StepArgs<S>) / 4); k += nthr) to[k] = from[k];
     }
@@ -167,8 +177,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
     }
     fresh = false;
     __syncthreads();  // every thread has read next_it for this item
-    const int x0 = item.y, y0 = item.z, z0 = item.w;
-    const int z1 = min(z0 + lz, A.n3);
+    const int x0 = item.x0, y0 = item.y0, z0 = item.z0, z1 = item.z1;
     const bool p3 = A.bc[4] == LBW_BC_PERIODIC;
     if (tid < A.nprobe) {
       const int pq1 = A.probe_q[3 * tid], pq2 = A.probe_q[3 * tid + 1], pq3 = A.probe_q[3 * tid + 2];
@@ -176,8 +185,8 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
         probe_list[atomicAdd(&probe_cnt, 1)] = tid;
     }
     __syncthreads();
-    const CUtensorMap* tm_f = maps + 3 * item.x + src;
-    const CUtensorMap* tm_t = maps + 3 * item.x + 2;
+    const CUtensorMap* tm_f = maps + 3 * item.member + src;
+    const CUtensorMap* tm_t = maps + 3 * item.member + 2;
 
     auto wait_bar = [&](unsigned bar, unsigned parity) -> bool {
       long long n = 0;
@@ -378,14 +387,22 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
         }
       };
 
-      auto stepB = [&](int zc, R (&fc)[7][NPT], const R (&rp)[NPT], const R (&rc)[NPT],
-                       const R (&rn)[NPT], int slz, int rbz) {
+      // step B's shared inputs of the plane that collides, read before step A of the plane ahead
+      // writes another rho plane, so their latency overlaps with it (as in step_tma_kernel)
+      struct BIn { R ru[NPT], rd[NPT], lft, rgt; };
+      auto loadB = [&](BIn& b, int rbz) {
         const unsigned cur = RHO + rbz * (PS * RS) + myrho;
-        R ru[NPT], rd[NPT];
-        VecN<R, NPT>::ld(reinterpret_cast<const R*>(smem_raw + cur + PW * RS), ru);
-        VecN<R, NPT>::ld(reinterpret_cast<const R*>(smem_raw + cur - PW * RS), rd);
-        const R rl[NPT] = {ldr(cur - RS), rc[0]};
-        const R rrt[NPT] = {rc[1], ldr(cur + NPT * RS)};
+        VecN<R, NPT>::ld(reinterpret_cast<const R*>(smem_raw + cur + PW * RS), b.ru);
+        VecN<R, NPT>::ld(reinterpret_cast<const R*>(smem_raw + cur - PW * RS), b.rd);
+        b.lft = ldr(cur - RS);
+        b.rgt = ldr(cur + NPT * RS);
+      };
+      auto stepB = [&](int zc, R (&fc)[7][NPT], const R (&rp)[NPT], const R (&rc)[NPT],
+                       const R (&rn)[NPT], int slz, const BIn& bi) {
+        const R (&ru)[NPT] = bi.ru;
+        const R (&rd)[NPT] = bi.rd;
+        const R rl[NPT] = {bi.lft, rc[0]};
+        const R rrt[NPT] = {rc[1], bi.rgt};
         const unsigned T = TAB + slz * TABB + (w - 1) * (T_SLOTS * RS);
         R c[T_SLOTS];
 #pragma unroll
@@ -493,10 +510,17 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
       auto iter = [&](int zz, R (&fc)[7][NPT], R (&fn)[7][NPT], const R (&rp)[NPT],
                       const R (&rc)[NPT], R (&rn)[NPT], bool collide) {
         const bool in = wait_bar(full_at(RG ? s1 : s2), (unsigned)(uw & 1));
-        if (in) stepA(zz + 1, fn, rn, sz, s1, s2, rb1, true);
-        const bool go = !named_sync_or(1, NCW * 32, !in || abort_flag);
-        if (go && collide) stepB(zz, fc, rp, rc, rn, sz, rbz);
+        // plane zz collides before the barrier: it needs rho of plane zz + 1 only at the warp's own
+        // nodes (measured against the barrier first: FP32 870 -> 859 us, FP16 934 -> 897 us on 48
+        // trumpets; the full-row kernel, whose registers are capped, spills and is 3 % slower)
+        if (in) {
+          BIn bi;
+          if (collide) loadB(bi, rbz);
+          stepA(zz + 1, fn, rn, sz, s1, s2, rb1, true);
+          if (collide) stepB(zz, fc, rp, rc, rn, sz, bi);
+        }
         if (lane == 0) mbar_arrive(empty_at(sz));
+        const bool go = !named_sync_or(1, NCW * 32, !in || abort_flag);
         advance();
         return go;
       };
@@ -566,11 +590,10 @@ constexpr size_t batch_row_smem() {
   return 128 + 128 + 5 * (size_t)L::SLOTB + L::RHOB + 5 * (size_t)L::TABB;
 }
 
-// items: (member, BY_m, first interior row y0 (may be -1), z0)
 template <typename S>
 __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) batch_row_kernel(
     const StepArgs<S>* __restrict__ members, const CUtensorMap* __restrict__ maps, int src,
-    const int4* __restrict__ items, int n_items, int lz, unsigned long long* counters, int nprobe,
+    const BatchItem* __restrict__ items, int n_items, unsigned long long* counters, int nprobe,
     long long cap) {
   using R = typename Store<S>::R;
   using L = BatchRowLayout<S>;
@@ -595,6 +618,10 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
   const unsigned SL = OFF + 128, RHO = SL + NB * SLOTB, TAB = RHO + L::RHOB;
   auto full_at = [&](int k) { return sbase + OFF + 8u * k; };
   auto empty_at = [&](int k) { return sbase + OFF + 8u * (NB + k); };
+  // programmatic dependent launch, as in step_tma_kernel: the next step's CTAs may be scheduled while
+  // this one drains, and nothing of the previous step is touched before it has completed
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   if (tid == 0) {
     abort_flag = 0;
     t_sample = counters[1];
@@ -604,9 +631,9 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
 
   bool fresh = true;
   for (int it = next_it; it < n_items;) {
-    const int4 item = items[it];
+    const BatchItem item = items[it];
     {
-      const unsigned* from = reinterpret_cast<const unsigned*>(members + item.x);
+      const unsigned* from = reinterpret_cast<const unsigned*>(members + item.member);
       unsigned* to = reinterpret_cast<unsigned*>(&A);
       for (int k = tid; k < (int)(sizeof(StepArgs<S>) / 4); k += nthr) to[k] = from[k];
     }
@@ -624,8 +651,7 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
     }
     fresh = false;
     __syncthreads();  // every thread has read next_it for this item
-    const int BYm = item.y, y0 = item.z, z0 = item.w, ROWS = BYm + 2;
-    const int z1 = min(z0 + lz, A.n3);
+    const int BYm = item.by, y0 = item.y0, z0 = item.z0, z1 = item.z1, ROWS = BYm + 2;
     const bool p3 = A.bc[4] == LBW_BC_PERIODIC;
     const int n2 = A.n2, n2w = n2 + (n2 & 1), BW = (n2 + V - 1) / V * V;
     if (tid < A.nprobe) {
@@ -633,8 +659,8 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
       if (pq1 >= y0 && pq1 < y0 + BYm && pq3 >= z0 && pq3 < z1) probe_list[atomicAdd(&probe_cnt, 1)] = tid;
     }
     __syncthreads();
-    const CUtensorMap* tm_f = maps + 3 * item.x + src;
-    const CUtensorMap* tm_t = maps + 3 * item.x + 2;
+    const CUtensorMap* tm_f = maps + 3 * item.member + src;
+    const CUtensorMap* tm_t = maps + 3 * item.member + 2;
 
     auto wait_bar = [&](unsigned bar, unsigned parity) -> bool {
       long long n = 0;
@@ -932,17 +958,17 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
   finish_step(counters, nprobe, cap, gridDim.x);
 }
 
-// Ghost columns of padded rows from the data columns they copy (G on each side: ghost-left =
-// the last G data columns, ghost-right = the first G), for a member's buffer f: the full-row
-// kernel does not keep them, the 64-column kernel reads them.
+// Rows of one layout into another's, for a member's populations: `rows` rows of n2 values, with
+// the ghost columns of the periodic wrap where the new layout has them (G > 0).
 template <typename S>
-__global__ void ghost_fill_kernel(S* __restrict__ f, long long rows, int pitch, int n2, int G) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < rows * 2 * G;
-       k += (long long)gridDim.x * blockDim.x) {
-    S* row = f + (k / (2 * G)) * pitch;
-    const int j = (int)(k % (2 * G));
-    if (j < G) row[j] = row[n2 + j];
-    else row[n2 + j] = row[j];
+__global__ void relayout_kernel(const S* __restrict__ from, S* __restrict__ to, long long rows, int n2, int pitch0,
+                                int col0, int pitch1, int G) {
+  const int w = n2 + 2 * G;
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < rows * w; k += (long long)gridDim.x * blockDim.x) {
+    const long long r = k / w;
+    const int c = (int)(k - r * w);
+    const int q2 = c < G ? n2 - G + c : (c >= G + n2 ? c - G - n2 : c - G);
+    to[r * pitch1 + c] = from[r * pitch0 + col0 + q2];
   }
 }
 
@@ -1004,7 +1030,7 @@ struct lbw_batch {
   int nprobe = 0;
   int64_t cap = 0;
   void* members[2] = {nullptr, nullptr};  // StepArgs arrays for source buffer 0 / 1
-  int4* items = nullptr;
+  BatchItem* items = nullptr;
   int n_items = 0, blocks = 0;
   Shape shape;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -1020,6 +1046,8 @@ struct lbw_batch {
   int nsrc = 0, src_kind = 0;
   double src_amp = 0.0;
   void* src = nullptr;
+  std::vector<int32_t> src_q;      // their nodes and frequencies, for another storage layout
+  std::vector<double> src_omega;
 };
 
 namespace {
@@ -1132,6 +1160,75 @@ int padded_pitch(int n2, size_t es) {
   return (n2 + 2 * ghost_cols(es) + v - 1) / v * v;
 }
 
+// The device list of the harmonic sources in the members' present storage layout.
+lbw_status build_sources(lbw_batch* b) {
+  std::vector<SourceEntry> h;
+  const size_t per = b->src_q.size() / 3 / b->n;
+  h.reserve(per * b->n);
+  for (int m = 0; m < b->n; ++m) {
+    const Grid& g = b->views[m];
+    const int pitch = g.pitch ? g.pitch : g.d.n[1], n2 = g.d.n[1];
+    for (size_t k = 0; k < per; ++k) {
+      const int32_t* q = b->src_q.data() + (m * per + k) * 3;
+      SourceEntry e{};
+      e.off = (long long)b->foff[m] + ((long long)q[2] * g.d.n[0] + q[0]) * pitch + g.col0 + q[1];
+      e.ps = pop_stride(&g);
+      // a ghost column near the wrap holds a copy
+      e.ghost = g.col0 == 0 ? 0 : q[1] < g.col0 ? n2 : q[1] >= n2 - g.col0 ? -n2 : 0;
+      e.sg = lattice_sqrtg(g.d, q[0], q[2]);
+      e.omega = b->src_omega[m];
+      e.cs2 = g.d.cs2;
+      h.push_back(e);
+    }
+  }
+  drop_graphs(b);  // captured chains carry the source list
+  if (b->src) { cudaFreeAsync(b->src, b->stream); b->src = nullptr; }
+  b->nsrc = 0;
+  if (!h.empty()) {
+    LBW_CUDA(cudaMallocAsync((void**)&b->src, sizeof(SourceEntry) * h.size(), b->stream));
+    LBW_CUDA(cudaMemcpyAsync(b->src, h.data(), sizeof(SourceEntry) * h.size(), cudaMemcpyHostToDevice, b->stream));
+    LBW_CUDA(cudaStreamSynchronize(b->stream));
+    b->nsrc = (int)h.size();
+  }
+  return LBW_OK;
+}
+
+// Rows as the full-row kernel stores them: no ghost columns, n2 rounded up to 16 bytes.  Ghost
+// columns lie between the rows and share their sectors, so whole rows fetch them too: without
+// them (and with longer segments) 32 trumpets move 60.9 instead of 71.2 bytes per node from and to
+// DRAM, 728 -> 601 us per step of 48 trumpets.
+int dense_pitch(int n2, size_t es) {
+  const int v = (int)(16 / es);
+  return (n2 + v - 1) / v * v;
+}
+
+// The current state into the layout that the launch shape wants (dense rows for full-row tiles,
+// else ghost columns, rebuilt even where the layout stays: the resident kernel does not keep
+// them), through the other buffer.
+lbw_status use_layout(lbw_batch* b, bool rebuild) {
+  if (!b->tma) return LBW_OK;
+  const size_t es = es_of(b->prec);
+  const int G = b->shape.by == 0 ? 0 : ghost_cols(es);
+  if (b->views[0].col0 == G && !(rebuild && G > 0)) return LBW_OK;
+  for (Grid& g : b->views) {
+    const int n2 = g.d.n[1], pitch = G ? padded_pitch(n2, es) : dense_pitch(n2, es);
+    const long long rows = 7LL * g.d.n[0] * g.d.n[2];
+    const int blocks = (int)std::min<long long>((rows * n2 + 255) / 256, 4096);
+    prec_dispatch(b->prec, [&](auto tag) {
+      using S = decltype(tag);
+      relayout_kernel<S><<<blocks, 256, 0, b->stream>>>(reinterpret_cast<const S*>(g.f[b->cur]),
+                                                        reinterpret_cast<S*>(g.f[1 - b->cur]), rows, n2, g.pitch, g.col0,
+                                                        pitch, G);
+      return 0;
+    });
+    g.pitch = pitch;
+    g.col0 = G;
+  }
+  LBW_CUDA(cudaGetLastError());
+  b->cur = 1 - b->cur;
+  return build_sources(b);
+}
+
 // Tensor maps of every member for tile rows `by`: 4-D views (stored column, q1, q3,
 // population) of both buffers with (64 + 2 G) x (by + 2) boxes, 3-D view of the table.
 lbw_status build_batch_maps(lbw_batch* b, int by) {
@@ -1165,43 +1262,96 @@ lbw_status build_batch_maps(lbw_batch* b, int by) {
   return LBW_OK;
 }
 
-// work list for the current shape: items of each member in (q3 segment, q1 tile, q2 tile)
-// order, so consecutive CTAs hold spatial neighbours.  TMA tiles are 64 columns wide and
-// start at q1 = -1 when (n1 - 1) is a multiple of the tile rows (no halo row on a face).
-// Full-row tiles (shape.by == 0) have the member's own row count: items (member, rows, y0, z0).
-lbw_status build_items(lbw_batch* b) {
-  std::vector<int4> items;
-  for (int m = 0; m < b->n; ++m) {
-    const lbw_grid_desc& d = b->views[m].d;
-    if (b->tma && b->shape.by == 0) {
-      const int by = row_tile_rows(d.n[1], b->views[m].elem) - 2;
-      if (by < kRowMinBY) return fail(LBW_EINVAL, "ensemble member does not fit a full-row tile");
-      const int y_start = (d.n[0] - 1) % by == 0 ? -1 : 0;
-      for (int z0 = 0; z0 < d.n[2]; z0 += b->shape.lz)
-        for (int y0 = y_start; y0 < d.n[0]; y0 += by) items.push_back(make_int4(m, by, y0, z0));
-      continue;
-    }
-    const int bx = b->tma ? kTmaBatchBX : kBatchBX;
-    const int y_start = (b->tma && (d.n[0] - 1) % b->shape.by == 0) ? -1 : 0;
-    for (int z0 = 0; z0 < d.n[2]; z0 += b->shape.lz)
-      for (int y0 = y_start; y0 < d.n[0]; y0 += b->shape.by)
-        for (int x0 = 0; x0 < d.n[1]; x0 += bx) items.push_back(make_int4(m, x0, y0, z0));
-  }
-  if (b->items) cudaFreeAsync(b->items, b->stream);
-  b->items = nullptr;
-  LBW_CUDA(cudaMallocAsync((void**)&b->items, sizeof(int4) * items.size(), b->stream));
-  LBW_CUDA(cudaMemcpyAsync(b->items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice,
-                           b->stream));
-  b->n_items = (int)items.size();
+// CTAs of the persistent grid for a launch shape
+size_t grid_slots(const Shape& shape) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  b->blocks = std::max(1, std::min(b->n_items, sms * b->shape.cps));
+  return (size_t)sms * shape.cps;
+}
+
+// work list for a launch shape: items of each member in (q3 segment, q1 tile, q2 tile) order, so
+// consecutive CTAs hold spatial neighbours.  TMA tiles are 64 columns wide and start at q1 = -1
+// when (n1 - 1) is a multiple of the tile rows (no halo row on a face).  Full-row tiles
+// (by == 0) have the member's own row count.  Persistent kernels end when the last item does, so
+// on the tile kernels the last two turns of the list are cut into halves and the last turn of
+// those again: long segments, which re-read fewer boundary planes, then cost nothing at the end
+// (48 trumpets: 64-plane segments 601 us per step, 16-plane segments 637; cutting more turns or
+// again: 605 to 609).
+lbw_status list_items(const lbw_batch* b, const Shape& shape, std::vector<BatchItem>& items) {
+  items.clear();
+  for (int m = 0; m < b->n; ++m) {
+    const lbw_grid_desc& d = b->views[m].d;
+    const bool rows = b->tma && shape.by == 0;
+    const int by = rows ? row_tile_rows(d.n[1], b->views[m].elem) - 2 : shape.by;
+    if (rows && by < kRowMinBY) return fail(LBW_EINVAL, "ensemble member does not fit a full-row tile");
+    const int bx = rows ? d.n[1] : b->tma ? kTmaBatchBX : kBatchBX;
+    const int y_start = (b->tma && (d.n[0] - 1) % by == 0) ? -1 : 0;
+    for (long long z0 = 0; z0 < d.n[2]; z0 += shape.lz)
+      for (int y0 = y_start; y0 < d.n[0]; y0 += by)
+        for (int x0 = 0; x0 < d.n[1]; x0 += bx)
+          items.push_back(BatchItem{m, x0, y0, (int)z0, (int)std::min<long long>(z0 + shape.lz, d.n[2]), by, {0, 0}});
+  }
+  const size_t slots = grid_slots(shape);
+  if (b->tma && items.size() > 2 * slots)
+    for (const size_t turns : {2, 1}) {
+      const size_t first = items.size() - std::min(items.size(), turns * slots);
+      const std::vector<BatchItem> tail(items.begin() + first, items.end());
+      items.resize(first);
+      for (const bool upper : {false, true})
+        for (BatchItem t : tail) {
+          const int mid = t.z1 - t.z0 > 4 ? (t.z0 + t.z1) / 2 : t.z1;
+          (upper ? t.z0 : t.z1) = mid;
+          if (t.z0 < t.z1) items.push_back(t);
+        }
+    }
+  return LBW_OK;
+}
+
+// Segment length (and the kernel, among the tile rows `bys`) that ends a step first when CTAs
+// claim the items in order: an item costs its planes and some four more to fill the pipeline, a
+// plane as measured at two CTAs per SM (us: full-row tile 1.0, 7 rows of 64 columns 1.25, 4 rows 0.9).
+Shape best_shape(const lbw_batch* b, const std::vector<int>& bys) {
+  Shape best = b->shape;
+  double best_cost = 1e300;
+  std::vector<BatchItem> items;
+  for (const int by : bys)
+    for (const int lz : {8, 12, 16, 24, 32, 48, 64}) {
+      const Shape shape{by, lz, std::min(2, tma_cps(b->prec, by))};
+      if (shape.cps < 1 || list_items(b, shape, items) != LBW_OK) continue;
+      const double plane = by == 0 ? 1.0 : by == 7 ? 1.25 : 0.9;
+      std::vector<double> free_at(std::min(items.size(), grid_slots(shape)), 0.0);  // a heap, earliest first
+      for (const BatchItem& t : items) {
+        std::pop_heap(free_at.begin(), free_at.end(), std::greater<double>());
+        free_at.back() += plane * (t.z1 - t.z0 + 4);
+        std::push_heap(free_at.begin(), free_at.end(), std::greater<double>());
+      }
+      const double cost = *std::max_element(free_at.begin(), free_at.end());
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = shape;
+      }
+    }
+  return best;
+}
+
+lbw_status build_items(lbw_batch* b) {
+  std::vector<BatchItem> items;
+  const lbw_status st = list_items(b, b->shape, items);
+  if (st != LBW_OK) return st;
+  if (b->items) cudaFreeAsync(b->items, b->stream);
+  b->items = nullptr;
+  LBW_CUDA(cudaMallocAsync((void**)&b->items, sizeof(BatchItem) * items.size(), b->stream));
+  LBW_CUDA(cudaMemcpyAsync(b->items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice,
+                           b->stream));
+  b->n_items = (int)items.size();
+  b->blocks = (int)std::max<size_t>(1, std::min(items.size(), grid_slots(b->shape)));
   drop_graphs(b);
   return LBW_OK;
 }
 
-lbw_status refresh(lbw_batch* b) {
-  lbw_status st = build_items(b);
+lbw_status refresh(lbw_batch* b, bool rebuild_ghosts = false) {
+  lbw_status st = use_layout(b, rebuild_ghosts);
+  if (st == LBW_OK) st = build_items(b);
   if (st != LBW_OK) return st;
   if (b->tma) {
     st = build_batch_maps(b, b->shape.by);
@@ -1218,27 +1368,32 @@ lbw_status refresh(lbw_batch* b) {
 template <typename S>
 cudaError_t launch_batch_t(lbw_batch* b, int src) {
   using R = typename Store<S>::R;
-  if constexpr (sizeof(S) >= 4) {
-    if (b->tma && b->shape.by == 0) {
-      batch_row_kernel<S><<<b->blocks, dim3(32, kRowWarps + 1), batch_row_smem<S>(), b->stream>>>(
-          reinterpret_cast<const StepArgs<S>*>(b->members[src]), reinterpret_cast<const CUtensorMap*>(b->maps),
-          src, b->items, b->n_items, b->shape.lz, b->counters, b->nprobe, b->cap);
-      return cudaGetLastError();
-    }
-  }
   if (b->tma) {
-    return batch_tma_dispatch<S>(b->shape.by, [&](auto kern, size_t smem) {
-      kern<<<b->blocks, dim3(32, b->shape.by + 3), smem, b->stream>>>(
-          reinterpret_cast<const StepArgs<S>*>(b->members[src]), reinterpret_cast<const CUtensorMap*>(b->maps),
-          src, b->items, b->n_items, b->shape.lz, b->counters, b->nprobe, b->cap);
-      return cudaGetLastError();
-    });
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(b->blocks);
+    cfg.stream = b->stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto launch = [&](auto kern, size_t smem, int warps) {
+      cfg.blockDim = dim3(32, warps);
+      cfg.dynamicSmemBytes = smem;
+      return cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<const StepArgs<S>*>(b->members[src]),
+                                reinterpret_cast<const CUtensorMap*>(b->maps), src, (const BatchItem*)b->items, b->n_items,
+                                b->counters, b->nprobe, (long long)b->cap);
+    };
+    if constexpr (sizeof(S) >= 4) {
+      if (b->shape.by == 0) return launch(batch_row_kernel<S>, batch_row_smem<S>(), kRowWarps + 1);
+    }
+    return batch_tma_dispatch<S>(b->shape.by,
+                                 [&](auto kern, size_t smem) { return launch(kern, smem, b->shape.by + 3); });
   }
   const dim3 block(kBatchBX, b->shape.by);
   const size_t smem = 3 * (size_t)(kBatchBX + 2) * (b->shape.by + 2) * sizeof(R);
   batch_step_kernel<S><<<b->blocks, block, smem, b->stream>>>(
-      reinterpret_cast<const StepArgs<S>*>(b->members[src]), b->items, b->n_items, b->shape.lz,
-      b->counters, b->nprobe, b->cap);
+      reinterpret_cast<const StepArgs<S>*>(b->members[src]), b->items, b->n_items, b->counters, b->nprobe, b->cap);
   return cudaGetLastError();
 }
 
@@ -1413,9 +1568,13 @@ lbw_status lbw_batch_create(const lbw_grid_desc* descs, int32_t n, void* stream,
       g.col0 = ghost_cols(g.elem);
     }
     b->foff[m] = ftot;
-    // 256-byte aligned member slices
+    // 256-byte aligned member slices, with room for the ghost columns in every layout
     const size_t align = 256 / g.elem;
     ftot += (7 * (size_t)pop_stride(&g) + align - 1) / align * align;
+    if (b->rowk) {
+      g.pitch = dense_pitch(d.n[1], g.elem);
+      g.col0 = 0;
+    }
     b->toff[m] = tab_all.size();
     tab_all.insert(tab_all.end(), tab.begin(), tab.end());
     while (tab_all.size() % 64) tab_all.push_back(0.0);
@@ -1453,13 +1612,8 @@ lbw_status lbw_batch_create(const lbw_grid_desc* descs, int32_t n, void* stream,
     g.table = static_cast<unsigned char*>(b->table) + b->toff[m] * rs;
     g.counters = b->counters;
   }
-  if (b->rowk) {  // full-row tiles where every member fits one (the autotuner's pick on trumpets)
-    b->shape.by = 0;
-    b->shape.lz = 16;
-    b->shape.cps = std::min(2, row_cps(b->prec));
-  } else if (b->tma) {
-    b->shape.by = 7;
-    b->shape.cps = std::min(2, tma_cps(b->prec, 7));
+  if (b->tma) {  // full-row tiles where every member fits one (the autotuner's pick on trumpets)
+    b->shape = best_shape(b, {b->rowk ? 0 : 7});
   } else {
     b->shape.cps = std::min(2, b->prec == LBW_F32 ? max_cps<float>() : 2);
   }
@@ -1573,42 +1727,21 @@ lbw_status lbw_batch_source(lbw_batch* b, const int32_t* host_q, int32_t per_mem
   if (per_member > 0 && (!host_q || !host_omega)) return fail(LBW_EINVAL, "sources need nodes and frequencies");
   if (kind != 0 && kind != 1) return fail(LBW_EINVAL, "kind must be 0 (P) or 1 (J'_z)");
   if (!std::isfinite(amp)) return fail(LBW_EINVAL, "amp must be finite");
-  const bool p_all = b->tma;  // padded members carry ghost copies of nodes near the wrap
-  std::vector<SourceEntry> h;
-  h.reserve((size_t)b->n * per_member);
   for (int m = 0; m < b->n && per_member > 0; ++m) {
-    const Grid& g = b->views[m];
+    const lbw_grid_desc& d = b->views[m].d;
     if (!std::isfinite(host_omega[m])) return fail(LBW_EINVAL, "omega must be finite");
-    const int pitch = g.pitch ? g.pitch : g.d.n[1], col0 = g.col0, n2 = g.d.n[1];
     for (int k = 0; k < per_member; ++k) {
       const int32_t* q = host_q + ((size_t)m * per_member + k) * 3;
-      if (q[0] < 0 || q[0] >= g.d.n[0] || q[1] < 0 || q[1] >= n2 || q[2] < 0 || q[2] >= g.d.n[2])
-        return fail(LBW_EINVAL, "source node outside its member's lattice");
-      SourceEntry e{};
-      e.off = (long long)b->foff[m] + ((long long)q[2] * g.d.n[0] + q[0]) * pitch + col0 + q[1];
-      e.ps = pop_stride(&g);
-      e.ghost = 0;
-      if (p_all && col0 > 0 && g.d.bc[2] == LBW_BC_PERIODIC) {
-        if (q[1] < col0) e.ghost = n2;
-        else if (q[1] >= n2 - col0) e.ghost = -n2;
-      }
-      e.sg = lattice_sqrtg(g.d, q[0], q[2]);
-      e.omega = host_omega[m];
-      e.cs2 = g.d.cs2;
-      h.push_back(e);
+      for (int a = 0; a < 3; ++a)
+        if (q[a] < 0 || q[a] >= d.n[a]) return fail(LBW_EINVAL, "source node outside its member's lattice");
     }
   }
-  drop_graphs(b);  // captured chains carry the source list
-  if (b->src) { cudaFreeAsync(b->src, b->stream); b->src = nullptr; }
-  b->nsrc = 0;
-  if (!h.empty()) {
-    LBW_CUDA(cudaMallocAsync(&b->src, sizeof(SourceEntry) * h.size(), b->stream));
-    LBW_CUDA(cudaMemcpyAsync(b->src, h.data(), sizeof(SourceEntry) * h.size(), cudaMemcpyHostToDevice, b->stream));
-    LBW_CUDA(cudaStreamSynchronize(b->stream));
-    b->nsrc = (int)h.size();
-    b->src_kind = kind;
-    b->src_amp = amp;
-  }
+  b->src_q.assign(host_q, host_q + (size_t)b->n * per_member * 3);
+  b->src_omega.assign(host_omega, host_omega + (per_member > 0 ? b->n : 0));
+  b->src_kind = kind;
+  b->src_amp = amp;
+  const lbw_status st = build_sources(b);
+  if (st != LBW_OK) return st;
   return b->res ? resident_sources(b->res, host_q, per_member, b->stream) : LBW_OK;
 }
 
@@ -1790,11 +1923,12 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
     }
   }
   b->shape = best;
+  const bool was_resident = b->res != nullptr && !resident;
   if (!resident) {
     resident_destroy(b->res, b->stream);
     b->res = nullptr;
   }
-  lbw_status st = refresh(b);
+  lbw_status st = refresh(b, was_resident);
   if (st != LBW_OK) return st;
   // trial steps ran on the ensemble's buffers: callers tune before lbw_batch_init
   LBW_CUDA(cudaMemsetAsync(b->counters, 0, 4 * sizeof(unsigned long long), b->stream));
@@ -1824,25 +1958,11 @@ lbw_status lbw_batch_set_shape(lbw_batch* b, int32_t tile_rows, int32_t seg_plan
   resident_destroy(b->res, b->stream);
   b->res = nullptr;
   b->shape = Shape{tile_rows, seg_planes, ctas_per_sm};
-  lbw_status st = refresh(b);
+  lbw_status st = refresh(b, was_resident);
   if (st != LBW_OK) {
     b->shape = old;
     refresh(b);
     return st;
-  }
-  if (b->tma && (old.by == 0 || was_resident) && tile_rows != 0) {  // the 64-column kernel reads ghost columns
-    for (int m = 0; m < b->n; ++m) {
-      const Grid& g = b->views[m];
-      const long long rows = 7LL * g.d.n[0] * g.d.n[2];
-      const int blocks = (int)std::min<long long>((rows * 2 * g.col0 + 255) / 256, 1024);
-      prec_dispatch(b->prec, [&](auto tag) {
-        using S = decltype(tag);
-        ghost_fill_kernel<S><<<blocks, 256, 0, b->stream>>>(reinterpret_cast<S*>(g.f[b->cur]), rows, g.pitch,
-                                                             g.d.n[1], g.col0);
-        return 0;
-      });
-    }
-    LBW_CUDA(cudaGetLastError());
   }
   LBW_CUDA(cudaStreamSynchronize(b->stream));
   return LBW_OK;
