@@ -252,6 +252,8 @@ cudaError_t apply_sources(Grid* g, int buf) {
                         g->src_kind, g->src_amp, g->counters, g->stream);
 }
 
+cudaError_t step_once(Grid* g, int src) { return g->ragged ? ragged_launch(g, src) : launch_step(g, src); }
+
 // A chain of `len` steps starting from buffer `start`, captured once and replayed.
 lbw_status ensure_graph(Grid* g, int start, int len) {
   if (g->graph[start] && g->graph_len == len) return LBW_OK;
@@ -261,7 +263,7 @@ lbw_status ensure_graph(Grid* g, int start, int len) {
   int src = start;
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < len && e == cudaSuccess; ++s) {
-    e = launch_step(g, src);
+    e = step_once(g, src);
     if (e == cudaSuccess) e = apply_sources(g, 1 - src);
     src = 1 - src;
   }
@@ -330,7 +332,11 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
     lbw_destroy(g);
     return s;
   };
-  const size_t fbytes = (size_t)7 * g->nn * g->elem;
+  if (d.geom_mode != LBW_GEOM_ANALYTIC && ragged_fits(d)) {
+    st = ragged_plan(g);
+    if (st != LBW_OK) return cleanup(st);
+  }
+  const size_t fbytes = (size_t)7 * pop_stride(g) * g->elem;
   for (int k = 0; k < 2; ++k) {
     cudaError_t e = cudaMallocAsync(&g->f[k], fbytes, g->stream);
     if (e != cudaSuccess) {
@@ -357,7 +363,12 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
   if (e == cudaSuccess) e = cudaMemsetAsync(g->f[0], 0, fbytes, g->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "create: upload"));
-  step_launch_shape(g);
+  if (g->ragged) {
+    st = ragged_refresh(g);
+    if (st != LBW_OK) return cleanup(st);
+  } else {
+    step_launch_shape(g);
+  }
   if (d.geom_mode == LBW_GEOM_ANALYTIC && g->tma_by == 0)
     return cleanup(fail(LBW_EINVAL, "geom_mode ANALYTIC needs the tile kernel: q2 extent a multiple of "
                                     "the tile width (64, or 128 for 16-bit storage) and non-periodic q1"));
@@ -378,6 +389,7 @@ void lbw_destroy(lbw_grid* g) {
   if (!g) return;
   drop_graphs(g);
   resident_destroy(g->res, g->stream);
+  ragged_destroy(g);
   for (int k = 0; k < 2; ++k)
     if (g->f[k]) cudaFreeAsync(g->f[k], g->stream);
   if (g->table) cudaFreeAsync(g->table, g->stream);
@@ -447,7 +459,7 @@ lbw_status lbw_step(lbw_grid* g, int64_t n_steps) {
     }
   }
   while (left > 0) {
-    LBW_CUDA(launch_step(g, g->cur));
+    LBW_CUDA(step_once(g, g->cur));
     LBW_CUDA(apply_sources(g, 1 - g->cur));
     g->cur = 1 - g->cur;
     --left;
@@ -485,9 +497,10 @@ lbw_status lbw_source(lbw_grid* g, const int32_t* host_q, int32_t n, int32_t kin
     const int q1 = host_q[3 * k], q2 = host_q[3 * k + 1], q3 = host_q[3 * k + 2];
     if (q1 < 0 || q1 >= g->d.n[0] || q2 < 0 || q2 >= g->d.n[1] || q3 < 0 || q3 >= g->d.n[2])
       return fail(LBW_EINVAL, "source node outside the lattice");
-    h[k].off = ((long long)q3 * g->d.n[0] + q1) * g->d.n[1] + q2;
-    h[k].ps = g->nn;
-    h[k].ghost = 0;
+    const int n2 = g->d.n[1];
+    h[k].off = ((long long)q3 * g->d.n[0] + q1) * (g->pitch ? g->pitch : n2) + g->col0 + q2;
+    h[k].ps = pop_stride(g);
+    h[k].ghost = g->col0 == 0 ? 0 : q2 < g->col0 ? n2 : q2 >= n2 - g->col0 ? -n2 : 0;
     h[k].pad = 0;
     h[k].sg = lattice_sqrtg(g->d, q1, q3);
     h[k].omega = omega;
@@ -530,6 +543,10 @@ lbw_status lbw_probe(lbw_grid* g, const int32_t* host_q, int32_t n, int64_t capa
     LBW_CUDA(cudaMemsetAsync(g->series, 0, sizeof(double) * n * capacity, g->stream));
     g->nprobe = n;
     g->cap = capacity;
+  }
+  if (g->ragged) {
+    const lbw_status st = ragged_refresh(g);
+    if (st != LBW_OK) return st;
   }
   // restart the sample counter (counters[1]); the step count is kept
   LBW_CUDA(cudaMemsetAsync(g->counters + 1, 0, sizeof(unsigned long long), g->stream));

@@ -1314,12 +1314,17 @@ Shape best_shape(const lbw_batch* b, const std::vector<int>& bys) {
   Shape best = b->shape;
   double best_cost = 1e300;
   std::vector<BatchItem> items;
-  for (const int by : bys)
-    for (const int lz : {8, 12, 16, 24, 32, 48, 64}) {
-      const Shape shape{by, lz, std::min(2, tma_cps(b->prec, by))};
+  for (const int by : bys) {
+    const int cps = std::min(2, tma_cps(b->prec, by));
+    for (const int lz : {64, 48, 32, 24, 16, 12, 8}) {
+      const Shape shape{by, lz, cps};
       if (shape.cps < 1 || list_items(b, shape, items) != LBW_OK) continue;
       const double plane = by == 0 ? 1.0 : by == 7 ? 1.25 : 0.9;
-      std::vector<double> free_at(std::min(items.size(), grid_slots(shape)), 0.0);  // a heap, earliest first
+      const size_t slots = std::min(items.size(), grid_slots(shape));
+      double work = 0.0;
+      for (const BatchItem& t : items) work += plane * (t.z1 - t.z0 + 4);
+      if (work >= best_cost * slots) continue;  // not even with every CTA busy to the end
+      std::vector<double> free_at(slots, 0.0);  // a heap, earliest first
       for (const BatchItem& t : items) {
         std::pop_heap(free_at.begin(), free_at.end(), std::greater<double>());
         free_at.back() += plane * (t.z1 - t.z0 + 4);
@@ -1331,6 +1336,7 @@ Shape best_shape(const lbw_batch* b, const std::vector<int>& bys) {
         best = shape;
       }
     }
+  }
   return best;
 }
 
@@ -1349,6 +1355,10 @@ lbw_status build_items(lbw_batch* b) {
   return LBW_OK;
 }
 
+lbw_status upload_members(lbw_batch* b) {
+  return prec_dispatch(b->prec, [&](auto tag) { return upload_args<decltype(tag)>(b); });
+}
+
 lbw_status refresh(lbw_batch* b, bool rebuild_ghosts = false) {
   lbw_status st = use_layout(b, rebuild_ghosts);
   if (st == LBW_OK) st = build_items(b);
@@ -1357,12 +1367,7 @@ lbw_status refresh(lbw_batch* b, bool rebuild_ghosts = false) {
     st = build_batch_maps(b, b->shape.by);
     if (st != LBW_OK) return st;
   }
-  switch (b->prec) {
-    case LBW_F64: return upload_args<double>(b);
-    case LBW_F32: return upload_args<float>(b);
-    case LBW_F16S: return upload_args<__half>(b);
-    default: return upload_args<__nv_bfloat16>(b);
-  }
+  return upload_members(b);
 }
 
 template <typename S>
@@ -1979,3 +1984,69 @@ lbw_status lbw_batch_info(lbw_batch* b, int64_t* total_nodes, int32_t* tile_rows
 }
 
 }  // extern "C"
+
+// ---------------------------------------------------------------- ragged single lattices ----
+//
+// A single lattice whose q2 extent is no multiple of the tile width steps as an ensemble of one
+// member on the kernels above (the register-pipelined kernel it took before reaches a third of
+// their rate: 100 x 100 x 250 FP32 80 -> 35 us per step, 200 x 250 x 256 291 -> 143, FP64 1483
+// -> 1233).  The lbw_batch only refers to the lattice's buffers and counters.
+namespace lbw {
+
+bool ragged_fits(const lbw_grid_desc& d) {
+  const size_t es = es_of(d.prec);
+  const long long nn = (long long)d.n[0] * d.n[1] * d.n[2];
+  // FP32 and FP64 only: 16-bit storage would round in another order than the kernel it has had;
+  // smaller lattices run many steps per launch
+  if ((d.prec != LBW_F32 && d.prec != LBW_F64) || nn <= (d.prec == LBW_F32 ? 640000 : 320000)) return false;
+  if (d.n[1] % kTmaBatchBX == 0 || d.bc[2] != LBW_BC_PERIODIC || d.bc[0] == LBW_BC_PERIODIC || d.n[0] < 2 ||
+      d.n[1] < 2 * ghost_cols(es) || 7LL * d.n[0] * d.n[2] * padded_pitch(d.n[1], es) >= (1LL << 31))
+    return false;
+  return tma_cps(d.prec, 7) > 0 && tma_cps(d.prec, 4) > 0;
+}
+
+lbw_status ragged_plan(Grid* g) {
+  lbw_batch* b = new (std::nothrow) lbw_batch();
+  if (!b) return fail(LBW_ENOMEM, "host allocation failed");
+  b->n = 1;
+  b->prec = g->d.prec;
+  b->stream = g->stream;
+  b->tma = true;
+  b->rowk = row_tile_rows(g->d.n[1], g->elem) > 0 && row_cps(g->d.prec) > 0;
+  b->views.assign(1, *g);
+  b->foff.assign(1, 0);
+  std::vector<int> bys = {7, 4};
+  if (b->rowk) bys.push_back(0);
+  b->shape = best_shape(b, bys);
+  Grid& v = b->views[0];
+  v.pitch = g->pitch = b->shape.by == 0 ? dense_pitch(g->d.n[1], g->elem) : padded_pitch(g->d.n[1], g->elem);
+  v.col0 = g->col0 = b->shape.by == 0 ? 0 : ghost_cols(g->elem);
+  g->ragged = b;
+  return LBW_OK;
+}
+
+lbw_status ragged_refresh(Grid* g) {
+  lbw_batch* b = g->ragged;
+  Grid& v = b->views[0];
+  for (int k = 0; k < 2; ++k) b->f[k] = v.f[k] = g->f[k];
+  v.table = g->table;
+  v.counters = b->counters = g->counters;
+  b->nprobe = g->nprobe;
+  b->probe_q = g->probe_q;
+  b->series = g->series;
+  b->cap = g->cap;
+  return b->items ? upload_members(b) : refresh(b);
+}
+
+cudaError_t ragged_launch(Grid* g, int src) { return launch_batch(g->ragged, src); }
+
+void ragged_destroy(Grid* g) {
+  lbw_batch* b = g->ragged;
+  if (!b) return;
+  for (void* p : {b->members[0], b->members[1], (void*)b->items, b->maps})
+    if (p) cudaFreeAsync(p, g->stream);
+  delete b;
+  g->ragged = nullptr;
+}
+
+}  // namespace lbw

@@ -28,6 +28,9 @@ enum TableSlot {
 
 constexpr int kMaxProbes = 64;
 
+}  // namespace lbw
+struct lbw_batch;
+namespace lbw {
 struct Resident;  // plan of the multi-step kernel (lbw_resident.h)
 
 struct Grid {
@@ -64,6 +67,7 @@ struct Grid {
   alignas(64) unsigned char tmaps[5 * 128];  // tensor maps: f[0] main/halo, f[1] main/halo, table
   dim3 grid_dim;
   Resident* res = nullptr;  // small lattices: many steps per launch (nullptr: a launch per step)
+  lbw_batch* ragged = nullptr;  // ragged q2 extents: stepped by the ensemble kernels (lbw_batch.cu)
   // captured step chains, one per parity of the starting buffer
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   int graph_len = 0;
@@ -114,6 +118,15 @@ inline void equilibrium_coefs(const lbw_grid_desc& d, double* E, double* two0) {
 inline long long pop_stride(const Grid* g) {
   return g->pitch ? (long long)g->d.n[0] * g->d.n[2] * g->pitch : g->nn;
 }
+
+// single lattices on the ensemble kernels (lbw_batch.cu): whether a descriptor takes them, the launch
+// shape and storage layout (before the buffers are allocated), the launch arguments (after, and when
+// the probes change) and one time step
+bool ragged_fits(const lbw_grid_desc& d);
+lbw_status ragged_plan(Grid* g);
+lbw_status ragged_refresh(Grid* g);
+cudaError_t ragged_launch(Grid* g, int src);
+void ragged_destroy(Grid* g);
 
 // kernels (lbw_step.cu) ---------------------------------------------------------------------
 cudaError_t launch_step(Grid* g, int src);             // one time step, buffer src -> 1-src
