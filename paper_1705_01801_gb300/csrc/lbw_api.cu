@@ -279,11 +279,12 @@ lbw_status ensure_graph(Grid* g, int start, int len) {
 
 // Samples recorded so far (counters[1]) and the wait flag (counters[3]): a step whose bounded
 // wait for staged data ran out raises the flag and leaves the state undefined.
-lbw_status read_counters(Grid* g, unsigned long long* recorded) {
-  unsigned long long c[3] = {0, 0, 0};
+lbw_status read_counters(Grid* g, unsigned long long* recorded, unsigned long long* bad = nullptr) {
+  unsigned long long c[5] = {0, 0, 0, 0, 0};
   LBW_CUDA(cudaMemcpyAsync(c, g->counters + 1, sizeof(c), cudaMemcpyDeviceToHost, g->stream));
   LBW_CUDA(cudaStreamSynchronize(g->stream));
   if (recorded) *recorded = c[0];
+  if (bad) *bad = c[4];
   if (c[2]) return fail(LBW_ETIMEOUT, "a time step's bounded wait for staged data ran out; the state is "
                                       "undefined until lbw_init");
   return LBW_OK;
@@ -347,7 +348,7 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
   const size_t rs = real_size(d.prec);
   const size_t tbytes = tab.size() * rs;
   cudaError_t e = cudaMallocAsync(&g->table, tbytes, g->stream);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&g->counters, 5 * sizeof(unsigned long long), g->stream);
+  if (e == cudaSuccess) e = cudaMallocAsync((void**)&g->counters, 6 * sizeof(unsigned long long), g->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cleanup(fail(LBW_ENOMEM, "table allocation failed"));
@@ -359,7 +360,7 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
     src = tf.data();
   }
   e = cudaMemcpyAsync(g->table, src, tbytes, cudaMemcpyHostToDevice, g->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->counters, 0, 5 * sizeof(unsigned long long), g->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->counters, 0, 6 * sizeof(unsigned long long), g->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(g->f[0], 0, fbytes, g->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "create: upload"));
@@ -408,21 +409,15 @@ lbw_status lbw_init(lbw_grid* g, const lbw_pulse* host_pulses, int32_t n_pulses)
   if (n_pulses > 0 && !host_pulses) return fail(LBW_EINVAL, "host_pulses is NULL");
   for (int k = 0; k < n_pulses; ++k)
     if (!(host_pulses[k].sigma > 0)) return fail(LBW_EINVAL, "pulse sigma must be > 0");
-  double* d_p = nullptr;
-  const size_t pb = sizeof(double) * 5 * std::max(1, n_pulses);
-  LBW_CUDA(cudaMallocAsync(&d_p, pb, g->stream));
-  std::vector<double> hp(5 * std::max(1, n_pulses), 0.0);
-  for (int k = 0; k < n_pulses; ++k) {
-    hp[5 * k] = host_pulses[k].x[0];
-    hp[5 * k + 1] = host_pulses[k].x[1];
-    hp[5 * k + 2] = host_pulses[k].x[2];
-    hp[5 * k + 3] = host_pulses[k].sigma;
-    hp[5 * k + 4] = host_pulses[k].amp;
-  }
+  unsigned char* d_p = nullptr;
+  const size_t pb = pulse_bytes(n_pulses);
+  LBW_CUDA(cudaMallocAsync((void**)&d_p, pb + init_scratch_bytes(g->d), g->stream));
+  std::vector<unsigned char> hp(pb);
+  pack_pulses(host_pulses, n_pulses, hp.data());
   cudaError_t e = cudaMemcpyAsync(d_p, hp.data(), pb, cudaMemcpyHostToDevice, g->stream);
-  if (e == cudaSuccess) e = launch_init(g, d_p, n_pulses);
+  if (e == cudaSuccess) e = launch_init(g, d_p, n_pulses, d_p + pb);
   cudaFreeAsync(d_p, g->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->counters, 0, 5 * sizeof(unsigned long long), g->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->counters, 0, 6 * sizeof(unsigned long long), g->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   if (e != cudaSuccess) return cuda_fail(e, "init");
   g->steps = 0;
@@ -627,41 +622,24 @@ lbw_status lbw_spectrum_series(const double* host_x, int64_t T, int32_t n_series
 
 lbw_status lbw_get_field(lbw_grid* g, double* host_P) {
   if (!g || !host_P) return fail(LBW_EINVAL, "NULL argument");
-  double* d = nullptr;
-  LBW_CUDA(cudaMallocAsync(&d, sizeof(double) * g->nn, g->stream));
-  cudaError_t e = launch_field(g, d);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(host_P, d, sizeof(double) * g->nn, cudaMemcpyDeviceToHost, g->stream);
-  cudaFreeAsync(d, g->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+  const cudaError_t e = read_field(g, host_P, g->counters + 5);
   if (e != cudaSuccess) return cuda_fail(e, "get_field");
-  const lbw_status st = read_counters(g, nullptr);
+  unsigned long long bad = 0;
+  const lbw_status st = read_counters(g, nullptr, &bad);
   if (st != LBW_OK) return st;
-  for (int64_t x = 0; x < g->nn; ++x)
-    if (!std::isfinite(host_P[x])) return fail(LBW_EUNSTABLE, "field holds a non-finite value (unstable run)");
-  return LBW_OK;
+  return bad ? fail(LBW_EUNSTABLE, "field holds a non-finite value (unstable run)") : LBW_OK;
 }
 
 lbw_status lbw_get_populations(lbw_grid* g, double* host_f) {
   if (!g || !host_f) return fail(LBW_EINVAL, "NULL argument");
-  double* d = nullptr;
-  LBW_CUDA(cudaMallocAsync(&d, sizeof(double) * 7 * g->nn, g->stream));
-  cudaError_t e = launch_to_double(g, d);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(host_f, d, sizeof(double) * 7 * g->nn, cudaMemcpyDeviceToHost, g->stream);
-  cudaFreeAsync(d, g->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+  const cudaError_t e = read_populations(g, host_f);
   if (e != cudaSuccess) return cuda_fail(e, "get_populations");
   return read_counters(g, nullptr);
 }
 
 lbw_status lbw_set_populations(lbw_grid* g, const double* host_f) {
   if (!g || !host_f) return fail(LBW_EINVAL, "NULL argument");
-  double* d = nullptr;
-  LBW_CUDA(cudaMallocAsync(&d, sizeof(double) * 7 * g->nn, g->stream));
-  cudaError_t e = cudaMemcpyAsync(d, host_f, sizeof(double) * 7 * g->nn, cudaMemcpyHostToDevice, g->stream);
-  if (e == cudaSuccess) e = launch_from_double(g, d);
-  cudaFreeAsync(d, g->stream);
+  cudaError_t e = write_populations(g, host_f);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   if (e != cudaSuccess) return cuda_fail(e, "set_populations");
   g->initialised = true;

@@ -1661,28 +1661,25 @@ void lbw_batch_destroy(lbw_batch* b) {
 
 lbw_status lbw_batch_init(lbw_batch* b, const lbw_pulse* host_pulses, const int32_t* host_counts) {
   if (!b || !host_counts) return fail(LBW_EINVAL, "NULL argument");
-  size_t total = 0;
+  size_t total = 0, scratch = 0;
   for (int m = 0; m < b->n; ++m) {
     if (host_counts[m] < 0) return fail(LBW_EINVAL, "negative pulse count");
     total += host_counts[m];
+    scratch = std::max(scratch, init_scratch_bytes(b->views[m].d));  // one member's at a time
   }
   if (total > 0 && !host_pulses) return fail(LBW_EINVAL, "host_pulses is NULL");
-  std::vector<double> hp(5 * std::max<size_t>(1, total), 0.0);
-  for (size_t k = 0; k < total; ++k) {
+  for (size_t k = 0; k < total; ++k)
     if (!(host_pulses[k].sigma > 0)) return fail(LBW_EINVAL, "pulse sigma must be > 0");
-    hp[5 * k] = host_pulses[k].x[0];
-    hp[5 * k + 1] = host_pulses[k].x[1];
-    hp[5 * k + 2] = host_pulses[k].x[2];
-    hp[5 * k + 3] = host_pulses[k].sigma;
-    hp[5 * k + 4] = host_pulses[k].amp;
-  }
-  double* d_p = nullptr;
-  LBW_CUDA(cudaMallocAsync(&d_p, hp.size() * sizeof(double), b->stream));
-  cudaError_t e = cudaMemcpyAsync(d_p, hp.data(), hp.size() * sizeof(double), cudaMemcpyHostToDevice, b->stream);
+  std::vector<unsigned char> hp(pulse_bytes((int)total));
+  pack_pulses(host_pulses, (int)total, hp.data());
+  unsigned char* d_p = nullptr;
+  LBW_CUDA(cudaMallocAsync((void**)&d_p, hp.size() + scratch, b->stream));
+  cudaError_t e = cudaMemcpyAsync(d_p, hp.data(), hp.size(), cudaMemcpyHostToDevice, b->stream);
+  const size_t one = pulse_bytes(1);
   size_t off = 0;
   for (int m = 0; m < b->n && e == cudaSuccess; ++m) {
     b->views[m].cur = b->cur;
-    e = launch_init(&b->views[m], d_p + 5 * off, host_counts[m]);
+    e = launch_init(&b->views[m], d_p + one * off, host_counts[m], d_p + hp.size());
     off += host_counts[m];
   }
   cudaFreeAsync(d_p, b->stream);
@@ -1826,13 +1823,7 @@ lbw_status lbw_batch_get_populations(lbw_batch* b, int32_t member, double* host_
   if (member < 0 || member >= b->n) return fail(LBW_EINVAL, "member out of range");
   Grid& g = b->views[member];
   g.cur = b->cur;
-  double* d = nullptr;
-  LBW_CUDA(cudaMallocAsync(&d, sizeof(double) * 7 * g.nn, b->stream));
-  cudaError_t e = launch_to_double(&g, d);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(host_f, d, sizeof(double) * 7 * g.nn, cudaMemcpyDeviceToHost, b->stream);
-  cudaFreeAsync(d, b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  const cudaError_t e = read_populations(&g, host_f);
   if (e != cudaSuccess) return cuda_fail(e, "batch populations");
   return batch_counters(b, nullptr);
 }

@@ -48,7 +48,8 @@ struct Grid {
   double* series = nullptr;       // device, nprobe x cap
   int64_t cap = 0;
   // device counters: [0] steps since init, [1] samples recorded, [2] last-block ticket,
-  // [3] timeout flag of a bounded wait, [4] injected-timeout request (tests)
+  // [3] timeout flag of a bounded wait, [4] injected-timeout request (tests), [5] a value of the
+  // field read last is not finite
   unsigned long long* counters = nullptr;
   int64_t steps = 0;       // host mirror of counters[0]
   bool initialised = false;
@@ -130,10 +131,6 @@ void ragged_destroy(Grid* g);
 
 // kernels (lbw_step.cu) ---------------------------------------------------------------------
 cudaError_t launch_step(Grid* g, int src);             // one time step, buffer src -> 1-src
-cudaError_t launch_init(Grid* g, const double* d_pulses, int npulse);
-cudaError_t launch_field(Grid* g, double* d_P);        // P of the current state
-cudaError_t launch_to_double(Grid* g, double* d_f);    // current populations -> doubles
-cudaError_t launch_from_double(Grid* g, const double* d_f);
 void step_launch_shape(Grid* g);                       // choose bx, by, lz, grid_dim
 // After step t (counters[0] = t): every source node's populations become the equilibrium that
 // carries amp sin(omega t) as P (kind 0) or as J'_z (kind 1).
@@ -143,6 +140,18 @@ cudaError_t launch_sources(int prec, void* base, const SourceEntry* d_entries, i
 // first, strides in bytes of dimensions 1 .. rank - 1; false when the driver refuses it
 bool encode_tiled_map(void* map, int prec, int rank, void* base, const uint64_t* dims,
                       const uint64_t* strides, const uint32_t* box);
+
+// state (lbw_state.cu) -----------------------------------------------------------------------
+// Initial state of buffer g->cur from packed pulses and scratch on the device (enqueued)
+size_t init_scratch_bytes(const lbw_grid_desc& d);
+size_t pulse_bytes(int n);
+void pack_pulses(const lbw_pulse* p, int n, void* out);
+cudaError_t launch_init(Grid* g, const void* d_pulses, int npulse, void* d_scratch);
+// P and the populations of the current state to host arrays, and back from one (enqueued, through
+// the other population buffer); *d_bad tells whether a value of P is not finite
+cudaError_t read_field(Grid* g, double* host_P, unsigned long long* d_bad);
+cudaError_t read_populations(Grid* g, double* host_f);
+cudaError_t write_populations(Grid* g, const double* host_f);
 
 // spectrum (lbw_spectrum.cu) ----------------------------------------------------------------
 // For each of `count` estimates (est_stride values apart in d_x) the k strongest peaks (lowest =

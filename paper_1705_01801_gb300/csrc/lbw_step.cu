@@ -1,4 +1,4 @@
-// lbw_step.cu -- the fused stream + collide time step and the state kernels.
+// lbw_step.cu -- the fused stream + collide time step.
 //
 // One launch advances the whole lattice by one time step of the paper's scheme
 // (Sec. III "Summarizing"): pull streaming along xi_i with the face rules of Sec. IV.A,
@@ -962,132 +962,6 @@ bool build_tmaps(Grid* g, int by, int bx) {
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// ---------------------------------------------------------------- initial state ----------
-
-struct InitGeom {
-  int kind, profile;
-  double h[3], x0[3], geom[4];
-};
-
-__device__ void embed_dev(const InitGeom& G, double u1, double u2, double u3, double X[3]) {
-  double s2, c2;
-  switch (G.kind) {
-    case LBW_CARTESIAN: X[0] = u1; X[1] = u2; X[2] = u3; break;
-    case LBW_POLAR:
-    case LBW_CYLINDRICAL:
-      sincos(u2, &s2, &c2);
-      X[0] = u1 * c2; X[1] = u1 * s2; X[2] = u3;
-      break;
-    case LBW_TRUMPET: {
-      double s;
-      if (G.profile == 0) s = pow(G.geom[0] - u3, -G.geom[1]);
-      else s = (G.geom[0] + G.geom[1] * exp(G.geom[2] * u3)) / (G.geom[0] + G.geom[1]);
-      sincos(u2, &s2, &c2);
-      X[0] = u1 * s * c2; X[1] = u1 * s * s2; X[2] = u3;
-      break;
-    }
-    default: {
-      double s3, c3;
-      sincos(u3, &s3, &c3);
-      sincos(u2, &s2, &c2);
-      const double rr = G.geom[0] + u1 * c3;
-      X[0] = rr * c2; X[1] = rr * s2; X[2] = u1 * s3;
-    }
-  }
-}
-
-// rho0 = sqrt(g) P0, P0 a sum of Gaussian pulses in the embedding distance (FP64 math).
-template <typename R>
-__global__ void init_rho_kernel(InitGeom G, const double* __restrict__ pulses, int npulse,
-                                const R* __restrict__ tab, int n1, int n2, int n3, R* rho0) {
-  const long long nn = (long long)n1 * n2 * n3;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < nn;
-       x += (long long)gridDim.x * blockDim.x) {
-    const int q2 = (int)(x % n2);
-    const int q1 = (int)((x / n2) % n1);
-    const int q3 = (int)(x / ((long long)n1 * n2));
-    double X[3];
-    embed_dev(G, G.x0[0] + (q1 + 0.5) * G.h[0], G.x0[1] + (q2 + 0.5) * G.h[1],
-              G.x0[2] + (q3 + 0.5) * G.h[2], X);
-    double P0 = 0.0;
-    for (int k = 0; k < npulse; ++k) {
-      const double* p = pulses + 5 * k;
-      const double d2 = (X[0] - p[0]) * (X[0] - p[0]) + (X[1] - p[1]) * (X[1] - p[1]) +
-                        (X[2] - p[2]) * (X[2] - p[2]);
-      const double e = d2 / (2.0 * p[3] * p[3]);
-      if (e < 80.0) P0 += p[4] * exp(-e);  // beyond: below 2e-35 of the amplitude
-    }
-    rho0[x] = (R)((double)tab[((long long)q3 * n1 + q1) * T_SLOTS + T_SG] * P0);
-  }
-}
-
-// Post-collision state at rest: f*_i = f_i^eq(rho0, F(rho0) / 2), F from the same table.
-template <typename S>
-__global__ void init_f_kernel(const StepArgs<S> a, const typename Store<S>::R* __restrict__ rho0) {
-  using R = typename Store<S>::R;
-  const bool p1 = a.bc[0] == LBW_BC_PERIODIC, p2 = a.bc[2] == LBW_BC_PERIODIC,
-             p3 = a.bc[4] == LBW_BC_PERIODIC;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < a.nn;
-       x += (long long)gridDim.x * blockDim.x) {
-    const int q2 = (int)(x % a.n2);
-    const int q1 = (int)((x / a.n2) % a.n1);
-    const int q3 = (int)(x / ((long long)a.n1 * a.n2));
-    auto at = [&](int r1, int r2, int r3) -> R {
-      r1 = resolve(r1, a.n1, p1); r2 = resolve(r2, a.n2, p2); r3 = resolve(r3, a.n3, p3);
-      if (r1 < 0 || r2 < 0 || r3 < 0) return R(0);
-      return rho0[node(r1, r2, r3, a.n1, a.n2)];
-    };
-    const R* c = a.tab + ((long long)q3 * a.n1 + q1) * T_SLOTS;
-    const R rho = rho0[x];
-    const R ru = at(q1 + 1, q2, q3), rd = at(q1 - 1, q2, q3);
-    const R rn = at(q1, q2, q3 + 1), rp = at(q1, q2, q3 - 1);
-    R rr = at(q1, q2 + 1, q3), rl = at(q1, q2 - 1, q3);
-    if (q2 == 0 && !p2) rl = a.s2lo * rho;
-    if (q2 == a.n2 - 1 && !p2) rr = a.s2hi * rho;
-    const R D1 = c[T_A1P] * ru - c[T_A1M] * rd + c[T_C13P] * rn - c[T_C13M] * rp + c[T_S1] * rho;
-    const R D3 = c[T_B13P] * ru - c[T_B13M] * rd + c[T_C33P] * rn - c[T_C33M] * rp + c[T_S3] * rho;
-    const R D2 = c[T_H22] * (rr - rl);
-    const R j1 = R(0.5) * (c[T_MG1] * rho - D1), j2 = R(-0.5) * D2,
-            j3 = R(0.5) * (c[T_MG3] * rho - D3);
-    const R e = R(0.5) * a.cs2 * rho;
-    R o[7] = {R(0.5) * a.two_w0 * rho, e + R(0.5) * j1, e - R(0.5) * j1, e + R(0.5) * j2,
-              e - R(0.5) * j2, e + R(0.5) * j3, e - R(0.5) * j3};
-    const long long px = ((long long)q3 * a.n1 + q1) * a.pitch + a.col0 + q2;
-    // ghost copy of a node near the periodic wrap (padded storage only)
-    int gq = -1;
-    if (a.col0 > 0 && p2) gq = q2 < a.col0 ? a.col0 + a.n2 + q2 : (q2 >= a.n2 - a.col0 ? q2 - a.n2 + a.col0 : -1);
-#pragma unroll
-    for (int i = 0; i < 7; ++i) {
-      R v = o[i];
-      if (Store<S>::kScaled) v *= a.inv_w[i];
-      Store<S>::st(a.fout + (long long)i * a.ps + px, v);
-      if (gq >= 0) Store<S>::st(a.fout + (long long)i * a.ps + (px - a.col0 - q2) + gq, v);
-    }
-  }
-}
-
-template <typename S>
-cudaError_t launch_init_t(Grid* g, const double* d_pulses, int npulse) {
-  using R = typename Store<S>::R;
-  InitGeom G;
-  G.kind = g->d.kind;
-  G.profile = g->d.horn_profile;
-  for (int a = 0; a < 3; ++a) { G.h[a] = g->d.h[a]; G.x0[a] = g->d.x0[a]; }
-  for (int k = 0; k < 4; ++k) G.geom[k] = g->d.geom[k];
-  // rho0 goes to the scratch bytes of the other population buffer (>= N values of R)
-  R* rho0 = reinterpret_cast<R*>(g->f[1 - g->cur]);
-  const int threads = 256;
-  const int blocks = (int)std::min<long long>((g->nn + threads - 1) / threads, 152LL * 16);
-  init_rho_kernel<R><<<blocks, threads, 0, g->stream>>>(
-      G, d_pulses, npulse, reinterpret_cast<const R*>(g->table), g->d.n[0], g->d.n[1],
-      g->d.n[2], rho0);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  StepArgs<S> a = step_args<S>(*g, 1 - g->cur);  // fout = current buffer
-  init_f_kernel<S><<<blocks, threads, 0, g->stream>>>(a, rho0);
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- harmonic sources -------
 
 template <typename S>
@@ -1097,88 +971,6 @@ __global__ void source_kernel(S* __restrict__ base, const SourceEntry* __restric
   if (k >= n) return;
   const SourceEntry s = e[k];
   impose_source(base, s, kind, amp * sin(s.omega * (double)counters[0]));
-}
-
-// ---------------------------------------------------------------- read-out ---------------
-
-// Storage address of dense node x (q2 fastest) in a possibly padded layout.
-struct Pad {
-  int n2, pitch, col0;
-  __device__ long long at(long long x) const {
-    return (x / n2) * pitch + col0 + (x % n2);
-  }
-};
-
-template <typename S>
-__global__ void field_kernel(const S* __restrict__ f, long long nn, long long ps, Pad pad, int n1,
-                             const typename Store<S>::R* __restrict__ tab, double w0, double w1,
-                             double* __restrict__ P) {
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < nn;
-       x += (long long)gridDim.x * blockDim.x) {
-    const int q1 = (int)((x / pad.n2) % n1);
-    const int q3 = (int)(x / ((long long)n1 * pad.n2));
-    const long long px = pad.at(x);
-    double r = 0.0;
-    for (int i = 0; i < 7; ++i) {
-      double v = (double)Store<S>::ld(f + (long long)i * ps + px);
-      if (Store<S>::kScaled) v *= (i == 0 ? w0 : w1);
-      r += v;
-    }
-    P[x] = r * (double)tab[((long long)q3 * n1 + q1) * T_SLOTS + T_INVSG];
-  }
-}
-
-template <typename S>
-__global__ void to_double_kernel(const S* __restrict__ f, long long nn, long long ps, Pad pad,
-                                 double w0, double w1, double* __restrict__ out) {
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < 7 * nn;
-       x += (long long)gridDim.x * blockDim.x) {
-    const long long i = x / nn, node = x - i * nn;
-    double v = (double)Store<S>::ld(f + i * ps + pad.at(node));
-    if (Store<S>::kScaled) v *= (i == 0 ? w0 : w1);
-    out[x] = v;
-  }
-}
-
-// Dense doubles into storage; padded storage also gets the ghost copies of a periodic q2.
-template <typename S>
-__global__ void from_double_kernel(const double* __restrict__ in, long long nn, long long ps,
-                                   Pad pad, bool p2, double w0, double w1, S* __restrict__ f) {
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < 7 * nn;
-       x += (long long)gridDim.x * blockDim.x) {
-    const long long i = x / nn, node = x - i * nn;
-    double v = in[x];
-    if (Store<S>::kScaled) v /= (i == 0 ? w0 : w1);
-    const long long px = pad.at(node);
-    const typename Store<S>::R r = (typename Store<S>::R)v;
-    Store<S>::st(f + i * ps + px, r);
-    if (pad.col0 > 0 && p2) {
-      const int q2 = (int)(node % pad.n2);
-      const long long row = px - pad.col0 - q2;
-      if (q2 < pad.col0) Store<S>::st(f + i * ps + row + pad.col0 + pad.n2 + q2, r);
-      if (q2 >= pad.n2 - pad.col0) Store<S>::st(f + i * ps + row + q2 - pad.n2 + pad.col0, r);
-    }
-  }
-}
-
-template <typename S>
-cudaError_t launch_readout_t(Grid* g, int what, double* d_out, const double* d_in) {
-  const int threads = 256;
-  const int blocks = 152 * 8;
-  const S* f = reinterpret_cast<const S*>(g->f[g->cur]);
-  const Pad pad{g->d.n[1], g->pitch ? g->pitch : g->d.n[1], g->col0};
-  const long long ps = pop_stride(g);
-  if (what == 0)
-    field_kernel<S><<<blocks, threads, 0, g->stream>>>(
-        f, g->nn, ps, pad, g->d.n[0], reinterpret_cast<const typename Store<S>::R*>(g->table),
-        g->w0, g->w1, d_out);
-  else if (what == 1)
-    to_double_kernel<S><<<blocks, threads, 0, g->stream>>>(f, g->nn, ps, pad, g->w0, g->w1, d_out);
-  else
-    from_double_kernel<S><<<blocks, threads, 0, g->stream>>>(
-        d_in, g->nn, ps, pad, g->d.bc[2] == LBW_BC_PERIODIC, g->w0, g->w1,
-        reinterpret_cast<S*>(g->f[g->cur]));
-  return cudaGetLastError();
 }
 
 template <typename F>
@@ -1228,26 +1020,6 @@ bool encode_tiled_map(void* map, int prec, int rank, void* base, const uint64_t*
 
 cudaError_t launch_step(Grid* g, int src) {
   return dispatch(g->d.prec, [&](auto tag) { return launch_step_t<decltype(tag)>(g, src); });
-}
-
-cudaError_t launch_init(Grid* g, const double* d_pulses, int npulse) {
-  return dispatch(g->d.prec,
-                  [&](auto tag) { return launch_init_t<decltype(tag)>(g, d_pulses, npulse); });
-}
-
-cudaError_t launch_field(Grid* g, double* d_P) {
-  return dispatch(g->d.prec,
-                  [&](auto tag) { return launch_readout_t<decltype(tag)>(g, 0, d_P, nullptr); });
-}
-
-cudaError_t launch_to_double(Grid* g, double* d_f) {
-  return dispatch(g->d.prec,
-                  [&](auto tag) { return launch_readout_t<decltype(tag)>(g, 1, d_f, nullptr); });
-}
-
-cudaError_t launch_from_double(Grid* g, const double* d_f) {
-  return dispatch(g->d.prec,
-                  [&](auto tag) { return launch_readout_t<decltype(tag)>(g, 2, nullptr, d_f); });
 }
 
 // Launch shape.  TMA tile kernel (q2 extent a multiple of the tile width, non-periodic q1):
