@@ -10,12 +10,17 @@
 // other CTAs own), puts their post-stream rho into shared memory, and after one __syncthreads
 // collides its nodes (the populations stay in registers) and stores them to the other buffer.
 // Measured per step, a launch per step -> here: disk 10.6 -> 3.2 us, the paper's 20 x 200 x 30
-// torus in FP64 with a ring source 29.3 -> 13.7 us, 41 pipes of 10,000 FP32 nodes with sources
-// 176 -> 16 us.  What bounds it: 2.2 us of barrier and load latency for the smallest lattices,
-// the FP64 pipe for FP64, instruction issue and L1 beyond a few hundred nodes per CTA.
+// torus in FP64 with a ring source 29.3 -> 11.3 us, 41 pipes of 10,000 FP32 nodes with sources
+// 176 -> 9.5 us (38 + 3 of them in two turns).  What bounds it: 2.0 us of barrier and load
+// latency for the smallest lattices, the FP64 pipe for FP64, load latency beyond a few hundred
+// nodes per CTA (25 % of the issue slots busy).
 //
-// One CTA per SM: 512 threads with one or two nodes each for small boxes, else 1024 with two or
-// four (512 threads of eight nodes spilled and measured the same).
+// Sources that impose P replace the node's outputs as they are stored, from values that the last
+// threads compute (an FP64 sine) while thread 0 waits at the barrier; other sources take a pass
+// through memory behind one more __syncthreads (which cost 5 us per step when all did).
+//
+// One CTA per SM, of as many threads as leave the populations in registers (kResShapes; 1024
+// threads of two or three nodes spilled and were 10 to 30 % slower).
 //
 // The launch is cooperative, so all CTAs are resident and the barrier (one arrival counter per
 // lattice, cleared before each launch) completes; its wait is bounded like every device wait
@@ -66,23 +71,38 @@ template <typename S> __device__ __forceinline__ typename Store<S>::R ld_pop(con
   return Store<S>::ld_smem(p);
 }
 
-struct Face {
+// Strides of the populations and of the q1 and q3 axes, in elements.
+struct Strides {
   int ps, s1, s3;
-  int off[6];  // source of the population that streams in through a face, from the node
+};
+// Per face, the source of the population that streams in through it (relative to the node) and
+// the factor it arrives with.  In shared memory: most nodes need neither.
+template <typename R>
+struct Faces {
+  int off[6];
+  R m[6];
 };
 
 // Pull streaming of the seven populations into the node at element x (flag bit 2 axis + side:
-// the node lies on that face).  `m` are the faces' factors, `walls` the faces where it is not 1.
-template <typename S, bool TILE>
-__device__ __forceinline__ void pull_node(const S* f, int x, unsigned fl, unsigned walls, const Face& F,
-                                          const typename Store<S>::R (&m)[6],
-                                          const typename Store<S>::R (&wt)[2],
-                                          typename Store<S>::R (&v)[7]) {
-  using R = typename Store<S>::R;
+// the node lies on that face), in two parts: the loads, which have no branches, so that those of
+// all of a thread's nodes are in flight together, then the factors of the walls it lies on.
+template <typename S>
+__device__ __forceinline__ void load_node(const S* f, int x, unsigned fl, const Strides& F,
+                                          const Faces<typename Store<S>::R>& faces, typename Store<S>::R (&v)[7]) {
   const int o[6] = {F.ps - F.s1, 2 * F.ps + F.s1, 3 * F.ps - 1, 4 * F.ps + 1, 5 * F.ps - F.s3, 6 * F.ps + F.s3};
   v[0] = ld_pop(f + x);
 #pragma unroll
-  for (int i = 0; i < 6; ++i) v[i + 1] = ld_pop(f + (x + ((fl >> i) & 1 ? F.off[i] : o[i])));
+  for (int i = 0; i < 6; ++i) {
+    int d = o[i];
+    if ((fl >> i) & 1) d = faces.off[i];
+    v[i + 1] = ld_pop(f + (x + d));
+  }
+}
+
+// `walls`: the faces whose factor is not 1.
+template <typename S, bool TILE>
+__device__ __forceinline__ void finish_node(unsigned fl, unsigned walls, const Faces<typename Store<S>::R>& faces,
+                                            const typename Store<S>::R (&wt)[2], typename Store<S>::R (&v)[7]) {
   if constexpr (Store<S>::kScaled && !TILE) {
     v[0] *= wt[0];
 #pragma unroll
@@ -90,7 +110,8 @@ __device__ __forceinline__ void pull_node(const S* f, int x, unsigned fl, unsign
   }
   if (fl & walls) {
 #pragma unroll
-    for (int i = 0; i < 6; ++i) v[i + 1] = (fl >> i) & 1 ? m[i] * v[i + 1] : v[i + 1];
+    for (int i = 0; i < 6; ++i)
+      if ((fl >> i) & 1) v[i + 1] *= faces.m[i];
   }
 }
 
@@ -206,11 +227,26 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   using R = typename Store<S>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) StepArgs<S> A;
+  __shared__ Faces<R> faces;
   __shared__ int probe_x[kMaxProbes], probe_id[kMaxProbes];
   __shared__ int probe_cnt, halo_cnt, bad, x13_any;
-  __shared__ double src_val[NT];  // this step's value of the box's first sources
+  // kind 0 sources of the box (P imposed; up to kNear): element and this step's populations at
+  // rest and in motion, stored in place of the node's own; the others go through memory
+  constexpr int kNear = 64;
+  __shared__ int near_x[kNear];
+  __shared__ R near_v[kNear][2];
+  __shared__ double near_sg[kNear], near_om[kNear], near_cs2;
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const ResItem it = ra.items[blockIdx.x];
+  // what only the prologue, the edges and thread 0 need stays in shared memory: 1024 threads have
+  // 64 registers each
+  __shared__ ResItem it;
+  __shared__ unsigned long long t0, sample0;
+  if (tid == 0) {
+    it = ra.items[blockIdx.x];
+    t0 = ra.counters[0];
+    sample0 = ra.counters[1];
+  }
+  __syncthreads();
   {
     const unsigned* from = reinterpret_cast<const unsigned*>(ra.members ? ra.members + it.member : &ra.one);
     unsigned* to = reinterpret_cast<unsigned*>(&A);
@@ -228,24 +264,18 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   __syncthreads();
 
   const int n1 = A.n1, n2 = A.n2, n3 = A.n3;
-  Face F;
-  F.ps = (int)A.ps;
-  F.s1 = A.pitch;
-  F.s3 = n1 * A.pitch;
-  R m[6];
-  unsigned walls = 0;
+  const Strides F{(int)A.ps, A.pitch, n1 * A.pitch};
   const R wt[2] = {A.w[0], A.w[1]};
-  {
-    const int wrap[3] = {(n1 - 1) * F.s1, n2 - 1, (n3 - 1) * F.s3};
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      const int b = A.bc[i], opp = i & 1 ? i : i + 2;  // the population reflected into pop i + 1
-      F.off[i] = b == LBW_BC_PERIODIC ? (i + 1) * F.ps + (i & 1 ? -wrap[i >> 1] : wrap[i >> 1])
-                 : b == LBW_BC_FREE   ? (i + 1) * F.ps : opp * F.ps;
-      m[i] = b == LBW_BC_BOUNCE ? A.damping : (b == LBW_BC_ANTIBOUNCE ? R(-1) : R(1));
-      if (m[i] != R(1)) walls |= 1u << i;
-    }
+  if (tid < 6) {
+    const int b = A.bc[tid], opp = tid & 1 ? tid : tid + 2;  // the population reflected into pop tid + 1
+    const int wrap = tid >> 1 == 0 ? (n1 - 1) * F.s1 : tid >> 1 == 1 ? n2 - 1 : (n3 - 1) * F.s3;
+    faces.off[tid] = b == LBW_BC_PERIODIC ? (tid + 1) * F.ps + (tid & 1 ? -wrap : wrap)
+                     : b == LBW_BC_FREE   ? (tid + 1) * F.ps : opp * F.ps;
+    faces.m[tid] = b == LBW_BC_BOUNCE ? A.damping : (b == LBW_BC_ANTIBOUNCE ? R(-1) : R(1));
   }
+  __syncthreads();
+  unsigned walls = 0;
+  for (int i = 0; i < 6; ++i) walls |= faces.m[i] != R(1) ? 1u << i : 0u;
   const bool p1 = A.bc[0] == LBW_BC_PERIODIC, p2 = A.bc[2] == LBW_BC_PERIODIC, p3 = A.bc[4] == LBW_BC_PERIODIC;
   auto flags_of = [&](int q1, int q2, int q3) -> unsigned {
     return (q1 == 0) | (q1 == n1 - 1) << 1 | (q2 == 0) << 2 | (q2 == n2 - 1) << 3 | (q3 == 0) << 4 |
@@ -263,24 +293,20 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   }
   __syncthreads();
 
-  // own nodes: element and packed word (flags | probe << 6 | valid << 7 | slot << 8 | row << 22)
+  // own nodes: element and packed word (flags | probe << 6 | source << 7 | slot << 8 | row << 22)
   const int nbox = it.bx * it.by * it.bz;
   int xe[K];
   unsigned pk[K];
+  const int own = tid < nbox ? (nbox - tid - 1) / nthr + 1 : 0;  // the thread's nodes
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const int id = tid + k * nthr;
-    xe[k] = 0;
-    pk[k] = 0;
-    if (id < nbox) {
-      const int ix = id % it.bx, r = id / it.bx, iy = r % it.by, iz = r / it.by;
-      const int q2 = it.x0 + ix, q1 = it.y0 + iy, q3 = it.z0 + iz;
-      xe[k] = elem_of(q1, q2, q3);
-      pk[k] = flags_of(q1, q2, q3) | 1u << 7 | (unsigned)((iz + 1) * pxy + (iy + 1) * px + ix + 1) << 8 |
-              (unsigned)r << 22;
-      for (int s = 0; s < probe_cnt; ++s)
-        if (probe_x[s] == xe[k]) pk[k] |= 1u << 6;
-    }
+    const int id = k < own ? tid + k * nthr : 0;  // past them the box's first node is loaded and dropped
+    const int ix = id % it.bx, r = id / it.bx, iy = r % it.by, iz = r / it.by;
+    const int q2 = it.x0 + ix, q1 = it.y0 + iy, q3 = it.z0 + iz;
+    xe[k] = elem_of(q1, q2, q3);
+    pk[k] = flags_of(q1, q2, q3) | (unsigned)((iz + 1) * pxy + (iy + 1) * px + ix + 1) << 8 | (unsigned)r << 22;
+    for (int s = 0; s < probe_cnt; ++s)
+      if (probe_x[s] == xe[k]) pk[k] |= 1u << 6;
   }
   for (int k = tid; k < it.by * it.bz * T_SLOTS; k += nthr) {
     const int r = k / T_SLOTS, q1 = it.y0 + r % it.by, q3 = it.z0 + r / it.by;
@@ -316,42 +342,81 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   const bool x13 = x13_any != 0;
   // along a spanned periodic axis the first and the last nodes' rho also go to the border
   const unsigned img = (sy && p1 ? 3u : 0u) | (sx && p2 ? 12u : 0u) | (sz && p3 ? 48u : 0u);
-  const int ish[3] = {it.by * px, it.bx, it.bz * pxy};
 
   S* const buf[2] = {const_cast<S*>(A.fin), A.fout};
-  unsigned* const bar = ra.bars + 32 * it.group;
-  const unsigned long long t0 = ra.counters[0], sample0 = ra.counters[1];
   const int nsrc = it.src_hi - it.src_lo;
+  const bool near = nsrc <= kNear && ra.src_kind == 0;
   auto source_entry = [&](int e) { return ra.src[ra.src_order[it.src_lo + e]]; };
   auto source_value = [&](const SourceEntry& s, unsigned long long t) { return ra.src_amp * sin(s.omega * (double)t); };
-  if (tid < nsrc) src_val[tid] = source_value(source_entry(tid), t0 + 1);
+  // near source `mine`'s populations at time t, as impose_source writes them; the last threads
+  // compute them, thread 0 waits at the barrier meanwhile
+  const int mine = nthr - 1 - tid;
+  auto set_near = [&](unsigned long long t) {
+    const double rho = near_sg[mine] * (ra.src_amp * sin(near_om[mine] * (double)t));
+    const double w0 = 1.0 - 3.0 * near_cs2, w1 = 0.5 * near_cs2;
+    double rest = w0 * rho, moving = w1 * rho;
+    if (Store<S>::kScaled) {
+      rest /= w0;
+      moving /= w1;
+    }
+    near_v[mine][0] = (R)rest;
+    near_v[mine][1] = (R)moving;
+  };
+  if (near && mine < nsrc) {
+    const SourceEntry e = source_entry(mine);
+    near_x[mine] = (int)(e.off - (A.fin - ra.base[0]));  // relative to the lattice's own buffer
+    near_sg[mine] = e.sg;
+    near_om[mine] = e.omega;
+    near_cs2 = e.cs2;
+  }
+  __syncthreads();
+  if (near && mine < nsrc) set_near(t0 + 1);
+  __syncthreads();
+  if (near && nsrc > 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      for (int e = 0; e < nsrc; ++e)
+        if (near_x[e] == xe[k]) pk[k] |= 1u << 7;
+  }
   bool ok = bad == 0;
   if (ok && ra.stall && *ra.stall) {  // injected timeout: a bounded wait that nothing completes
     if (tid == 0) {
       int n = 0;
-      while (ld_acquire(bar) != 0xffffffffu && ++n < kStallTries) {}
+      while (ld_acquire(ra.bars + 32 * it.group) != 0xffffffffu && ++n < kStallTries) {}
       ra.counters[3] = 1;
     }
     ok = false;
   }
 
+  // FP32 values land in the registers they stay in, so all of a thread's loads go out first (204,800
+  // nodes 5.9 -> 4.9 us per step); 16-bit values need a conversion each and FP64 twice the
+  // registers, and node by node is faster (240,000 nodes: FP16 7.1 -> 5.5 us)
+  constexpr bool kTogether = sizeof(S) == 4;
   int cur = ra.cur;
   for (int s = 0; ok && s < ra.steps; ++s) {
     const S* const f = buf[cur];
     S* const g = buf[1 - cur];
     R v[K][7];
 #pragma unroll
-    for (int k = 0; k < K; ++k)
-      if (pk[k]) pull_node<S, TILE>(f, xe[k], pk[k], walls, F, m, wt, v[k]);
+    for (int k = 0; k < K; ++k) {
+      if constexpr (kTogether) {
+        load_node(f, xe[k], pk[k], F, faces, v[k]);
+      } else if (k < own) {
+        load_node(f, xe[k], pk[k], F, faces, v[k]);
+        finish_node<S, TILE>(pk[k], walls, faces, wt, v[k]);
+      }
+    }
     for (int h = nthr - 1 - tid; h < nhalo; h += nthr) {  // threads without a last node first
       const int2 e = halo[h];
       R u[7];
-      pull_node<S, TILE>(f, e.x, (unsigned)e.y, walls, F, m, wt, u);
+      load_node(f, e.x, (unsigned)e.y, F, faces, u);
+      finish_node<S, TILE>((unsigned)e.y, walls, faces, wt, u);
       rho[(unsigned)e.y >> 8] = rho_of<S, TILE>(u, wt);
     }
 #pragma unroll
     for (int k = 0; k < K; ++k)
-      if (pk[k]) {
+      if (k < own) {
+        if constexpr (kTogether) finish_node<S, TILE>(pk[k], walls, faces, wt, v[k]);
         const int slot = (pk[k] >> 8) & (kResMaxSlots - 1);
         const R r = rho_of<S, TILE>(v[k], wt);
         rho[slot] = r;
@@ -359,15 +424,16 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
         if (edge) {
 #pragma unroll
           for (int a = 0; a < 3; ++a) {
-            if (edge & (1u << (2 * a))) rho[slot + ish[a]] = r;
-            if (edge & (2u << (2 * a))) rho[slot - ish[a]] = r;
+            const int shift = a == 0 ? it.by * px : a == 1 ? it.bx : it.bz * pxy;
+            if (edge & (1u << (2 * a))) rho[slot + shift] = r;
+            if (edge & (2u << (2 * a))) rho[slot - shift] = r;
           }
         }
       }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < K; ++k)
-      if (pk[k]) {
+      if (k < own) {
         const int slot = (pk[k] >> 8) & (kResMaxSlots - 1);
         const R* T = tab + (pk[k] >> 22) * T_SLOTS;
         R c[T_SLOTS];
@@ -390,11 +456,16 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
         collide_node<S, TILE>(c, x13, A.cs2, A.two_w0, r, rho[slot + px], rho[slot - px], rr, rl, rho[slot + pxy],
                               rho[slot - pxy], v[k]);
 #pragma unroll
-        for (int i = 0; i < 7; ++i) {
-          R o = v[k][i];
-          if (Store<S>::kScaled && !TILE) o *= i == 0 ? A.inv_w[0] : A.inv_w[1];
-          Store<S>::st(g + (xe[k] + i * F.ps), o);
+        for (int i = 0; i < 7; ++i)
+          if (Store<S>::kScaled && !TILE) v[k][i] *= i == 0 ? A.inv_w[0] : A.inv_w[1];
+        if (pk[k] & 128u) {
+          int e = 0;
+          while (near_x[e] != xe[k]) ++e;
+#pragma unroll
+          for (int i = 0; i < 7; ++i) v[k][i] = near_v[e][i > 0];
         }
+#pragma unroll
+        for (int i = 0; i < 7; ++i) Store<S>::st(g + (xe[k] + i * F.ps), v[k][i]);
         if (pk[k] & 64u) {
           const unsigned long long t = sample0 + s;
           if (t < (unsigned long long)A.cap)
@@ -402,22 +473,23 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
               if (probe_x[q] == xe[k]) A.series[(long long)probe_id[q] * A.cap + t] = (double)r * (double)c[T_INVSG];
         }
       }
-    if (nsrc > 0) {  // harmonic sources on the state just written (as source_kernel does)
+    if (nsrc > 0 && !near) {  // harmonic sources on the state just written (as source_kernel does)
       __syncthreads();
       for (int e = tid; e < nsrc; e += nthr) {
         const SourceEntry se = source_entry(e);
-        impose_source(ra.base[1 - cur], se, ra.src_kind, e < nthr ? src_val[e] : source_value(se, t0 + s + 1));
+        impose_source(ra.base[1 - cur], se, ra.src_kind, source_value(se, t0 + s + 1));
       }
     }
     cur ^= 1;
     if (s + 1 == ra.steps) break;
     __syncthreads();
-    if (tid == 0) red_release(bar);
-    // the next step's source value, while the other CTAs arrive
-    if (tid < nsrc) src_val[tid] = source_value(source_entry(tid), t0 + s + 2);
+    if (tid == 0) red_release(ra.bars + 32 * it.group);
+    // the next step's source values, while the other CTAs arrive
+    if (near && mine < nsrc) set_near(t0 + s + 2);
     if (tid == 0) {
       const unsigned want = (unsigned)(s + 1) * (unsigned)it.group_size;
       long long n = 0;
+      const unsigned* const bar = ra.bars + 32 * it.group;
       while (ld_acquire(bar) < want) {
         if (++n > kResWaitLimit) {
           ra.counters[3] = 1;
@@ -445,19 +517,32 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
 }
 
 
-// Nodes per thread and threads of a box of `own` nodes: (512, 1), (512, 2), (1024, 2) and, for
-// 16- and 32-bit storage (64 registers hold four nodes' populations), (1024, 4).
-int nodes_per_thread(int own) { return own <= 512 ? 1 : own <= 2048 ? 2 : 4; }
-int max_threads(int own) { return own <= 1024 ? 512 : 1024; }
+// Threads and nodes per thread of a box of `own` nodes.
+struct ResShape {
+  int threads, k;
+};
+constexpr ResShape kResShapes[] = {{512, 1}, {512, 2}, {768, 2}, {768, 3}, {768, 4}, {1024, 4}};
+
+int shape_of(int own) {
+  int i = 0;
+  while (kResShapes[i].threads * kResShapes[i].k < own) ++i;
+  return i;
+}
 
 template <typename S, bool TILE, typename F>
 auto with_shape(int own, F&& f) {
-  if (own <= 512) return f(resident_kernel<S, TILE, 512, 1>);
-  if (own <= 1024) return f(resident_kernel<S, TILE, 512, 2>);
-  if constexpr (sizeof(S) < 8) {
-    if (own > 2048) return f(resident_kernel<S, TILE, 1024, 4>);
+  switch (shape_of(own)) {
+    case 0: return f(resident_kernel<S, TILE, 512, 1>);
+    case 1: return f(resident_kernel<S, TILE, 512, 2>);
+    case 2: return f(resident_kernel<S, TILE, 768, 2>);
+    case 3: return f(resident_kernel<S, TILE, 768, 3>);
   }
-  return f(resident_kernel<S, TILE, 1024, 2>);
+  if constexpr (sizeof(S) < 8) {
+    if (shape_of(own) == 4) return f(resident_kernel<S, TILE, 768, 4>);
+    return f(resident_kernel<S, TILE, 1024, 4>);
+  } else {
+    return f(resident_kernel<S, TILE, 768, 3>);
+  }
 }
 
 // The kernel for (storage, arithmetic form, nodes per box): f(kernel).
@@ -624,9 +709,9 @@ lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool ti
     }
     L.count = (int)items.size() - L.first;
     if (L.count > sms) return LBW_OK;
-    const int k = nodes_per_thread(own);
+    const ResShape shape = kResShapes[shape_of(own)];
     L.own = own;
-    L.threads = std::min(max_threads(own), std::max(64, round32((own + k - 1) / k + (k == 1 ? halo : 0))));
+    L.threads = std::min(shape.threads, std::max(64, round32((own + shape.k - 1) / shape.k + (shape.k == 1 ? halo : 0))));
     int per = 0;
     const cudaError_t e = with_prec(prec, [&](auto tag) {
       return with_kernel<decltype(tag)>(tile, own, [&](auto kern) {
