@@ -374,7 +374,7 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
     return cleanup(fail(LBW_EINVAL, "geom_mode ANALYTIC needs the tile kernel: q2 extent a multiple of "
                                     "the tile width (64, or 128 for 16-bit storage) and non-periodic q1"));
   // Lattices that fit run many steps per launch: faster up to all the SMs hold (us per step,
-  // before -> now: FP64 16k nodes 10.6 -> 3.2, 120k 24.8 -> 10.9; FP32 16k 7.1 -> 2.2, 500k 20.5
+  // before -> now: FP64 16k nodes 10.6 -> 3.2, 120k 24.8 -> 10.2; FP32 16k 7.1 -> 2.2, 500k 20.5
   // -> 10.9), except 16-bit storage on the tile kernel, which is ahead from about 300k nodes
   // (205k: 10.1 -> 4.7, 410k: 8.4 against 8.5).
   const Grid* self = g;

@@ -18,6 +18,7 @@
 #include <functional>
 #include <sstream>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lbw_internal.h"
@@ -363,7 +364,10 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
         } else {
 #pragma unroll
           for (int k = 0; k < NPT; ++k) {
-            f[1][k] *= m1; f[2][k] *= m2; f[5][k] *= m5; f[6][k] *= m6;
+            if (m1 != R(1)) f[1][k] *= m1;
+            if (m2 != R(1)) f[2][k] *= m2;
+            if (m5 != R(1)) f[5][k] *= m5;
+            if (m6 != R(1)) f[6][k] *= m6;
             const R sum = ((f[0][k] + f[1][k]) + (f[2][k] + f[3][k])) + ((f[4][k] + f[5][k]) + f[6][k]);
             rr[k] = ghost ? R(0) : sum;
           }
@@ -450,26 +454,19 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
             fc[i][1] = o[i].y;
           }
         } else {
+          auto nodes = [&](auto x13) {
 #pragma unroll
-          for (int k = 0; k < NPT; ++k) {
-            const R rho = rc[k];
-            const R D1 = c[T_A1P] * ru[k] - c[T_A1M] * rd[k] + c[T_C13P] * rn[k] - c[T_C13M] * rp[k] +
-                         c[T_S1] * rho;
-            const R D3 = c[T_B13P] * ru[k] - c[T_B13M] * rd[k] + c[T_C33P] * rn[k] - c[T_C33M] * rp[k] +
-                         c[T_S3] * rho;
-            const R D2 = c[T_H22] * (rrt[k] - rl[k]);
-            const R j1 = (fc[1][k] - fc[2][k]) + R(0.5) * (c[T_MG1] * rho - D1);
-            const R j2 = (fc[3][k] - fc[4][k]) - R(0.5) * D2;
-            const R j3 = (fc[5][k] - fc[6][k]) + R(0.5) * (c[T_MG3] * rho - D3);
-            const R e = A.cs2 * rho;
-            fc[0][k] = A.two_w0 * rho - fc[0][k];
-            fc[1][k] = e + j1 - fc[1][k];
-            fc[2][k] = e - j1 - fc[2][k];
-            fc[3][k] = e + j2 - fc[3][k];
-            fc[4][k] = e - j2 - fc[4][k];
-            fc[5][k] = e + j3 - fc[5][k];
-            fc[6][k] = e - j3 - fc[6][k];
-          }
+            for (int k = 0; k < NPT; ++k) {
+              double v[7];
+#pragma unroll
+              for (int i = 0; i < 7; ++i) v[i] = fc[i][k];
+              collide_f64<decltype(x13)::value>(c, A.cs2, A.two_w0, rc[k], ru[k], rd[k], rn[k], rp[k], rrt[k] - rl[k], v);
+#pragma unroll
+              for (int i = 0; i < 7; ++i) fc[i][k] = v[i];
+            }
+          };
+          if (A.x13) nodes(std::true_type{});
+          else nodes(std::false_type{});
         }
         S* dst = dst_z0 + (long long)(zc - z0) * row_stride;
 #pragma unroll
@@ -807,7 +804,10 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
         } else {
 #pragma unroll
           for (int k = 0; k < NPT; ++k) {
-            f[1][k] *= m1; f[2][k] *= m2; f[5][k] *= m5; f[6][k] *= m6;
+            if (m1 != R(1)) f[1][k] *= m1;
+            if (m2 != R(1)) f[2][k] *= m2;
+            if (m5 != R(1)) f[5][k] *= m5;
+            if (m6 != R(1)) f[6][k] *= m6;
             const R sum = ((f[0][k] + f[1][k]) + (f[2][k] + f[3][k])) + ((f[4][k] + f[5][k]) + f[6][k]);
             rr[k] = ghost ? R(0) : sum;
           }
@@ -871,26 +871,19 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
             fc[i][1] = o[i].y;
           }
         } else {
+          auto nodes = [&](auto x13) {
 #pragma unroll
-          for (int k = 0; k < NPT; ++k) {
-            const R rho = rc[k];
-            const R D1 = c[T_A1P] * ru[k] - c[T_A1M] * rd[k] + c[T_C13P] * rn[k] - c[T_C13M] * rp[k] +
-                         c[T_S1] * rho;
-            const R D3 = c[T_B13P] * ru[k] - c[T_B13M] * rd[k] + c[T_C33P] * rn[k] - c[T_C33M] * rp[k] +
-                         c[T_S3] * rho;
-            const R D2 = c[T_H22] * (rrt[k] - rl[k]);
-            const R j1 = (fc[1][k] - fc[2][k]) + R(0.5) * (c[T_MG1] * rho - D1);
-            const R j2 = (fc[3][k] - fc[4][k]) - R(0.5) * D2;
-            const R j3 = (fc[5][k] - fc[6][k]) + R(0.5) * (c[T_MG3] * rho - D3);
-            const R e = A.cs2 * rho;
-            fc[0][k] = A.two_w0 * rho - fc[0][k];
-            fc[1][k] = e + j1 - fc[1][k];
-            fc[2][k] = e - j1 - fc[2][k];
-            fc[3][k] = e + j2 - fc[3][k];
-            fc[4][k] = e - j2 - fc[4][k];
-            fc[5][k] = e + j3 - fc[5][k];
-            fc[6][k] = e - j3 - fc[6][k];
-          }
+            for (int k = 0; k < NPT; ++k) {
+              double v[7];
+#pragma unroll
+              for (int i = 0; i < 7; ++i) v[i] = fc[i][k];
+              collide_f64<decltype(x13)::value>(c, A.cs2, A.two_w0, rc[k], ru[k], rd[k], rn[k], rp[k], rrt[k] - rl[k], v);
+#pragma unroll
+              for (int i = 0; i < 7; ++i) fc[i][k] = v[i];
+            }
+          };
+          if (A.x13) nodes(std::true_type{});
+          else nodes(std::false_type{});
         }
         S* dst = dst_z0 + (long long)(zc - z0) * row_stride;
 #pragma unroll

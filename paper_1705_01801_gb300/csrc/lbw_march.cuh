@@ -167,6 +167,7 @@ struct StepArgs {
   // ghost columns that mirror the periodic wrap)
   int pitch, col0;
   long long ps;
+  int x13;          // the metric couples q1 and q3 (otherwise those coefficients are zero)
   GeomArgs<R> geo;  // closed-form geometry (used by the tile kernel in the analytic mode)
 };
 
@@ -204,6 +205,7 @@ StepArgs<S> step_args(const Grid& lattice, int src) {
   a.pitch = g->pitch ? g->pitch : g->d.n[1];
   a.col0 = g->col0;
   a.ps = pop_stride(g);
+  a.x13 = g->d.kind == LBW_TRUMPET;
   a.geo.kind = g->d.kind;
   a.geo.profile = g->d.horn_profile;
   a.geo.x0r = (R)g->d.x0[0];
@@ -248,6 +250,29 @@ __device__ __forceinline__ void impose_source(S* base, const SourceEntry& s, int
     Store<S>::st(f + (long long)i * s.ps, r);
     if (s.ghost != 0) Store<S>::st(f + (long long)i * s.ps + s.ghost, r);
   }
+}
+
+// FP64 collision of one node: v holds its pulled populations and receives the post-collision ones;
+// dr2 = rho(q2 + 1) - rho(q2 - 1), X13: the metric couples q1 and q3.  With h^a half the forcing term, j^a = f_a+ - f_a- + h^a, so
+// f*_a+ = e + j^a - f_a+ = (e + h^a) - f_a- and f*_a- = (e - h^a) - f_a+: with the density sum 30
+// to 34 FP64 operations a node where forming j^a takes 46, and FP64 (2 a cycle and SM) is what bounds
+// the tile kernels in this storage (torus 96 x 512 x 128
+// 606 -> 536 us per step, cylinder 200 x 250 x 256 1233 -> 1087, trumpet 256 x 256 x 512 3122 -> 2970;
+// the choice on x13 stands outside the loop over a lane's nodes, whose chains then overlap).
+template <bool X13>
+__device__ __forceinline__ void collide_f64(const double (&c)[T_SLOTS], double cs2, double two_w0, double rho,
+                                            double ru, double rd, double rn, double rp, double dr2, double (&v)[7]) {
+  double n1 = (c[T_MG1] - c[T_S1]) * rho - c[T_A1P] * ru + c[T_A1M] * rd;
+  double n3 = (c[T_MG3] - c[T_S3]) * rho - c[T_C33P] * rn + c[T_C33M] * rp;
+  if constexpr (X13) {
+    n1 = n1 - c[T_C13P] * rn + c[T_C13M] * rp;
+    n3 = n3 - c[T_B13P] * ru + c[T_B13M] * rd;
+  }
+  const double n2 = -c[T_H22] * dr2, e = cs2 * rho;
+  const double a1 = fma(0.5, n1, e) - v[2], a2 = fma(-0.5, n1, e) - v[1], a3 = fma(0.5, n2, e) - v[4],
+               a4 = fma(-0.5, n2, e) - v[3], a5 = fma(0.5, n3, e) - v[6], a6 = fma(-0.5, n3, e) - v[5];
+  v[0] = two_w0 * rho - v[0];
+  v[1] = a1; v[2] = a2; v[3] = a3; v[4] = a4; v[5] = a5; v[6] = a6;
 }
 
 __device__ __forceinline__ long long node(int q1, int q2, int q3, int n1, int n2) {

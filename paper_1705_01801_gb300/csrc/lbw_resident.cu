@@ -10,7 +10,7 @@
 // other CTAs own), puts their post-stream rho into shared memory, and after one __syncthreads
 // collides its nodes (the populations stay in registers) and stores them to the other buffer.
 // Measured per step, a launch per step -> here: disk 10.6 -> 3.2 us, the paper's 20 x 200 x 30
-// torus in FP64 with a ring source 29.3 -> 11.3 us, 41 pipes of 10,000 FP32 nodes with sources
+// torus in FP64 with a ring source 29.3 -> 10.5 us, 41 pipes of 10,000 FP32 nodes with sources
 // 176 -> 9.5 us (38 + 3 of them in two turns).  What bounds it: 2.0 us of barrier and load
 // latency for the smallest lattices, the FP64 pipe for FP64, load latency beyond a few hundred
 // nodes per CTA (25 % of the issue slots busy).
@@ -129,15 +129,15 @@ __device__ __forceinline__ typename Store<S>::R rho_of(const typename Store<S>::
 }
 
 // Collision of one node: v holds its pulled populations and receives the post-collision ones;
-// `x13` says whether the metric couples q1 and q3 (otherwise those coefficients are zero).
+// X13: the metric couples q1 and q3 (FP64; otherwise those coefficients are zero).
 // 64-bit storage: with h^a half the forcing term, j^a = f_a+ - f_a- + h^a, so
 // f*_a+ = e + j^a - f_a+ = (e + h^a) - f_a- and f*_a- = (e - h^a) - f_a+: 28 to 32 operations a
 // node where forming j^a takes 46, which is what FP64 (2 a cycle and SM) is bound by
-// (120k nodes: 14.0 -> 11.7 us per step).  The rows then hold half the coefficients, signed,
+// (120k nodes: 14.0 -> 10.2 us per step).  The rows then hold half the coefficients, signed,
 // and the node's own in one (coef_row).  32- and 16-bit storage repeats the operations of the
 // kernels that step once per launch, so the results do not depend on which of them runs.
-template <typename S, bool TILE>
-__device__ __forceinline__ void collide_node(const typename Store<S>::R (&c)[T_SLOTS], bool x13,
+template <typename S, bool TILE, bool X13>
+__device__ __forceinline__ void collide_node(const typename Store<S>::R (&c)[T_SLOTS],
                                              typename Store<S>::R cs2, typename Store<S>::R two_w0,
                                              typename Store<S>::R rho, typename Store<S>::R ru,
                                              typename Store<S>::R rd, typename Store<S>::R rr,
@@ -147,7 +147,7 @@ __device__ __forceinline__ void collide_node(const typename Store<S>::R (&c)[T_S
   if constexpr (sizeof(R) == 8) {
     R h1 = c[T_MG1] * rho + c[T_A1P] * ru + c[T_A1M] * rd;
     R h3 = c[T_MG3] * rho + c[T_C33P] * rn + c[T_C33M] * rp;
-    if (x13) {
+    if constexpr (X13) {
       h1 = h1 + c[T_C13P] * rn + c[T_C13M] * rp;
       h3 = h3 + c[T_B13P] * ru + c[T_B13M] * rd;
     }
@@ -222,14 +222,14 @@ __device__ __forceinline__ void red_release(unsigned* p) {
 
 // Shared memory: rho of the box with a one-node border ((bx + 2) (by + 2) (bz + 2)), the
 // coefficient rows of the box (by bz), and per halo node its element and packed word.
-template <typename S, bool TILE, int NT, int K>
+template <typename S, bool TILE, int NT, int K, bool X13>
 __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   using R = typename Store<S>::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) StepArgs<S> A;
   __shared__ Faces<R> faces;
   __shared__ int probe_x[kMaxProbes], probe_id[kMaxProbes];
-  __shared__ int probe_cnt, halo_cnt, bad, x13_any;
+  __shared__ int probe_cnt, halo_cnt, bad;
   // kind 0 sources of the box (P imposed; up to kNear): element and this step's populations at
   // rest and in motion, stored in place of the node's own; the others go through memory
   constexpr int kNear = 64;
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
     for (int k = tid; k < (int)(sizeof(StepArgs<S>) / 4); k += nthr) to[k] = from[k];
   }
   if (tid == 0) {
-    probe_cnt = halo_cnt = x13_any = 0;
+    probe_cnt = halo_cnt = 0;
     bad = ra.counters[3] != 0ull;  // an earlier step timed out: nothing to advance
   }
   const int px = it.bx + 2, pxy = px * (it.by + 2), nslot = pxy * (it.bz + 2);
@@ -310,9 +310,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   }
   for (int k = tid; k < it.by * it.bz * T_SLOTS; k += nthr) {
     const int r = k / T_SLOTS, q1 = it.y0 + r % it.by, q3 = it.z0 + r / it.by;
-    const R v = coef_row<S>(A.tab + ((long long)q3 * n1 + q1) * T_SLOTS, k % T_SLOTS);
-    tab[k] = v;
-    if (k % T_SLOTS >= T_B13P && k % T_SLOTS <= T_C13M && v != R(0)) x13_any = 1;
+    tab[k] = coef_row<S>(A.tab + ((long long)q3 * n1 + q1) * T_SLOTS, k % T_SLOTS);
   }
   // halo nodes: the box's six faces, except along an axis that the box spans (its periodic wrap
   // is served by the border copies below) and beyond walls
@@ -339,7 +337,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   }
   __syncthreads();
   const int nhalo = halo_cnt, npr = probe_cnt;
-  const bool x13 = x13_any != 0;
+
   // along a spanned periodic axis the first and the last nodes' rho also go to the border
   const unsigned img = (sy && p1 ? 3u : 0u) | (sx && p2 ? 12u : 0u) | (sz && p3 ? 48u : 0u);
 
@@ -453,7 +451,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
           if (pk[k] & 4u) rl = A.s2lo * r;
           if (pk[k] & 8u) rr = A.s2hi * r;
         }
-        collide_node<S, TILE>(c, x13, A.cs2, A.two_w0, r, rho[slot + px], rho[slot - px], rr, rl, rho[slot + pxy],
+        collide_node<S, TILE, X13>(c, A.cs2, A.two_w0, r, rho[slot + px], rho[slot - px], rr, rl, rho[slot + pxy],
                               rho[slot - pxy], v[k]);
 #pragma unroll
         for (int i = 0; i < 7; ++i)
@@ -529,29 +527,31 @@ int shape_of(int own) {
   return i;
 }
 
-template <typename S, bool TILE, typename F>
+template <typename S, bool TILE, bool X13, typename F>
 auto with_shape(int own, F&& f) {
   switch (shape_of(own)) {
-    case 0: return f(resident_kernel<S, TILE, 512, 1>);
-    case 1: return f(resident_kernel<S, TILE, 512, 2>);
-    case 2: return f(resident_kernel<S, TILE, 768, 2>);
-    case 3: return f(resident_kernel<S, TILE, 768, 3>);
+    case 0: return f(resident_kernel<S, TILE, 512, 1, X13>);
+    case 1: return f(resident_kernel<S, TILE, 512, 2, X13>);
+    case 2: return f(resident_kernel<S, TILE, 768, 2, X13>);
+    case 3: return f(resident_kernel<S, TILE, 768, 3, X13>);
   }
   if constexpr (sizeof(S) < 8) {
-    if (shape_of(own) == 4) return f(resident_kernel<S, TILE, 768, 4>);
-    return f(resident_kernel<S, TILE, 1024, 4>);
+    if (shape_of(own) == 4) return f(resident_kernel<S, TILE, 768, 4, X13>);
+    return f(resident_kernel<S, TILE, 1024, 4, X13>);
   } else {
-    return f(resident_kernel<S, TILE, 768, 3>);
+    return f(resident_kernel<S, TILE, 768, 3, X13>);
   }
 }
 
-// The kernel for (storage, arithmetic form, nodes per box): f(kernel).
+// The kernel for (storage, arithmetic form, coupled axes, nodes per box): f(kernel).
 template <typename S, typename F>
-auto with_kernel(bool tile, int own, F&& f) {
-  if constexpr (sizeof(S) < 8) {
-    if (!tile) return with_shape<S, false>(own, f);
+auto with_kernel(bool tile, bool x13, int own, F&& f) {
+  if constexpr (sizeof(S) == 8) {
+    if (x13) return with_shape<S, true, true>(own, f);
+  } else {
+    if (!tile) return with_shape<S, false, false>(own, f);
   }
-  return with_shape<S, true>(own, f);
+  return with_shape<S, true, false>(own, f);
 }
 
 template <typename F>
@@ -646,7 +646,7 @@ cudaError_t launch_t(const Resident* r, const Resident::Launch& L, const StepArg
   cfg.stream = st.stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return with_kernel<S>(r->tile, L.own, [&](auto kern) { return cudaLaunchKernelEx(&cfg, kern, ra); });
+  return with_kernel<S>(r->tile, r->x13, L.own, [&](auto kern) { return cudaLaunchKernelEx(&cfg, kern, ra); });
 }
 
 }  // namespace
@@ -669,6 +669,7 @@ lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool ti
   Resident r;
   r.prec = prec;
   r.tile = tile;
+  for (int m = 0; m < n; ++m) r.x13 |= lattices[m]->d.kind == LBW_TRUMPET;
   for (int first = 0; first < n;) {
     // the lattices of one launch: as many as the SMs hold at the most nodes per thread
     long long nodes = 0;
@@ -714,7 +715,7 @@ lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool ti
     L.threads = std::min(shape.threads, std::max(64, round32((own + shape.k - 1) / shape.k + (shape.k == 1 ? halo : 0))));
     int per = 0;
     const cudaError_t e = with_prec(prec, [&](auto tag) {
-      return with_kernel<decltype(tag)>(tile, own, [&](auto kern) {
+      return with_kernel<decltype(tag)>(tile, r.x13, own, [&](auto kern) {
         cudaError_t f = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (f == cudaSuccess) f = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, L.threads, L.smem);
         return f;

@@ -25,6 +25,7 @@ struct Resident {
   std::vector<ResItem> host_items;
   int prec = 0;
   bool tile = false;             // operations of the tile kernels (see lbw_resident.cu)
+  bool x13 = false;              // some lattice's metric couples q1 and q3
   ResItem* items = nullptr;
   unsigned* bars = nullptr;
   int* src_order = nullptr;
