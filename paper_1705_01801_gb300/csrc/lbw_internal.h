@@ -28,6 +28,15 @@ enum TableSlot {
 
 constexpr int kMaxProbes = 64;
 
+// Blocks of the tile kernel on a single lattice.  An item is one of `tiles` (nx along q2) times
+// one of `segs` equal q3 segments; consecutive items are neighbouring tiles of the same segment,
+// so the blocks in flight share their halos through L2.  The first `full` items, as many as fill
+// the SMs a whole number of times, are a block each; of the others every one is cut into `split`
+// pieces along q3, so they too fill the SMs once.
+struct TileCuts {
+  unsigned tiles, nx, segs, full, split;
+};
+
 }  // namespace lbw
 struct lbw_batch;
 namespace lbw {
@@ -55,7 +64,8 @@ struct Grid {
   bool initialised = false;
   // launch shape of the step kernel
   int bx = 0, by = 0, lz = 0;
-  int tma_by = 0;          // 0: register-pipelined kernel; 4 or 7: TMA tile kernel rows
+  TileCuts cuts = {};     // the tile kernel's blocks
+  int tma_by = 0;          // 0: register-pipelined kernel; 4, 5 or 7: TMA tile kernel rows
   int tma_npt = 2;         // TMA tile kernel: nodes per lane (tile width 32 x tma_npt)
   // padded storage (ensembles on the tile kernel): row length and first data column in
   // elements; pitch 0 means dense rows of n2 values

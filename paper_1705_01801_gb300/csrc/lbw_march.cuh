@@ -151,6 +151,7 @@ struct StepArgs {
   S* __restrict__ fout;
   const R* __restrict__ tab;
   int n1, n2, n3, lz;
+  TileCuts cuts;  // tile kernel
   long long nn;
   int bc[6];
   R damping, cs2, two_w0;
@@ -182,6 +183,7 @@ StepArgs<S> step_args(const Grid& lattice, int src) {
   a.tab = reinterpret_cast<const R*>(g->table);
   a.n1 = g->d.n[0]; a.n2 = g->d.n[1]; a.n3 = g->d.n[2];
   a.lz = g->lz;
+  a.cuts = g->cuts;
   a.nn = g->nn;
   for (int k = 0; k < 6; ++k) a.bc[k] = g->d.bc[k];
   a.damping = (R)g->d.damping;

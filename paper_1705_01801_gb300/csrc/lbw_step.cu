@@ -108,7 +108,7 @@ struct TmaLayout {
 // The slot's full mbarrier completes on the bytes, and a slot is refilled only after every
 // consumer warp has released it (empty mbarrier), so the producer runs up to NB - 2 (16-bit:
 // NB - 3) planes ahead.  Per plane u the consumers read step B's shared inputs of plane
-// u - 1, pull the populations of plane u and write its rho into one of three rotating rho
+// u - 1, pull the populations of plane u and write its rho into one of two alternating rho
 // planes (step A), collide plane u - 1 (step B, rows of the tile only), release the slot of
 // plane u - 1 and synchronise among themselves (named barrier).  Face rules are reads of other staged values (bounce-back /
 // anti-bounce-back: the node's own opposite population; free: the node's own population),
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
   constexpr int C0 = NPT, PW = BX + 2 * NPT;
   constexpr int PS = ROWS * PW;
   constexpr int TABB = ((BY * T_SLOTS * RS) + 127) / 128 * 128;
-  constexpr int RHOB = ((3 * PS * RS) + 127) / 128 * 128;  // three rho planes
+  constexpr int RHOB = ((2 * PS * RS) + 127) / 128 * 128;  // two rho planes
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int probe_list[kMaxProbes];
   __shared__ int probe_cnt;
@@ -155,14 +155,22 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int lane = threadIdx.x, w = threadIdx.y, tid = w * 32 + lane;
-  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY, z0 = blockIdx.z * a.lz;
-  const int z1 = min(z0 + a.lz, a.n3);
+  // block -> tile and planes (see TileCuts): segment-major, the blocks past `full` being pieces
+  // of the remaining (tile, segment) items
+  const TileCuts& tc = a.cuts;
+  const unsigned bid = blockIdx.x, piece = bid < tc.full ? 0u : (bid - tc.full) % tc.split;
+  const unsigned item = bid < tc.full ? bid : tc.full + (bid - tc.full) / tc.split;
+  const unsigned seg = item / tc.tiles, tile = item % tc.tiles;
+  const unsigned za = seg * (unsigned)a.n3 / tc.segs, zl = (seg + 1) * (unsigned)a.n3 / tc.segs - za;
+  const unsigned pieces = bid < tc.full ? 1u : tc.split;
+  const int x0 = (int)(tile % tc.nx) * BX, y0 = (int)(tile / tc.nx) * BY;
+  const int z0 = (int)(za + piece * zl / pieces), z1 = (int)(za + (piece + 1) * zl / pieces);
   const bool p2 = a.bc[2] == LBW_BC_PERIODIC, p3 = a.bc[4] == LBW_BC_PERIODIC;
   // 16-bit: the tile's halo column on this side wraps around the periodic q2 axis
   const bool wrapL = p2 && x0 == 0, wrapR = p2 && x0 + BX == a.n2;
 
   // byte offsets from smem_raw (TMA destinations want 128-byte alignment): barriers, NB
-  // slots, three rho planes, NB coefficient blocks
+  // slots, two rho planes, NB coefficient blocks
   const unsigned sbase = smem_u32(smem_raw);
   const unsigned OFF = (128u - (sbase & 127u)) & 127u;
   const unsigned SL = OFF + 128, RHO = SL + NB * SLOTB, TAB = RHO + RHOB, MSC = TAB + NB * TABB;
@@ -433,6 +441,8 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
     const R m5_face = a.bc[4] == LBW_BC_FREE ? sc1 : sc1 * wall(a.bc[4]);
     const R m6_face = a.bc[5] == LBW_BC_FREE ? sc1 : sc1 * wall(a.bc[5]);
 
+    const bool wallrow = m1 != R(1) || m2 != R(1);
+
     // halo column node of a halo warp: warp 0 lane l -> (y0 + l, x0 - 1), warp BY+1 ->
     // (y0 + l, x0 + BX), lanes l < BY; the other lanes mirror lane BY - 1 and store nothing
     const bool hwarp = !interior;
@@ -552,19 +562,20 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
       const bool ghost = zghost || !rowin;
       if constexpr (sizeof(R) == 4) {
         const float2 W0S = bc2(a.w[0]), W1S = bc2(a.w[1]);
+        if (wallrow || zlo || zhi) {  // one branch for the warp; every factor is 1 elsewhere
+#pragma unroll
+          for (int k = 0; k < NPT; ++k) {  // rounded: never contracted with the sums below
+            f[1][k] = __fmul_rn(m1, f[1][k]);
+            f[2][k] = __fmul_rn(m2, f[2][k]);
+            f[5][k] = __fmul_rn(m5, f[5][k]);
+            f[6][k] = __fmul_rn(m6, f[6][k]);
+          }
+        }
 #pragma unroll
         for (int k = 0; k < NPT; k += 2) {
           float2 F[7];
 #pragma unroll
           for (int i = 0; i < 7; ++i) F[i] = f2(f[i][k], f[i][k + 1]);
-          F[1] = mul2(bc2(m1), F[1]);
-          F[2] = mul2(bc2(m2), F[2]);
-          F[5] = mul2(bc2(m5), F[5]);
-          F[6] = mul2(bc2(m6), F[6]);
-          f[1][k] = F[1].x; f[1][k + 1] = F[1].y;
-          f[2][k] = F[2].x; f[2][k + 1] = F[2].y;
-          f[5][k] = F[5].x; f[5][k + 1] = F[5].y;
-          f[6][k] = F[6].x; f[6][k + 1] = F[6].y;
           float2 sum;
           if constexpr (SC)
             sum = fma2(W0S, F[0], mul2(W1S, add2(add2(add2(F[1], F[2]), add2(F[3], F[4])), add2(F[5], F[6]))));
@@ -740,14 +751,13 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
       if (lane == 0) mbar_arrive(empty_at(1));  // nor is plane z0 - 1
       ok = !named_sync_or(1, NCW * 32, !ok || abort_flag);
       // slots of raw planes z, z + 1, z + 2 (plane z0 - 2 sits in slot 0) and the fill count of
-      // the awaited slot (plane z + 1's or z + 2's), advanced plane by plane.  rho planes rotate
-      // through three buffers: a warp writing plane z + 1's buffer has passed the barrier that
-      // follows every read of that buffer (plane z - 2); the rows of plane z0 - 1 in buffer 2
-      // are never written or read.
+      // the awaited slot (plane z + 1's or z + 2's), advanced plane by plane.  rho planes alternate
+      // between two buffers: a warp writing plane z + 1's buffer has passed the barrier that
+      // follows every read of that buffer (plane z - 1, read into registers before A(z))
       int sz = 2, s1 = 3, s2 = 4, uw = 0, rbz = 0, rb1 = 1;
       auto advance = [&]() {
         rbz = rb1;
-        rb1 = rb1 == 2 ? 0 : rb1 + 1;
+        rb1 ^= 1;
         sz = s1;
         s1 = s2;
         s2 = s2 == NB - 1 ? 0 : s2 + 1;
@@ -756,8 +766,8 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
       // iteration z: raw plane z + 1 (RG) or z + 2 in, B(z)'s shared-memory reads, A(z + 1),
       // B(z), release raw plane z, barrier.  B(z) needs rho of plane z + 1 only at the warp's
       // own nodes (its own A(z + 1)) and rho plane z, which every warp wrote before the previous
-      // iteration's barrier; A(z + 1) writes rho plane z + 1, whose buffer was last read by
-      // B(z - 2), two barriers back.  Every warp passes the same barriers; the barrier ORs the
+      // iteration's barrier; A(z + 1) writes rho plane z + 1, whose buffer was last read for
+      // B(z - 1), before that barrier.  Every warp passes the same barriers; the barrier ORs the
       // warps' abort states (a timed-out wait here, or the producer's flag), so all warps leave
       // after the same iteration.
       auto iter = [&](int zz, R (&fc)[7][NPT], R (&fn)[7][NPT], const R (&rp)[NPT],
@@ -816,7 +826,7 @@ constexpr size_t tma_smem_bytes() {
   constexpr int SLOTB = sizeof(S) == 2 ? PlaneLayout<BY, BX>::slot_bytes()
                                        : TmaLayout<BY, BX>::template slot_bytes<S>();
   return 128 /* alignment slack */ + 128 /* barriers */ + (size_t)NB * SLOTB +
-         ((3 * PS * sizeof(R) + 127) / 128) * 128 + (size_t)NB * TABB +
+         ((2 * PS * sizeof(R) + 127) / 128) * 128 + (size_t)NB * TABB +
          (ANA ? ((3 * (BY + 2) * sizeof(MetricR<R>) + 127) / 128) * 128 : 0);  // see step_tma_kernel
 }
 
@@ -828,7 +838,7 @@ template <typename S, typename F>
 auto tma_dispatch(int by, int npt, bool ana, F&& f) {
   if constexpr (sizeof(S) == 2) {
     if (npt == 4)
-      return by == 7 ? f(step_tma_kernel<S, 7, 4, false>, tma_smem_bytes<S, 7, 4, false>())
+      return by == 5 ? f(step_tma_kernel<S, 5, 4, false>, tma_smem_bytes<S, 5, 4, false>())
                      : f(step_tma_kernel<S, 4, 4, false>, tma_smem_bytes<S, 4, 4, false>());
   } else {
     if (ana)
@@ -1021,13 +1031,23 @@ cudaError_t launch_step(Grid* g, int src) {
 }
 
 // Launch shape.  TMA tile kernel (q2 extent a multiple of the tile width, non-periodic q1):
-// tiles of BX = 64 columns (two nodes per lane) or, for 16-bit storage when the q2 extent is
-// a multiple of 128, BX = 128 (four nodes per lane: at 16-bit byte rates the two-node form
-// runs out of instruction issue); BY in {4, 7} rows, never with a halo row on the q1 = n1 - 1
-// face.  The resident CTAs per SM follow from shared memory and the kernel's register count;
-// the number of q3 segments minimises waves x CTAs per SM x (planes per segment + 3) x
-// (BY + 2) x BX, the node-planes an SM stages with whole waves counted.  Otherwise the
-// register-pipelined kernel with 512-thread tiles.
+// tiles of BX = 64 columns (two nodes per lane) of 4 or 7 rows or, for 16-bit storage when the
+// q2 extent is a multiple of 128, BX = 128 (four nodes per lane: at 16-bit byte rates the
+// two-node form runs out of instruction issue) of 4 or 5 rows.  Five rows are the most of which
+// two CTAs fit an SM (8 warps x 128 registers, two rho planes): the halo rows' density is 2 of 7
+// rows' work instead of 2 of 6 (trumpet 250 x 256 x 512 FP16, same division into blocks: 176 us
+// a step of 4 rows, 169 of 5).  The resident CTAs per SM follow from shared memory and the
+// kernel's register count.
+//
+// Division into blocks (TileCuts).  A segment of L planes costs about L + 3 (the planes staged
+// around it), so few long segments are best, but whole waves of them leave SMs idle in the last
+// one.  So the items that fill the SMs a whole number of times run whole, and the remaining ones
+// are cut so finely that their pieces fill the SMs once more; cost = node-planes an SM stages,
+// per_sm x (BY + 2) x BX x (whole waves x (L + 3) + (L / pieces + 3)).  Against equal segments
+// only: torus 192 x 1024 x 256 BF16 290 -> 266 us a step (312 tiles on 304 slots), FP32 462 ->
+// 457; trumpet 256 x 256 x 512 FP16 184 -> 175.
+//
+// Otherwise the register-pipelined kernel with 512-thread tiles.
 void step_launch_shape(Grid* g) {
   const int n1 = g->d.n[0], n2 = g->d.n[1], n3 = g->d.n[2];
   int dev = 0, sms = 152, smem_max = 227 * 1024;
@@ -1039,13 +1059,14 @@ void step_launch_shape(Grid* g) {
   const int npt = (g->elem == 2 && n2 % 128 == 0) ? 4 : 2, bx = 32 * npt;
   const bool ana = g->d.geom_mode == LBW_GEOM_ANALYTIC;
   if (n2 % bx == 0 && g->d.bc[0] != LBW_BC_PERIODIC && g->nn * 7 < (1LL << 31)) {
-    const int bys[2] = {4, 7};
+    const int bys[2] = {4, npt == 4 ? 5 : 7};
     int per_sm_of[2] = {0, 0};
     for (int c = 0; c < 2; ++c) {
       const int by = bys[c], threads = 32 * (by + 3);
       const TmaInfo ti = tma_info(g->d.prec, by, npt, ana);
       if ((long long)ti.smem > smem_max || ti.regs > 255) continue;
-      if ((n1 - 1) % by == 0) continue;  // a halo row would sit on the q1 = n1 - 1 face
+      // 32/64-bit: no halo row on the q1 = n1 - 1 face, whose rule reads a row staged elsewhere
+      if (g->elem > 2 && (n1 - 1) % by == 0) continue;
       const int rr = (ti.regs + 7) & ~7;
       const int per_sm = std::min<int>(2048 / threads, (int)((228LL * 1024) / (ti.smem + 1024)));
       per_sm_of[c] = std::max(1, std::min(per_sm, 65536 / (rr * threads)));
@@ -1059,25 +1080,24 @@ void step_launch_shape(Grid* g) {
       if (per_sm == 0 || (two && per_sm < 2)) continue;
       const long long tiles = (long long)(n2 / bx) * ((n1 + by - 1) / by);
       const long long slots = (long long)sms * per_sm;
-      for (long long segs = 1; segs <= n3; ++segs) {
-        const int lz = (int)((n3 + segs - 1) / segs);
-        const long long blocks = tiles * ((n3 + lz - 1) / lz);
-        const long long waves = (blocks + slots - 1) / slots;
-        const double cost = (double)waves * per_sm * (lz + 3) * (by + 2) * bx;
-        if (cost < best) {
+      for (long long segs = 1; segs <= n3 && segs * n3 < (1LL << 31); ++segs) {
+        const long long items = tiles * segs, waves = items / slots, rem = items % slots;
+        const long long len = (n3 + segs - 1) / segs;
+        const long long split = waves && rem ? std::min(slots / rem, n3 / segs) : 1;
+        const long long planes = waves * (len + 3) + (rem ? (len + split - 1) / split + 3 : 0);
+        const double cost = (double)planes * per_sm * (by + 2) * bx;
+        if (cost < best && items + rem * (split - 1) < (1LL << 31)) {
           best = cost;
           g->tma_by = by;
-          g->lz = lz;
+          g->cuts = {(unsigned)tiles, (unsigned)(n2 / bx), (unsigned)segs, (unsigned)(items - rem), (unsigned)split};
+          g->grid_dim = dim3((unsigned)(items - rem + rem * split));
         }
       }
     }
     if (g->tma_by > 0) {
       g->tma_npt = npt;
       cudaError_t e = dispatch(g->d.prec, [&](auto tag) { return tma_prepare_t<decltype(tag)>(g->tma_by, npt, ana); });
-      if (e == cudaSuccess && build_tmaps(g, g->tma_by, bx)) {
-        g->grid_dim = dim3(n2 / bx, (n1 + g->tma_by - 1) / g->tma_by, (n3 + g->lz - 1) / g->lz);
-        return;
-      }
+      if (e == cudaSuccess && build_tmaps(g, g->tma_by, bx)) return;
       cudaGetLastError();
       g->tma_by = 0;
     }

@@ -1,0 +1,46 @@
+"""The tile kernel's division into blocks: sizes whose last blocks are pieces of the remaining
+(tile, segment) items, five-row tiles of 16-bit storage, a halo row on the q1 = n1 - 1 face
+((n1 - 1) a multiple of five), a last tile row of one lattice row, every kind of face.
+
+One device step from a shared state that the storage holds exactly against one FP64 oracle step
+at every node; FP32: 1e-6 of the largest population, 16-bit: half an ulp of the stored value more
+(FP16 2^-11, BF16 2^-8), as in the full-size parity test."""
+import numpy as np
+import pytest
+
+import lbw_workloads as W
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+RTOL = {W.PREC_F32: 0.0, W.PREC_F16S: 2.0 ** -11, W.PREC_BF16S: 2.0 ** -8}
+BOX = dict(h=(1, 1, 1), x0=(0, 0, 0), c=0.4, damping=0.7)
+SPECS = {
+    "torus-bf16": W.torus(101, 1024, 16).with_(prec=W.PREC_BF16S),       # 168 tiles, 8 pieces
+    "cylinder-f16": W.cylinder(161, 640, 16).with_(prec=W.PREC_F16S),
+    "walls-f16": W.GridSpec(kind=W.KIND_CARTESIAN, n=(161, 640, 16), bc=(3, 1, 1, 2, 2, 3), prec=W.PREC_F16S, **BOX),
+    "free-f16": W.GridSpec(kind=W.KIND_CARTESIAN, n=(101, 1024, 16), bc=(2, 3, 3, 3, 0, 0), prec=W.PREC_F16S, **BOX),
+    "torus-f32": W.torus(192, 768, 5).with_(prec=W.PREC_F32),            # 336 tiles, 5 pieces of a plane
+    "walls-f32": W.GridSpec(kind=W.KIND_CARTESIAN, n=(121, 640, 13), bc=(1, 3, 3, 1, 2, 2), prec=W.PREC_F32, **BOX),
+}
+
+
+@pytest.mark.parametrize("name", list(SPECS))
+def test_one_step(name):
+    from paper_1705_01801_gb300 import lbw
+    spec = SPECS[name].with_(geom_mode=1)  # a launch per step
+    rng = np.random.default_rng(3)
+    shape = (7, spec.n[2], spec.n[0], spec.n[1])
+    if spec.prec == W.PREC_F32:
+        f = rng.standard_normal(shape, dtype=np.float32).astype(np.float64)
+    else:
+        w = np.array([0.25] + [0.125] * 6)[:, None, None, None]
+        f = rng.integers(-64, 65, size=shape).astype(np.float64) / 64.0 * w
+    g, o = lbw.Grid(spec), oracle.OracleGrid(spec)
+    for s in (g, o):
+        s.set_f(f)
+        s.step(1)
+    fo = o.get_f()
+    np.testing.assert_allclose(g.get_f(), fo, rtol=RTOL[spec.prec], atol=1e-6 * np.abs(fo).max())
+    g.close()
+    o.close()
