@@ -65,7 +65,7 @@ struct Grid {
   // launch shape of the step kernel
   int bx = 0, by = 0, lz = 0;
   TileCuts cuts = {};     // the tile kernel's blocks
-  int tma_by = 0;          // 0: register-pipelined kernel; 4, 5 or 7: TMA tile kernel rows
+  int tma_by = 0;          // 0: register-pipelined kernel; otherwise the TMA tile kernel's rows
   int tma_npt = 2;         // TMA tile kernel: nodes per lane (tile width 32 x tma_npt)
   // padded storage (ensembles on the tile kernel): row length and first data column in
   // elements; pitch 0 means dense rows of n2 values

@@ -830,23 +830,43 @@ constexpr size_t tma_smem_bytes() {
          (ANA ? ((3 * (BY + 2) * sizeof(MetricR<R>) + 127) / 128) * 128 : 0);  // see step_tma_kernel
 }
 
+// Tile rows built for a storage size, nodes per lane and geometry (step_launch_shape chooses).
+struct TileRows {
+  int count, by[3];
+};
+TileRows tile_rows(size_t elem, int npt, bool ana) {
+  if (npt == 4) return {3, {5, 12, 13}};
+  return elem == 8 || ana ? TileRows{2, {4, 7, 0}} : TileRows{3, {4, 7, 16}};
+}
+
 // The tile kernel for (rows BY, nodes per lane NPT, analytic geometry or not): f(kernel,
 // dynamic shared bytes).  Four nodes per lane (128-column tiles) exist for the 16-bit storage
 // formats only, the analytic geometry for 32- and 64-bit storage only; the table-geometry
 // kernels carry none of the analytic code.
 template <typename S, typename F>
 auto tma_dispatch(int by, int npt, bool ana, F&& f) {
+  auto at = [&](auto rows, auto nodes, auto analytic) {
+    constexpr int BY = decltype(rows)::value, NPT = decltype(nodes)::value;
+    constexpr bool ANA = decltype(analytic)::value;
+    return f(step_tma_kernel<S, BY, NPT, ANA>, tma_smem_bytes<S, BY, NPT, ANA>());
+  };
+  using std::integral_constant;
+  const std::false_type table{};
+  const integral_constant<int, 2> two{};
   if constexpr (sizeof(S) == 2) {
+    const integral_constant<int, 4> four{};
     if (npt == 4)
-      return by == 5 ? f(step_tma_kernel<S, 5, 4, false>, tma_smem_bytes<S, 5, 4, false>())
-                     : f(step_tma_kernel<S, 4, 4, false>, tma_smem_bytes<S, 4, 4, false>());
+      return by == 5    ? at(integral_constant<int, 5>{}, four, table)
+             : by == 12 ? at(integral_constant<int, 12>{}, four, table)
+                        : at(integral_constant<int, 13>{}, four, table);
   } else {
     if (ana)
-      return by == 7 ? f(step_tma_kernel<S, 7, 2, true>, tma_smem_bytes<S, 7, 2, true>())
-                     : f(step_tma_kernel<S, 4, 2, true>, tma_smem_bytes<S, 4, 2, true>());
+      return by == 7 ? at(integral_constant<int, 7>{}, two, std::true_type{})
+                     : at(integral_constant<int, 4>{}, two, std::true_type{});
   }
-  return by == 7 ? f(step_tma_kernel<S, 7, 2, false>, tma_smem_bytes<S, 7, 2, false>())
-                 : f(step_tma_kernel<S, 4, 2, false>, tma_smem_bytes<S, 4, 2, false>());
+  if constexpr (sizeof(S) < 8)
+    if (by == 16) return at(integral_constant<int, 16>{}, two, table);
+  return by == 7 ? at(integral_constant<int, 7>{}, two, table) : at(integral_constant<int, 4>{}, two, table);
 }
 
 template <typename S>
@@ -1031,21 +1051,25 @@ cudaError_t launch_step(Grid* g, int src) {
 }
 
 // Launch shape.  TMA tile kernel (q2 extent a multiple of the tile width, non-periodic q1):
-// tiles of BX = 64 columns (two nodes per lane) of 4 or 7 rows or, for 16-bit storage when the
-// q2 extent is a multiple of 128, BX = 128 (four nodes per lane: at 16-bit byte rates the
-// two-node form runs out of instruction issue) of 4 or 5 rows.  Five rows are the most of which
-// two CTAs fit an SM (8 warps x 128 registers, two rho planes): the halo rows' density is 2 of 7
-// rows' work instead of 2 of 6 (trumpet 250 x 256 x 512 FP16, same division into blocks: 176 us
-// a step of 4 rows, 169 of 5).  The resident CTAs per SM follow from shared memory and the
-// kernel's register count.
+// tiles of BX = 64 columns (two nodes per lane) or, for 16-bit storage when the q2 extent is a
+// multiple of 128, BX = 128 (four nodes per lane: at 16-bit byte rates the two-node form runs
+// out of instruction issue).  The density of the two halo rows is work that the neighbouring
+// tiles repeat, so tall tiles are cheap: 13 (12) rows of 128 columns fill an SM's registers with
+// one CTA of 16 (15) warps of 128 registers, against two CTAs of 5 rows; 16 rows of 64 columns
+// with 19 warps, against two CTAs of 7 rows.  Fewer rows remain for lattices that they divide
+// better.  us a step, two short CTAs against a tall one: trumpet 256 x 256 x 512 FP16 175 / 161
+// (13 rows), torus 192 x 1024 x 256 BF16 266 / 253 (12), torus FP32 457 / 448 (16), cylinder
+// 128 x 128 x 256 FP32 43.5 / 41.5.
 //
 // Division into blocks (TileCuts).  A segment of L planes costs about L + 3 (the planes staged
 // around it), so few long segments are best, but whole waves of them leave SMs idle in the last
 // one.  So the items that fill the SMs a whole number of times run whole, and the remaining ones
 // are cut so finely that their pieces fill the SMs once more; cost = node-planes an SM stages,
-// per_sm x (BY + 2) x BX x (whole waves x (L + 3) + (L / pieces + 3)).  Against equal segments
-// only: torus 192 x 1024 x 256 BF16 290 -> 266 us a step (312 tiles on 304 slots), FP32 462 ->
-// 457; trumpet 256 x 256 x 512 FP16 184 -> 175.
+// per_sm x (BY + 2) x BX x (whole waves x (L + 3) + (L / pieces + 3)), times 1.08 for a lone CTA
+// per SM, which idles it at every plane barrier (measured 1.08 to 1.12 on trumpet and torus, 1.04
+// on the cylinder).  Against equal segments only, with tiles of 5 and 7 rows: torus 192 x 1024 x
+// 256 BF16 290 -> 266 us a step (312 tiles on 304 slots), FP32 462 -> 457; trumpet 256 x 256 x
+// 512 FP16 184 -> 175.
 //
 // Otherwise the register-pipelined kernel with 512-thread tiles.
 void step_launch_shape(Grid* g) {
@@ -1059,25 +1083,18 @@ void step_launch_shape(Grid* g) {
   const int npt = (g->elem == 2 && n2 % 128 == 0) ? 4 : 2, bx = 32 * npt;
   const bool ana = g->d.geom_mode == LBW_GEOM_ANALYTIC;
   if (n2 % bx == 0 && g->d.bc[0] != LBW_BC_PERIODIC && g->nn * 7 < (1LL << 31)) {
-    const int bys[2] = {4, npt == 4 ? 5 : 7};
-    int per_sm_of[2] = {0, 0};
-    for (int c = 0; c < 2; ++c) {
-      const int by = bys[c], threads = 32 * (by + 3);
+    const TileRows rows = tile_rows(g->elem, npt, ana);
+    double best = 1e300;
+    for (int c = 0; c < rows.count; ++c) {
+      const int by = rows.by[c], threads = 32 * (by + 3);
       const TmaInfo ti = tma_info(g->d.prec, by, npt, ana);
       if ((long long)ti.smem > smem_max || ti.regs > 255) continue;
       // 32/64-bit: no halo row on the q1 = n1 - 1 face, whose rule reads a row staged elsewhere
       if (g->elem > 2 && (n1 - 1) % by == 0) continue;
       const int rr = (ti.regs + 7) & ~7;
-      const int per_sm = std::min<int>(2048 / threads, (int)((228LL * 1024) / (ti.smem + 1024)));
-      per_sm_of[c] = std::max(1, std::min(per_sm, 65536 / (rr * threads)));
-    }
-    // a lone CTA per SM idles the SM at every plane barrier (measured: 16-bit trumpet 8% slower
-    // than two CTAs of fewer rows), so shapes with two or more resident CTAs come first
-    const bool two = per_sm_of[0] >= 2 || per_sm_of[1] >= 2;
-    double best = 1e300;
-    for (int c = 0; c < 2; ++c) {
-      const int by = bys[c], per_sm = per_sm_of[c];
-      if (per_sm == 0 || (two && per_sm < 2)) continue;
+      const int per_sm = std::max(1, std::min(std::min<int>(2048 / threads, (int)((228LL * 1024) / (ti.smem + 1024))),
+                                              65536 / (rr * threads)));
+      const double lone = per_sm == 1 ? 1.08 : 1.0;
       const long long tiles = (long long)(n2 / bx) * ((n1 + by - 1) / by);
       const long long slots = (long long)sms * per_sm;
       for (long long segs = 1; segs <= n3 && segs * n3 < (1LL << 31); ++segs) {
@@ -1085,7 +1102,7 @@ void step_launch_shape(Grid* g) {
         const long long len = (n3 + segs - 1) / segs;
         const long long split = waves && rem ? std::min(slots / rem, n3 / segs) : 1;
         const long long planes = waves * (len + 3) + (rem ? (len + split - 1) / split + 3 : 0);
-        const double cost = (double)planes * per_sm * (by + 2) * bx;
+        const double cost = lone * (double)planes * per_sm * (by + 2) * bx;
         if (cost < best && items + rem * (split - 1) < (1LL << 31)) {
           best = cost;
           g->tma_by = by;

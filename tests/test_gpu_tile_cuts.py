@@ -1,6 +1,7 @@
-"""The tile kernel's division into blocks: sizes whose last blocks are pieces of the remaining
-(tile, segment) items, five-row tiles of 16-bit storage, a halo row on the q1 = n1 - 1 face
-((n1 - 1) a multiple of five), a last tile row of one lattice row, every kind of face.
+"""The tile kernel's tiles and their division into blocks: tile heights 5, 7, 12, 13 and 16,
+sizes whose last blocks are pieces of the remaining (tile, segment) items, a halo row on the
+q1 = n1 - 1 face ((n1 - 1) a multiple of a 16-bit tile's rows), a last tile of few lattice rows,
+every kind of face.
 
 One device step from a shared state that the storage holds exactly against one FP64 oracle step
 at every node; FP32: 1e-6 of the largest population, 16-bit: half an ulp of the stored value more
@@ -16,12 +17,20 @@ pytestmark = pytest.mark.gpu
 RTOL = {W.PREC_F32: 0.0, W.PREC_F16S: 2.0 ** -11, W.PREC_BF16S: 2.0 ** -8}
 BOX = dict(h=(1, 1, 1), x0=(0, 0, 0), c=0.4, damping=0.7)
 SPECS = {
-    "torus-bf16": W.torus(101, 1024, 16).with_(prec=W.PREC_BF16S),       # 168 tiles, 8 pieces
+    "torus-bf16": W.torus(101, 1024, 16).with_(prec=W.PREC_BF16S),
     "cylinder-f16": W.cylinder(161, 640, 16).with_(prec=W.PREC_F16S),
     "walls-f16": W.GridSpec(kind=W.KIND_CARTESIAN, n=(161, 640, 16), bc=(3, 1, 1, 2, 2, 3), prec=W.PREC_F16S, **BOX),
     "free-f16": W.GridSpec(kind=W.KIND_CARTESIAN, n=(101, 1024, 16), bc=(2, 3, 3, 3, 0, 0), prec=W.PREC_F16S, **BOX),
-    "torus-f32": W.torus(192, 768, 5).with_(prec=W.PREC_F32),            # 336 tiles, 5 pieces of a plane
+    "torus-f32": W.torus(192, 768, 5).with_(prec=W.PREC_F32),
     "walls-f32": W.GridSpec(kind=W.KIND_CARTESIAN, n=(121, 640, 13), bc=(1, 3, 3, 1, 2, 2), prec=W.PREC_F32, **BOX),
+    "rows5-f16": W.cylinder(157, 512, 16).with_(prec=W.PREC_F16S),
+    "rows12-face-f16": W.GridSpec(kind=W.KIND_CARTESIAN, n=(61, 128, 24), bc=(2, 1, 2, 3, 1, 1), prec=W.PREC_F16S, **BOX),
+    "rows12-pieces-bf16": W.torus(196, 640, 16).with_(prec=W.PREC_BF16S),
+    "rows13-f16": W.cylinder(37, 128, 40).with_(prec=W.PREC_F16S),
+    "rows13-face-bf16": W.GridSpec(kind=W.KIND_CARTESIAN, n=(196, 128, 9), bc=(1, 3, 0, 0, 3, 2), prec=W.PREC_BF16S, **BOX),
+    "rows16-face-f16": W.GridSpec(kind=W.KIND_CARTESIAN, n=(145, 192, 5), bc=(3, 2, 1, 1, 0, 0), prec=W.PREC_F16S, **BOX),
+    "rows16-pieces-f32": W.cylinder(197, 384, 16).with_(prec=W.PREC_F32),
+    "rows16-f32": W.GridSpec(kind=W.KIND_CARTESIAN, n=(29, 64, 5), bc=(2, 1, 3, 2, 3, 1), prec=W.PREC_F32, **BOX),
 }
 
 
