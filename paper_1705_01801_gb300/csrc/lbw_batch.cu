@@ -558,44 +558,71 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
 // q2 tile.  The tile height follows the member (narrow rows give tall tiles).  The staging
 // pipeline, slot regrouping, faces and collision are those of batch_tma_kernel.  32- and
 // 64-bit storage.
-constexpr int kRowWarps = 9;                   // consumer warps
-constexpr int kRowNodes = kRowWarps * 32 * 2;  // nodes of a tile plane
-constexpr int kRowCap = 648;                   // staged elements of a population plane
-constexpr int kRowMaxBY = 16;                  // tile rows at most (coefficient slots)
-constexpr int kRowMinBY = 3;                   // fewer would put a halo row on a q1 face
+//
+// Two forms.  Nine consumer warps: two CTAs per SM (FP32), up to 16 rows.  FP32 also has a tall
+// one of 19 warps with one CTA per SM (cps = 1): the two halo rows, whose density the
+// neighbouring tiles compute again, are then a smaller part of the tile (96 columns: 2 of 12 rows
+// instead of 2 of 6).  There every member's rows are divided evenly over as few tiles as they
+// need.  us a step, FP32 cylinders: 100 x 100 x 250 34.6 -> 28.1, 60 x 100 x 400 34.6 -> 26.6,
+// 200 x 100 x 256 62 -> 51, 80 x 37 x 400 20.1 -> 16.6; 48 trumpets (bound by DRAM) 607 / 604.
+constexpr int kRowMinBY = 3;  // fewer would put a halo row on a q1 face
+template <int W>
+struct RowTile {
+  static constexpr int kNodes = W * 32 * 2;         // nodes of a tile plane
+  static constexpr int kCap = W == 9 ? 648 : 1368;  // staged elements of a population plane
+  static constexpr int kMaxBY = W == 9 ? 16 : 34;   // tile rows at most (coefficient slots)
+};
+constexpr int kTallWarps = 19;
 
-// Staged rows of a member's full-row tile (BY_m + 2), 0 when the member cannot use one.
+// Staged rows of a full-row tile that holds as many of n2 columns as fit (BY + 2), 0 when a
+// lattice cannot use one.
+template <int W>
 inline int row_tile_rows(int n2, size_t es) {
+  using T = RowTile<W>;
   const int v = (int)(16 / es), n2w = n2 + (n2 & 1), bw = (n2 + v - 1) / v * v;
   if (bw > 256) return 0;
-  const int rows = std::min(std::min(kRowNodes / n2w, kRowCap / bw), kRowMaxBY + 2);
+  const int rows = std::min(std::min(T::kNodes / n2w, T::kCap / bw), T::kMaxBY + 2);
   return rows - 2 >= kRowMinBY ? rows : 0;
 }
 
-template <typename S>
+// The form that a launch shape's CTAs per SM stand for, and the rows of a lattice's tiles in it
+// (tiles start at q1 = -1 when (n1 - 1) is a multiple of the rows, which may cost one more).
+inline bool tall_rows(size_t es, int cps) { return es == 4 && cps == 1; }
+inline int row_tile_by(int n1, int n2, size_t es, int cps) {
+  if (!tall_rows(es, cps)) return row_tile_rows<9>(n2, es) - 2;
+  const int most = row_tile_rows<kTallWarps>(n2, es) - 2;
+  if (most < kRowMinBY) return most;
+  const int tiles = (n1 + most - 1) / most;
+  int by = std::max(kRowMinBY, (n1 + tiles - 1) / tiles);
+  if ((n1 - 1) % by == 0 && by < most) ++by;
+  return by;
+}
+
+template <typename S, int W>
 struct BatchRowLayout {
   using R = typename Store<S>::R;
-  static constexpr int POPB = ((kRowCap * (int)sizeof(S)) + 127) / 128 * 128;
+  using T = RowTile<W>;
+  static constexpr int POPB = ((T::kCap * (int)sizeof(S)) + 127) / 128 * 128;
   static constexpr int SLOTB = 7 * POPB;
-  static constexpr int TABB = ((kRowMaxBY * T_SLOTS * (int)sizeof(R)) + 127) / 128 * 128;
-  static constexpr int RHOB = ((3 * kRowNodes * (int)sizeof(R)) + 127) / 128 * 128;
+  static constexpr int TABB = ((T::kMaxBY * T_SLOTS * (int)sizeof(R)) + 127) / 128 * 128;
+  static constexpr int RHOB = ((3 * T::kNodes * (int)sizeof(R)) + 127) / 128 * 128;
 };
 
-template <typename S>
+template <typename S, int W>
 constexpr size_t batch_row_smem() {
-  using L = BatchRowLayout<S>;
+  using L = BatchRowLayout<S, W>;
   return 128 + 128 + 5 * (size_t)L::SLOTB + L::RHOB + 5 * (size_t)L::TABB;
 }
 
-template <typename S>
-__global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) batch_row_kernel(
+template <typename S, int W>
+__global__ void __launch_bounds__(32 * (W + 1), sizeof(S) == 4 && W == 9 ? 2 : 1) batch_row_kernel(
     const StepArgs<S>* __restrict__ members, const CUtensorMap* __restrict__ maps, int src,
     const BatchItem* __restrict__ items, int n_items, unsigned long long* counters, int nprobe,
     long long cap) {
   using R = typename Store<S>::R;
-  using L = BatchRowLayout<S>;
+  using L = BatchRowLayout<S, W>;
   static_assert(sizeof(S) >= 4, "the full-row tile regroups slots: 32- and 64-bit storage");
-  constexpr int NPT = 2, NB = 5, NCW = kRowWarps;
+  constexpr int NPT = 2, NB = 5, NCW = W;
   constexpr int ES = (int)sizeof(S), RS = (int)sizeof(R), V = 16 / ES;
   constexpr int POPB = L::POPB, SLOTB = L::SLOTB, TABB = L::TABB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -754,7 +781,7 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1), sizeof(S) == 4 ? 2 : 1) 
       const unsigned myrho = (unsigned)((row * n2w + col) * RS);
       const unsigned lrho = (unsigned)((row * n2w + cl) * RS), rrho = (unsigned)((row * n2w + cr) * RS);
       const unsigned wrho = (unsigned)(row * n2w * RS);
-      constexpr unsigned PLANE = (unsigned)(kRowNodes * RS);
+      constexpr unsigned PLANE = (unsigned)(RowTile<W>::kNodes * RS);
 
       bool has_probe = false;
       if (owner && t_sample < (unsigned long long)A.cap)
@@ -1110,17 +1137,20 @@ auto prec_dispatch(int prec, F&& f) {
 
 // resident CTAs per SM of the full-row kernel (0 when it cannot run)
 int row_cps(int prec) {
-  auto occ = [](auto kern, size_t smem) {
+  auto occ = [](auto kern, size_t smem, int warps) {
     int per = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * (kRowWarps + 1), smem) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * (warps + 1), smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
     return per;
   };
-  if (prec == LBW_F32) return occ(batch_row_kernel<float>, batch_row_smem<float>());
-  if (prec == LBW_F64) return occ(batch_row_kernel<double>, batch_row_smem<double>());
+  if (prec == LBW_F32)
+    return occ(batch_row_kernel<float, kTallWarps>, batch_row_smem<float, kTallWarps>(), kTallWarps) > 0
+               ? occ(batch_row_kernel<float, 9>, batch_row_smem<float, 9>(), 9)
+               : 0;
+  if (prec == LBW_F64) return occ(batch_row_kernel<double, 9>, batch_row_smem<double, 9>(), 9);
   return 0;
 }
 
@@ -1224,7 +1254,8 @@ lbw_status use_layout(lbw_batch* b, bool rebuild) {
 
 // Tensor maps of every member for tile rows `by`: 4-D views (stored column, q1, q3,
 // population) of both buffers with (64 + 2 G) x (by + 2) boxes, 3-D view of the table.
-lbw_status build_batch_maps(lbw_batch* b, int by) {
+lbw_status build_batch_maps(lbw_batch* b, const Shape& shape) {
+  const int by = shape.by;
   const size_t es = es_of(b->prec);
   const int rprec = b->prec == LBW_F64 ? LBW_F64 : LBW_F32;
   const size_t rs = rs_of(b->prec);
@@ -1235,7 +1266,7 @@ lbw_status build_batch_maps(lbw_batch* b, int by) {
     const uint64_t dims[4] = {P, n1, n3, 7};
     const uint64_t strides[3] = {P * es, P * n1 * es, P * n1 * n3 * es};
     // by = 0: full-row tiles, the member's n2 data columns (rounded up to 16 bytes) x its rows
-    const int v = (int)(16 / es), rows = by == 0 ? row_tile_rows(g.d.n[1], es) : by + 2;
+    const int v = (int)(16 / es), rows = (by == 0 ? row_tile_by(g.d.n[0], g.d.n[1], es, shape.cps) : by) + 2;
     if (rows < 3) return fail(LBW_EINVAL, "ensemble member " + std::to_string(m) + " does not fit a full-row tile");
     const uint32_t box[4] = {(uint32_t)(by == 0 ? (g.d.n[1] + v - 1) / v * v : kTmaBatchBX + 2 * g.col0),
                              (uint32_t)rows, 1, 1};
@@ -1275,7 +1306,7 @@ lbw_status list_items(const lbw_batch* b, const Shape& shape, std::vector<BatchI
   for (int m = 0; m < b->n; ++m) {
     const lbw_grid_desc& d = b->views[m].d;
     const bool rows = b->tma && shape.by == 0;
-    const int by = rows ? row_tile_rows(d.n[1], b->views[m].elem) - 2 : shape.by;
+    const int by = rows ? row_tile_by(d.n[0], d.n[1], b->views[m].elem, shape.cps) : shape.by;
     if (rows && by < kRowMinBY) return fail(LBW_EINVAL, "ensemble member does not fit a full-row tile");
     const int bx = rows ? d.n[1] : b->tma ? kTmaBatchBX : kBatchBX;
     const int y_start = (b->tma && (d.n[0] - 1) % by == 0) ? -1 : 0;
@@ -1302,17 +1333,32 @@ lbw_status list_items(const lbw_batch* b, const Shape& shape, std::vector<BatchI
 
 // Segment length (and the kernel, among the tile rows `bys`) that ends a step first when CTAs
 // claim the items in order: an item costs its planes and some four more to fill the pipeline, a
-// plane as measured at two CTAs per SM (us: full-row tile 1.0, 7 rows of 64 columns 1.25, 4 rows 0.9).
+// plane as measured at two CTAs per SM (us: full-row tile 1.0, 7 rows of 64 columns 1.25, 4 rows
+// 0.9; the tall full-row tile, alone on its SM, 1.1: choices the same from 1.0 to 1.2).  A single
+// lattice has few items, so it also tries the lengths that divide its planes evenly and the tall
+// form; an ensemble's tail is cut (list_items) and DRAM bounds it in either form.
 Shape best_shape(const lbw_batch* b, const std::vector<int>& bys) {
   Shape best = b->shape;
   double best_cost = 1e300;
   std::vector<BatchItem> items;
+  struct Form {
+    int by, cps;
+  };
+  std::vector<Form> forms;
   for (const int by : bys) {
-    const int cps = std::min(2, tma_cps(b->prec, by));
-    for (const int lz : {64, 48, 32, 24, 16, 12, 8}) {
+    forms.push_back({by, std::min(2, tma_cps(b->prec, by))});
+    if (b->n == 1 && by == 0 && tall_rows(es_of(b->prec), 1)) forms.push_back({0, 1});
+  }
+  std::vector<int> lzs = {64, 48, 32, 24, 16, 12, 8};
+  if (b->n == 1) {
+    const int n3 = b->views[0].d.n[2];
+    for (int segs = 1; segs <= 32 && n3 / segs >= 8; ++segs) lzs.push_back((n3 + segs - 1) / segs);
+  }
+  for (const auto [by, cps] : forms) {
+    for (const int lz : lzs) {
       const Shape shape{by, lz, cps};
       if (shape.cps < 1 || list_items(b, shape, items) != LBW_OK) continue;
-      const double plane = by == 0 ? 1.0 : by == 7 ? 1.25 : 0.9;
+      const double plane = by == 0 ? (tall_rows(es_of(b->prec), cps) ? 1.1 : 1.0) : by == 7 ? 1.25 : 0.9;
       const size_t slots = std::min(items.size(), grid_slots(shape));
       double work = 0.0;
       for (const BatchItem& t : items) work += plane * (t.z1 - t.z0 + 4);
@@ -1357,7 +1403,7 @@ lbw_status refresh(lbw_batch* b, bool rebuild_ghosts = false) {
   if (st == LBW_OK) st = build_items(b);
   if (st != LBW_OK) return st;
   if (b->tma) {
-    st = build_batch_maps(b, b->shape.by);
+    st = build_batch_maps(b, b->shape);
     if (st != LBW_OK) return st;
   }
   return upload_members(b);
@@ -1383,7 +1429,12 @@ cudaError_t launch_batch_t(lbw_batch* b, int src) {
                                 b->counters, b->nprobe, (long long)b->cap);
     };
     if constexpr (sizeof(S) >= 4) {
-      if (b->shape.by == 0) return launch(batch_row_kernel<S>, batch_row_smem<S>(), kRowWarps + 1);
+      if (b->shape.by == 0) {
+        if constexpr (sizeof(S) == 4)
+          if (tall_rows(sizeof(S), b->shape.cps))
+            return launch(batch_row_kernel<S, kTallWarps>, batch_row_smem<S, kTallWarps>(), kTallWarps + 1);
+        return launch(batch_row_kernel<S, 9>, batch_row_smem<S, 9>(), 9 + 1);
+      }
     }
     return batch_tma_dispatch<S>(b->shape.by,
                                  [&](auto kern, size_t smem) { return launch(kern, smem, b->shape.by + 3); });
@@ -1536,7 +1587,7 @@ lbw_status lbw_batch_create(const lbw_grid_desc* descs, int32_t n, void* stream,
     // full-row tiles: 32- or 64-bit storage and every member's row in a tile
     b->rowk = b->tma && row_cps(b->prec) > 0;
     for (int m = 0; m < n && b->rowk; ++m)
-      if (row_tile_rows(descs[m].n[1], es) == 0) b->rowk = false;
+      if (row_tile_rows<9>(descs[m].n[1], es) == 0) b->rowk = false;
   }
   std::vector<double> tab_all;
   size_t ftot = 0;
@@ -1996,7 +2047,7 @@ lbw_status ragged_plan(Grid* g) {
   b->prec = g->d.prec;
   b->stream = g->stream;
   b->tma = true;
-  b->rowk = row_tile_rows(g->d.n[1], g->elem) > 0 && row_cps(g->d.prec) > 0;
+  b->rowk = row_tile_rows<9>(g->d.n[1], g->elem) > 0 && row_cps(g->d.prec) > 0;
   b->views.assign(1, *g);
   b->foff.assign(1, 0);
   std::vector<int> bys = {7, 4};
