@@ -2047,7 +2047,12 @@ lbw_status ragged_plan(Grid* g) {
   b->prec = g->d.prec;
   b->stream = g->stream;
   b->tma = true;
-  b->rowk = row_tile_rows<9>(g->d.n[1], g->elem) > 0 && row_cps(g->d.prec) > 0;
+  // the tall tile takes rows of up to 242 columns: 150 x 200 x 200 79.5 -> 57.5 us a step against
+  // 64-column tiles, 200 x 130 x 100 43.3 -> 31.5, 90 x 170 x 300 58.5 -> 49.7 (64-column tiles of
+  // 16 rows, one CTA per SM: 3 to 10 % on 100 x 400 x 120 and 64 x 700 x 100, slower on others)
+  const bool fits = row_tile_rows<9>(g->d.n[1], g->elem) > 0 ||
+                    (tall_rows(g->elem, 1) && row_tile_rows<kTallWarps>(g->d.n[1], g->elem) > 0);
+  b->rowk = fits && row_cps(g->d.prec) > 0;
   b->views.assign(1, *g);
   b->foff.assign(1, 0);
   std::vector<int> bys = {7, 4};

@@ -3,7 +3,8 @@ both sides of one tile (34 rows at most), (n1 - 1) a multiple of the rows, two r
 q2 extents, segments of one to all planes, every q1 and q3 face, probes.
 
 FP32: 2e-5 of the largest population and ten times that for the probes, as in the other parity
-tests."""
+tests.  Single ragged lattices of 720,000 nodes, past the multi-step kernel, on both sides of
+the tall tile's widest row (242 columns)."""
 import numpy as np
 import pytest
 
@@ -49,3 +50,17 @@ def test_matches_oracle(lz):
         np.testing.assert_allclose(series[m], so, rtol=0, atol=2e-4 * np.abs(fo).max())
         o.close()
     b.close()
+
+
+@pytest.mark.parametrize("n", [(90, 200, 40), (75, 242, 40), (75, 244, 40)])
+def test_wide_rows(n):
+    from paper_1705_01801_gb300 import lbw
+    spec = W.cylinder(*n).with_(prec=W.PREC_F32, bc=(1, 3, 0, 0, 2, 1), damping=0.8)
+    g, o = lbw.Grid(spec), oracle.OracleGrid(spec)
+    for s in (g, o):
+        s.init(W.pulses(spec, 5, 3))
+        s.step(8)
+    fo = o.get_f()
+    np.testing.assert_allclose(g.get_f(), fo, rtol=0, atol=2e-5 * np.abs(fo).max())
+    g.close()
+    o.close()
