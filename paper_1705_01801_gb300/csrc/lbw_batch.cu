@@ -124,8 +124,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
   constexpr bool RG = sizeof(S) >= 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) StepArgs<S> A;
-  __shared__ int probe_list[kMaxProbes];
-  __shared__ int probe_cnt;
+  __shared__ TileProbes probes;
   __shared__ int abort_flag;
   __shared__ int next_it;
   __shared__ unsigned long long t_sample;
@@ -174,7 +173,8 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
         mbar_init_count(empty_at(k), NCW);
       }
       asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-      probe_cnt = 0;
+      probes.count = 0;
+      for (unsigned& p : probes.planes) p = 0;
     }
     fresh = false;
     __syncthreads();  // every thread has read next_it for this item
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
     if (tid < A.nprobe) {
       const int pq1 = A.probe_q[3 * tid], pq2 = A.probe_q[3 * tid + 1], pq3 = A.probe_q[3 * tid + 2];
       if (pq1 >= y0 && pq1 < y0 + BY && pq2 >= x0 && pq2 < x0 + BX && pq3 >= z0 && pq3 < z1)
-        probe_list[atomicAdd(&probe_cnt, 1)] = tid;
+        probes.add(tid, pq1, pq2, pq3);
     }
     __syncthreads();
     const CUtensorMap* tm_f = maps + 3 * item.member + src;
@@ -302,9 +302,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
       const unsigned hrho = (unsigned)(((hl + 1) * PW + ((w == 0) ? C0 - 1 : C0 + BX)) * RS);
       const unsigned myrho = (unsigned)((w * PW + C0 + c0) * RS);
 
-      bool has_probe = false;
-      if (owner && t_sample < (unsigned long long)A.cap)
-        for (int s = 0; s < probe_cnt; ++s) has_probe |= A.probe_q[3 * probe_list[s]] == q1;
+      const bool has_probe = owner && t_sample < (unsigned long long)A.cap && probes.row(q1);
 
       R fA[7][NPT], fB[7][NPT], rA[NPT], rB[NPT], rC[NPT];
       // storage of this lane's nodes (padded rows) and their ghost copies near the wrap
@@ -477,11 +475,11 @@ __global__ void __launch_bounds__(32 * (BY + 3)) batch_tma_kernel(
           if (gh1 != 0 && nvalid == 2) Store<S>::st(dst + 1 + gh1, fc[i][1]);
           dst += A.ps;
         }
-        if (has_probe) {
-          for (int s = 0; s < probe_cnt; ++s) {
-            const int k = probe_list[s];
-            const int dq = A.probe_q[3 * k + 1] - q2;
-            if (A.probe_q[3 * k] == q1 && dq >= 0 && dq < NPT && A.probe_q[3 * k + 2] == zc)
+        if (has_probe && probes.plane(zc)) {
+          for (int s = 0; s < probes.count; ++s) {
+            const int k = probes.id[s];
+            const int dq = probes.at[3 * s + 1] - q2;
+            if (probes.at[3 * s] == q1 && dq >= 0 && dq < NPT && probes.at[3 * s + 2] == zc)
               A.series[(long long)k * A.cap + t_sample] = (double)(dq == 0 ? rc[0] : rc[1]) * (double)c[T_INVSG];
           }
         }
@@ -627,8 +625,7 @@ __global__ void __launch_bounds__(32 * (W + 1), sizeof(S) == 4 && W == 9 ? 2 : 1
   constexpr int POPB = L::POPB, SLOTB = L::SLOTB, TABB = L::TABB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) StepArgs<S> A;
-  __shared__ int probe_list[kMaxProbes];
-  __shared__ int probe_cnt;
+  __shared__ TileProbes probes;
   __shared__ int abort_flag;
   __shared__ int next_it;
   __shared__ unsigned long long t_sample;
@@ -671,7 +668,8 @@ __global__ void __launch_bounds__(32 * (W + 1), sizeof(S) == 4 && W == 9 ? 2 : 1
         mbar_init_count(empty_at(k), NCW);
       }
       asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-      probe_cnt = 0;
+      probes.count = 0;
+      for (unsigned& p : probes.planes) p = 0;
     }
     fresh = false;
     __syncthreads();  // every thread has read next_it for this item
@@ -679,8 +677,8 @@ __global__ void __launch_bounds__(32 * (W + 1), sizeof(S) == 4 && W == 9 ? 2 : 1
     const bool p3 = A.bc[4] == LBW_BC_PERIODIC;
     const int n2 = A.n2, n2w = n2 + (n2 & 1), BW = (n2 + V - 1) / V * V;
     if (tid < A.nprobe) {
-      const int pq1 = A.probe_q[3 * tid], pq3 = A.probe_q[3 * tid + 2];
-      if (pq1 >= y0 && pq1 < y0 + BYm && pq3 >= z0 && pq3 < z1) probe_list[atomicAdd(&probe_cnt, 1)] = tid;
+      const int pq1 = A.probe_q[3 * tid], pq2 = A.probe_q[3 * tid + 1], pq3 = A.probe_q[3 * tid + 2];
+      if (pq1 >= y0 && pq1 < y0 + BYm && pq3 >= z0 && pq3 < z1) probes.add(tid, pq1, pq2, pq3);
     }
     __syncthreads();
     const CUtensorMap* tm_f = maps + 3 * item.member + src;
@@ -783,9 +781,7 @@ __global__ void __launch_bounds__(32 * (W + 1), sizeof(S) == 4 && W == 9 ? 2 : 1
       const unsigned wrho = (unsigned)(row * n2w * RS);
       constexpr unsigned PLANE = (unsigned)(RowTile<W>::kNodes * RS);
 
-      bool has_probe = false;
-      if (owner && t_sample < (unsigned long long)A.cap)
-        for (int s = 0; s < probe_cnt; ++s) has_probe |= A.probe_q[3 * probe_list[s]] == q1;
+      const bool has_probe = owner && t_sample < (unsigned long long)A.cap && probes.row(q1);
 
       R fA[7][NPT], fB[7][NPT], rA[NPT], rB[NPT], rC[NPT];
       const long long row_stride = (long long)A.n1 * A.pitch;
@@ -919,11 +915,11 @@ __global__ void __launch_bounds__(32 * (W + 1), sizeof(S) == 4 && W == 9 ? 2 : 1
           else VecN<S, NPT>::st(dst, fc[i]);
           dst += A.ps;
         }
-        if (has_probe) {
-          for (int s = 0; s < probe_cnt; ++s) {
-            const int k = probe_list[s];
-            const int dq = A.probe_q[3 * k + 1] - col;
-            if (A.probe_q[3 * k] == q1 && dq >= 0 && dq < NPT && col + dq < n2 && A.probe_q[3 * k + 2] == zc)
+        if (has_probe && probes.plane(zc)) {
+          for (int s = 0; s < probes.count; ++s) {
+            const int k = probes.id[s];
+            const int dq = probes.at[3 * s + 1] - col;
+            if (probes.at[3 * s] == q1 && dq >= 0 && dq < NPT && col + dq < n2 && probes.at[3 * s + 2] == zc)
               A.series[(long long)k * A.cap + t_sample] = (double)(dq == 0 ? rc[0] : rc[1]) * (double)c[T_INVSG];
           }
         }
@@ -1335,8 +1331,8 @@ lbw_status list_items(const lbw_batch* b, const Shape& shape, std::vector<BatchI
 // claim the items in order: an item costs its planes and some four more to fill the pipeline, a
 // plane as measured at two CTAs per SM (us: full-row tile 1.0, 7 rows of 64 columns 1.25, 4 rows
 // 0.9; the tall full-row tile, alone on its SM, 1.1: choices the same from 1.0 to 1.2).  A single
-// lattice has few items, so it also tries the lengths that divide its planes evenly and the tall
-// form; an ensemble's tail is cut (list_items) and DRAM bounds it in either form.
+// lattice has few items, so its full-row tiles also try the lengths that divide its planes evenly
+// and the tall form; an ensemble's tail is cut (list_items) and DRAM bounds it in either form.
 Shape best_shape(const lbw_batch* b, const std::vector<int>& bys) {
   Shape best = b->shape;
   double best_cost = 1e300;
@@ -1349,13 +1345,14 @@ Shape best_shape(const lbw_batch* b, const std::vector<int>& bys) {
     forms.push_back({by, std::min(2, tma_cps(b->prec, by))});
     if (b->n == 1 && by == 0 && tall_rows(es_of(b->prec), 1)) forms.push_back({0, 1});
   }
-  std::vector<int> lzs = {64, 48, 32, 24, 16, 12, 8};
+  const std::vector<int> lengths = {64, 48, 32, 24, 16, 12, 8};
+  std::vector<int> even = lengths;
   if (b->n == 1) {
     const int n3 = b->views[0].d.n[2];
-    for (int segs = 1; segs <= 32 && n3 / segs >= 8; ++segs) lzs.push_back((n3 + segs - 1) / segs);
+    for (int segs = 1; segs <= 32 && n3 / segs >= 8; ++segs) even.push_back((n3 + segs - 1) / segs);
   }
   for (const auto [by, cps] : forms) {
-    for (const int lz : lzs) {
+    for (const int lz : by == 0 ? even : lengths) {
       const Shape shape{by, lz, cps};
       if (shape.cps < 1 || list_items(b, shape, items) != LBW_OK) continue;
       const double plane = by == 0 ? (tall_rows(es_of(b->prec), cps) ? 1.1 : 1.0) : by == 7 ? 1.25 : 0.9;

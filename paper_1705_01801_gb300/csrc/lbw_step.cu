@@ -143,8 +143,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
   constexpr int TABB = ((BY * T_SLOTS * RS) + 127) / 128 * 128;
   constexpr int RHOB = ((2 * PS * RS) + 127) / 128 * 128;  // two rho planes
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int probe_list[kMaxProbes];
-  __shared__ int probe_cnt;
+  __shared__ TileProbes probes;
   __shared__ int abort_flag;
   __shared__ int stall_req;
   __shared__ unsigned long long t_sample;
@@ -186,7 +185,8 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
     }
     mbar_init_count(stall_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    probe_cnt = 0;
+    probes.count = 0;
+    for (unsigned& p : probes.planes) p = 0;
     abort_flag = 0;
     stall_req = a.counters[4] != 0ull;  // failure injection (lbw_inject_wait_timeout)
     t_sample = a.counters[1];
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
   if (tid < a.nprobe) {
     const int pq1 = a.probe_q[3 * tid], pq2 = a.probe_q[3 * tid + 1], pq3 = a.probe_q[3 * tid + 2];
     if (pq1 >= y0 && pq1 < y0 + BY && pq2 >= x0 && pq2 < x0 + BX && pq3 >= z0 && pq3 < z1)
-      probe_list[atomicAdd(&probe_cnt, 1)] = tid;
+      probes.add(tid, pq1, pq2, pq3);
   }
   __syncthreads();
 
@@ -507,9 +507,7 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
     const unsigned myrho = (unsigned)((w * PW + C0 + c0) * RS);
 
     // probes of this warp's row (recorded while the sample counter is below capacity)
-    bool has_probe = false;
-    if (owner && t_sample < (unsigned long long)a.cap)
-      for (int s = 0; s < probe_cnt; ++s) has_probe |= a.probe_q[3 * probe_list[s]] == q1;
+    const bool has_probe = owner && t_sample < (unsigned long long)a.cap && probes.row(q1);
 
     R fA[7][NPT], fB[7][NPT], rA[NPT], rB[NPT], rC[NPT];
     const long long n12 = (long long)a.n1 * a.n2;
@@ -718,11 +716,11 @@ __global__ void __launch_bounds__(32 * (BY + 3)) step_tma_kernel(
         VecN<S, NPT>::st(dst, fc[i]);
         dst += a.nn;
       }
-      if (has_probe) {
-        for (int s = 0; s < probe_cnt; ++s) {
-          const int k = probe_list[s];
-          const int dq = a.probe_q[3 * k + 1] - q2;
-          if (a.probe_q[3 * k] == q1 && dq >= 0 && dq < NPT && a.probe_q[3 * k + 2] == zc) {
+      if (has_probe && probes.plane(zc)) {
+        for (int s = 0; s < probes.count; ++s) {
+          const int k = probes.id[s];
+          const int dq = probes.at[3 * s + 1] - q2;
+          if (probes.at[3 * s] == q1 && dq >= 0 && dq < NPT && probes.at[3 * s + 2] == zc) {
             R v = rc[0];
 #pragma unroll
             for (int j = 1; j < NPT; ++j) v = dq == j ? rc[j] : v;

@@ -53,3 +53,39 @@ def test_one_step(name):
     np.testing.assert_allclose(g.get_f(), fo, rtol=RTOL[spec.prec], atol=1e-6 * np.abs(fo).max())
     g.close()
     o.close()
+
+
+@pytest.mark.parametrize("n2", [64, 40], ids=["tile", "full-row"])
+def test_many_probes_of_a_tile(n2):
+    """64 probes in the tile and ensemble kernels: several in a plane, planes 256 apart, both ends
+    of a row, every row; FP32 as in the other parity tests (2e-5, probes ten times that)."""
+    from paper_1705_01801_gb300 import lbw
+    spec = W.GridSpec(kind=W.KIND_CARTESIAN, n=(9, n2, 600), bc=(1, 2, 0, 0, 3, 1), prec=W.PREC_F32, **BOX)
+    q = np.array([[k % 9, (0, n2 - 1, 17, 18)[k % 4], (3, 259, 515, 599)[k // 16] - (k % 3 == 0)] for k in range(64)])
+    o = oracle.OracleGrid(spec)
+    o.init(W.pulses(spec, 5, 4))
+    o.set_probes(q, 8)
+    o.step(10)
+    so, fmax = o.read_probes(), np.abs(o.get_f()).max()
+    o.close()
+    if n2 == 64:
+        g = lbw.Grid(spec.with_(geom_mode=1))
+        g.init(W.pulses(spec, 5, 4))
+        g.set_probes(q, 8)
+        g.step(10)
+        series = [g.read_probes()]
+        g.close()
+    else:
+        b = lbw.Batch([spec, spec])
+        b.init([W.pulses(spec, 5, 4)] * 2)
+        b.set_probes(np.stack([q, q]), 8)
+        series = []
+        for cps in (1, 2):
+            b.init([W.pulses(spec, 5, 4)] * 2)
+            b.set_shape(0, 300, cps)
+            b.step(10)
+            series += list(b.read_probes())
+        b.close()
+    for s in series:
+        assert np.asarray(s).shape == np.asarray(so).shape
+        np.testing.assert_allclose(s, so, rtol=0, atol=2e-4 * fmax)
