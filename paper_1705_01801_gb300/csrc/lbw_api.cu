@@ -24,6 +24,9 @@ lbw_status fail(lbw_status s, const std::string& msg) {
 
 lbw_status cuda_fail(cudaError_t e, const char* what) {
   g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
+  // reported here: left as the runtime's last error, a failed allocation would be read back as the
+  // failure of the next call that launches a kernel
+  (void)cudaGetLastError();
   return LBW_ECUDA;
 }
 

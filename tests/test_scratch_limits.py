@@ -1,0 +1,71 @@
+"""What is launched after an allocation or a launch has failed, on a fake CUDA runtime (tests/host):
+every pointer that the next launch of a step kernel is given has to be a live allocation.  No GPU."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import lbw_workloads as W
+from host import load
+
+SMALL = W.cylinder(20, 33, 10)           # on the multi-step kernel
+RAGGED = W.cylinder(100, 100, 70)        # on the ensemble kernels, as a single lattice
+TILED = W.cylinder(20, 64, 10).with_(geom_mode=W.GEOM_TABLE)
+
+
+@pytest.fixture(scope="module")
+def fake():
+    return load()
+
+
+@pytest.fixture(autouse=True)
+def _reset(fake):
+    yield
+    L = fake.lib()
+    L.fake_fail_allocation(0)
+    L.fake_largest_allocation(2 ** 63)
+    L.fake_fail_launch(b"")
+    L.fake_errors()
+
+
+def _until_it_succeeds(fake, call, after):
+    """`call` with its first, second, ... allocation failing until none is left to fail; `after` runs
+    behind each failure."""
+    for n in range(1, 50):
+        fake.lib().fake_fail_allocation(n)
+        try:
+            call()
+        except fake.LbwError:
+            failed = True
+        else:
+            failed = False
+        fake.lib().fake_fail_allocation(0)
+        after()
+        assert fake.lib().fake_errors() == b"", n
+        if not failed:
+            return n
+    raise AssertionError("the call never succeeded")
+
+
+def _grid(fake, spec):
+    g = fake.Grid(spec)
+    g.init(W.pulses(spec, 1, 1, margin=0))
+    return g
+
+
+def _batch(fake, specs):
+    b = fake.Batch(specs)
+    b.init([W.pulses(s, 1, 1, margin=0) for s in specs])
+    return b
+
+
+@pytest.mark.parametrize("spec", [SMALL, TILED], ids=["small", "tiled"])
+def test_a_failed_allocation_is_no_later_calls_error(fake, spec):
+    """The runtime hands a failed allocation's error to the next look at its last error, which every
+    launch takes: the call that failed clears it."""
+    g = _grid(fake, spec)
+    fake.lib().fake_fail_allocation(1)
+    with pytest.raises(fake.LbwError):
+        g.set_sources([[1, 1, 1]])
+    g.init(W.pulses(spec, 1, 1, margin=0))
+    g.close()
