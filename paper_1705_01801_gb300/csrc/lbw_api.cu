@@ -506,8 +506,17 @@ lbw_status lbw_source(lbw_grid* g, const int32_t* host_q, int32_t n, int32_t kin
     equilibrium_coefs(g->d, &h[k].cs2, &eq_two0);  // the equilibrium the source imposes
   }
   drop_graphs(g);  // captured chains carry the source list
-  if (g->src) { cudaFreeAsync(g->src, g->stream); g->src = nullptr; }
-  g->nsrc = 0;
+  // the boxes of the multi-step kernel let go of the old list before it is freed
+  if (g->res && g->nsrc > 0) {
+    const lbw_status st = resident_sources(g->res, nullptr, 0, g->stream);
+    if (st != LBW_OK) return st;
+  }
+  auto drop = [&]() {
+    if (g->src) cudaFreeAsync(g->src, g->stream);
+    g->src = nullptr;
+    g->nsrc = 0;
+  };
+  drop();
   if (n > 0) {
     LBW_CUDA(cudaMallocAsync(&g->src, sizeof(SourceEntry) * n, g->stream));
     LBW_CUDA(cudaMemcpyAsync(g->src, h.data(), sizeof(SourceEntry) * n, cudaMemcpyHostToDevice, g->stream));
@@ -515,8 +524,11 @@ lbw_status lbw_source(lbw_grid* g, const int32_t* host_q, int32_t n, int32_t kin
     g->nsrc = n;
     g->src_kind = kind;
     g->src_amp = amp;
+    const lbw_status st = g->res ? resident_sources(g->res, host_q, n, g->stream) : LBW_OK;
+    if (st != LBW_OK) drop();
+    return st;
   }
-  return g->res ? resident_sources(g->res, host_q, g->nsrc, g->stream) : LBW_OK;
+  return LBW_OK;
 }
 
 lbw_status lbw_probe(lbw_grid* g, const int32_t* host_q, int32_t n, int64_t capacity) {

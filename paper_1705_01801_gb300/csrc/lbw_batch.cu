@@ -1179,7 +1179,8 @@ int padded_pitch(int n2, size_t es) {
   return (n2 + 2 * ghost_cols(es) + v - 1) / v * v;
 }
 
-// The device list of the harmonic sources in the members' present storage layout.
+// The device list of the harmonic sources in the members' present storage layout, and their boxes of
+// the multi-step kernel (which let go of the old list before it is freed).  On failure there are none.
 lbw_status build_sources(lbw_batch* b) {
   std::vector<SourceEntry> h;
   const size_t per = b->src_q.size() / 3 / b->n;
@@ -1201,15 +1202,28 @@ lbw_status build_sources(lbw_batch* b) {
     }
   }
   drop_graphs(b);  // captured chains carry the source list
+  if (b->res && b->nsrc > 0) {
+    const lbw_status st = resident_sources(b->res, nullptr, 0, b->stream);
+    if (st != LBW_OK) return st;
+  }
   if (b->src) { cudaFreeAsync(b->src, b->stream); b->src = nullptr; }
   b->nsrc = 0;
-  if (!h.empty()) {
-    LBW_CUDA(cudaMallocAsync((void**)&b->src, sizeof(SourceEntry) * h.size(), b->stream));
-    LBW_CUDA(cudaMemcpyAsync(b->src, h.data(), sizeof(SourceEntry) * h.size(), cudaMemcpyHostToDevice, b->stream));
-    LBW_CUDA(cudaStreamSynchronize(b->stream));
-    b->nsrc = (int)h.size();
-  }
-  return LBW_OK;
+  if (h.empty()) return LBW_OK;
+  auto none = [&](lbw_status st) {
+    if (b->src) { cudaFreeAsync(b->src, b->stream); b->src = nullptr; }
+    b->nsrc = 0;
+    b->src_q.clear();
+    b->src_omega.clear();
+    return st;
+  };
+  cudaError_t e = cudaMallocAsync(&b->src, sizeof(SourceEntry) * h.size(), b->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->src, h.data(), sizeof(SourceEntry) * h.size(), cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  if (e != cudaSuccess) return none(cuda_fail(e, "source list"));
+  b->nsrc = (int)h.size();
+  const lbw_status st = b->res ? resident_sources(b->res, b->src_q.data(), (int)per, b->stream) : LBW_OK;
+  return st == LBW_OK ? st : none(st);
 }
 
 // Rows as the full-row kernel stores them: no ghost columns, n2 rounded up to 16 bytes.  Ghost
@@ -1783,9 +1797,7 @@ lbw_status lbw_batch_source(lbw_batch* b, const int32_t* host_q, int32_t per_mem
   b->src_omega.assign(host_omega, host_omega + (per_member > 0 ? b->n : 0));
   b->src_kind = kind;
   b->src_amp = amp;
-  const lbw_status st = build_sources(b);
-  if (st != LBW_OK) return st;
-  return b->res ? resident_sources(b->res, host_q, per_member, b->stream) : LBW_OK;
+  return build_sources(b);
 }
 
 lbw_status lbw_batch_step(lbw_batch* b, int64_t n_steps) {

@@ -755,10 +755,8 @@ void resident_destroy(Resident* r, cudaStream_t stream) {
 }
 
 lbw_status resident_sources(Resident* r, const int32_t* host_q, int per_lattice, cudaStream_t stream) {
-  if (r->src_order) cudaFreeAsync(r->src_order, stream);
-  r->src_order = nullptr;
   // boxes of a lattice are regular and listed with q2 fastest, then q1, then q3
-  std::vector<ResItem>& items = r->host_items;
+  std::vector<ResItem> items = r->host_items;
   std::vector<int> box_of, first_of, nx_of, ny_of;
   for (size_t k = 0; k < items.size(); ++k) {
     const ResItem& it = items[k];
@@ -787,12 +785,16 @@ lbw_status resident_sources(Resident* r, const int32_t* host_q, int per_lattice,
   }
   std::vector<int> order(box_of.size());
   for (size_t e = 0; e < box_of.size(); ++e) order[items[box_of[e]].src_hi++] = (int)e;
+  // the new order first: where it cannot be had, the boxes stay as they are
+  int* d_order = nullptr;
   if (!order.empty()) {
-    LBW_CUDA(cudaMallocAsync((void**)&r->src_order, sizeof(int) * order.size(), stream));
-    LBW_CUDA(cudaMemcpyAsync(r->src_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, stream));
+    LBW_CUDA(cudaMallocAsync((void**)&d_order, sizeof(int) * order.size(), stream));
+    LBW_CUDA(cudaMemcpyAsync(d_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, stream));
   }
-  LBW_CUDA(cudaMemcpyAsync(r->items, r->host_items.data(), sizeof(ResItem) * r->host_items.size(),
-                           cudaMemcpyHostToDevice, stream));
+  LBW_CUDA(cudaMemcpyAsync(r->items, items.data(), sizeof(ResItem) * items.size(), cudaMemcpyHostToDevice, stream));
+  if (r->src_order) cudaFreeAsync(r->src_order, stream);
+  r->src_order = d_order;
+  r->host_items.swap(items);
   LBW_CUDA(cudaStreamSynchronize(stream));
   return LBW_OK;
 }

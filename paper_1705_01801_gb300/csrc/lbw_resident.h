@@ -51,7 +51,8 @@ struct ResState {
 lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool tile, long long max_nodes,
                            cudaStream_t stream, Resident** out);
 void resident_destroy(Resident* r, cudaStream_t stream);
-// Assigns the sources (per_lattice nodes of each lattice, in SourceEntry order) to the boxes.
+// Assigns the sources (per_lattice nodes of each lattice, in SourceEntry order) to the boxes; none
+// (0) before their list is freed, which needs no memory.
 lbw_status resident_sources(Resident* r, const int32_t* host_q, int per_lattice, cudaStream_t stream);
 // `steps` <= kResChunk time steps from buffer st.cur: of the lattice `one`, or of an ensemble
 // with StepArgs array `members` (source buffer 0).

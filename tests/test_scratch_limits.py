@@ -69,3 +69,24 @@ def test_a_failed_allocation_is_no_later_calls_error(fake, spec):
         g.set_sources([[1, 1, 1]])
     g.init(W.pulses(spec, 1, 1, margin=0))
     g.close()
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("spec", [SMALL, RAGGED, TILED], ids=["small", "ragged", "tiled"])
+def test_sources_after_a_failed_allocation(fake, spec, kind):
+    g = _grid(fake, spec)
+    nodes = [[1, j, 2] for j in range(30)]
+    g.set_sources(nodes, kind)
+    assert _until_it_succeeds(fake, lambda: g.set_sources(nodes[:9], kind), lambda: g.step(3)) > 1
+    g.close()
+    assert fake.lib().fake_errors() == b""
+
+
+@pytest.mark.parametrize("specs", [[SMALL] * 3, [RAGGED] * 2], ids=["small", "large"])
+def test_ensemble_sources_after_a_failed_allocation(fake, specs):
+    b = _batch(fake, specs)
+    nodes = np.array([[[1, j, 2] for j in range(30)]] * len(specs))
+    b.set_sources(nodes, np.ones(len(specs)))
+    assert _until_it_succeeds(fake, lambda: b.set_sources(nodes[:, :9], np.ones(len(specs))), lambda: b.step(3)) > 1
+    b.close()
+    assert fake.lib().fake_errors() == b""
