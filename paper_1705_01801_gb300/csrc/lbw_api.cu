@@ -545,19 +545,22 @@ lbw_status lbw_probe(lbw_grid* g, const int32_t* host_q, int32_t n, int64_t capa
   drop_graphs(g);  // the captured launches carry the probe pointers
   g->nprobe = 0;
   g->cap = 0;
+  cudaError_t e = cudaSuccess;
   if (n > 0) {
-    LBW_CUDA(cudaMallocAsync((void**)&g->probe_q, sizeof(int32_t) * 3 * n, g->stream));
-    LBW_CUDA(cudaMallocAsync((void**)&g->series, sizeof(double) * n * capacity, g->stream));
-    LBW_CUDA(cudaMemcpyAsync(g->probe_q, host_q, sizeof(int32_t) * 3 * n, cudaMemcpyHostToDevice,
-                             g->stream));
-    LBW_CUDA(cudaMemsetAsync(g->series, 0, sizeof(double) * n * capacity, g->stream));
-    g->nprobe = n;
-    g->cap = capacity;
+    e = cudaMallocAsync((void**)&g->probe_q, sizeof(int32_t) * 3 * n, g->stream);
+    if (e == cudaSuccess) e = cudaMallocAsync((void**)&g->series, sizeof(double) * n * capacity, g->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(g->probe_q, host_q, sizeof(int32_t) * 3 * n, cudaMemcpyHostToDevice, g->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(g->series, 0, sizeof(double) * n * capacity, g->stream);
+    if (e == cudaSuccess) {
+      g->nprobe = n;
+      g->cap = capacity;
+    }
   }
-  if (g->ragged) {
-    const lbw_status st = ragged_refresh(g);
-    if (st != LBW_OK) return st;
-  }
+  // a ragged lattice's launch arguments are on the device: also a failure takes the old probes from them
+  const lbw_status st = g->ragged ? ragged_refresh(g) : LBW_OK;
+  if (e != cudaSuccess) return cuda_fail(e, "probe series");
+  if (st != LBW_OK) return st;
   // restart the sample counter (counters[1]); the step count is kept
   LBW_CUDA(cudaMemsetAsync(g->counters + 1, 0, sizeof(unsigned long long), g->stream));
   LBW_CUDA(cudaStreamSynchronize(g->stream));

@@ -1761,18 +1761,25 @@ lbw_status lbw_batch_probe(lbw_batch* b, const int32_t* host_q, int32_t per_memb
   if (b->series) { cudaFreeAsync(b->series, b->stream); b->series = nullptr; }
   b->nprobe = 0;
   b->cap = 0;
+  drop_graphs(b);  // the captured launches carry the number of probes
+  cudaError_t e = cudaSuccess;
   if (per_member > 0) {
     const size_t nq = (size_t)b->n * per_member;
-    LBW_CUDA(cudaMallocAsync((void**)&b->probe_q, sizeof(int32_t) * 3 * nq, b->stream));
-    LBW_CUDA(cudaMallocAsync((void**)&b->series, sizeof(double) * nq * capacity, b->stream));
-    LBW_CUDA(cudaMemcpyAsync(b->probe_q, host_q, sizeof(int32_t) * 3 * nq, cudaMemcpyHostToDevice, b->stream));
-    LBW_CUDA(cudaMemsetAsync(b->series, 0, sizeof(double) * nq * capacity, b->stream));
-    b->nprobe = per_member;
-    b->cap = capacity;
+    e = cudaMallocAsync((void**)&b->probe_q, sizeof(int32_t) * 3 * nq, b->stream);
+    if (e == cudaSuccess) e = cudaMallocAsync((void**)&b->series, sizeof(double) * nq * capacity, b->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(b->probe_q, host_q, sizeof(int32_t) * 3 * nq, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->series, 0, sizeof(double) * nq * capacity, b->stream);
+    if (e == cudaSuccess) {
+      b->nprobe = per_member;
+      b->cap = capacity;
+    }
   }
-  LBW_CUDA(cudaMemsetAsync(b->counters + 1, 0, sizeof(unsigned long long), b->stream));
-  lbw_status st = refresh(b);
+  // the members' arguments are on the device: also a failure takes the old probes from them
+  const lbw_status st = upload_members(b);
+  if (e != cudaSuccess) return cuda_fail(e, "probe series");
   if (st != LBW_OK) return st;
+  LBW_CUDA(cudaMemsetAsync(b->counters + 1, 0, sizeof(unsigned long long), b->stream));
   LBW_CUDA(cudaStreamSynchronize(b->stream));
   return LBW_OK;
 }

@@ -65,5 +65,13 @@ cudaError_t wrap_resident_run(const lbw::Resident* r, const lbw::Grid* one, cons
     fake_want_live(one->probe_q, "probe nodes");
     fake_want_live(one->series, "probe series");
   }
+  if (members) {
+    void* list = const_cast<void*>(members);
+    void* args[] = {&list, &list};  // no work list: the members stand in for it
+    if (r->prec == LBW_F64) check_ensemble<double>(args, 1);
+    else if (r->prec == LBW_F32) check_ensemble<float>(args, 1);
+    else if (r->prec == LBW_F16S) check_ensemble<__half>(args, 1);
+    else check_ensemble<__nv_bfloat16>(args, 1);
+  }
   return real_resident_run(r, one, members, st, steps);
 }

@@ -90,3 +90,24 @@ def test_ensemble_sources_after_a_failed_allocation(fake, specs):
     assert _until_it_succeeds(fake, lambda: b.set_sources(nodes[:, :9], np.ones(len(specs))), lambda: b.step(3)) > 1
     b.close()
     assert fake.lib().fake_errors() == b""
+
+
+@pytest.mark.parametrize("spec", [SMALL, RAGGED, TILED], ids=["small", "ragged", "tiled"])
+def test_probes_after_a_failed_allocation(fake, spec):
+    g = _grid(fake, spec)
+    g.set_probes([[1, 1, 1]] * 4, 100)
+    assert _until_it_succeeds(fake, lambda: g.set_probes([[2, 2, 2]] * 3, 50), lambda: g.step(3)) > 1
+    g.close()
+    assert fake.lib().fake_errors() == b""
+
+
+@pytest.mark.parametrize("shape", [None, (7, 16, 2)], ids=["created", "set"])
+@pytest.mark.parametrize("specs", [[SMALL] * 3, [RAGGED] * 2], ids=["small", "large"])
+def test_ensemble_probes_after_a_failed_allocation(fake, specs, shape):
+    b = _batch(fake, specs)
+    if shape:
+        b.set_shape(*shape)
+    b.set_probes([[[1, 1, 1]] * 4] * len(specs), 100)
+    assert _until_it_succeeds(fake, lambda: b.set_probes([[[2, 2, 2]] * 3] * len(specs), 50), lambda: b.step(3)) > 1
+    b.close()
+    assert fake.lib().fake_errors() == b""
