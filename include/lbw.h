@@ -255,7 +255,9 @@ lbw_status lbw_batch_init(lbw_batch* b, const lbw_pulse* host_pulses, const int3
  * samples each.  Resets the series. */
 lbw_status lbw_batch_probe(lbw_batch* b, const int32_t* host_q, int32_t per_member, int64_t capacity);
 
-/* Advance every member by n_steps (asynchronous on the ensemble's stream). */
+/* Advance every member by n_steps (asynchronous on the ensemble's stream).  LBW_ESTATE before
+ * lbw_batch_init, and where a change of launch shape has failed and the former one could not be
+ * set again. */
 lbw_status lbw_batch_step(lbw_batch* b, int64_t n_steps);
 
 /* Harmonic sources for every member (see lbw_source): per_member nodes each, host_q =

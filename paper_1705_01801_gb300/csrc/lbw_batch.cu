@@ -1049,6 +1049,7 @@ struct lbw_batch {
   BatchItem* items = nullptr;
   int n_items = 0, blocks = 0;
   Shape shape;
+  bool ready = false;  // work list, tensor maps and arguments on the device are those of `shape`
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   int graph_len = 0, cur = 0;
   int64_t steps = 0;
@@ -1394,9 +1395,10 @@ lbw_status build_items(lbw_batch* b) {
   std::vector<BatchItem> items;
   const lbw_status st = list_items(b, b->shape, items);
   if (st != LBW_OK) return st;
+  BatchItem* list = nullptr;
+  LBW_CUDA(cudaMallocAsync((void**)&list, sizeof(BatchItem) * items.size(), b->stream));
   if (b->items) cudaFreeAsync(b->items, b->stream);
-  b->items = nullptr;
-  LBW_CUDA(cudaMallocAsync((void**)&b->items, sizeof(BatchItem) * items.size(), b->stream));
+  b->items = list;
   LBW_CUDA(cudaMemcpyAsync(b->items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice,
                            b->stream));
   b->n_items = (int)items.size();
@@ -1410,14 +1412,13 @@ lbw_status upload_members(lbw_batch* b) {
 }
 
 lbw_status refresh(lbw_batch* b, bool rebuild_ghosts = false) {
+  b->ready = false;
   lbw_status st = use_layout(b, rebuild_ghosts);
   if (st == LBW_OK) st = build_items(b);
-  if (st != LBW_OK) return st;
-  if (b->tma) {
-    st = build_batch_maps(b, b->shape);
-    if (st != LBW_OK) return st;
-  }
-  return upload_members(b);
+  if (st == LBW_OK && b->tma) st = build_batch_maps(b, b->shape);
+  if (st == LBW_OK) st = upload_members(b);
+  b->ready = st == LBW_OK;
+  return st;
 }
 
 template <typename S>
@@ -1504,6 +1505,8 @@ cudaError_t run_resident(lbw_batch* b, int n) {
 }
 
 lbw_status advance(lbw_batch* b, int64_t n_steps) {
+  if (!b->ready)
+    return fail(LBW_ESTATE, "the ensemble's last change of launch shape failed; lbw_batch_set_shape sets one");
   const int chain = 64;
   int64_t left = n_steps;
   while (b->res && left > 0) {
@@ -1923,55 +1926,77 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
     cudaEvent_t e0, e1;
     LBW_CUDA(cudaEventCreate(&e0));
     LBW_CUDA(cudaEventCreate(&e1));
-    for (int by : bys)
-      for (int lz : lzs)
-        for (int cps : cpss) {
-          const int cps_max = b->tma ? tma_cps(b->prec, by) : (b->prec == LBW_F32 ? max_cps<float>() : 2);
-          if (cps > cps_max) continue;
-          b->shape = Shape{by, lz, cps};
-          lbw_status st = refresh(b);
-          if (st != LBW_OK) return st;
-          for (int w = 0; w < 2; ++w) {  // warm-up
-            LBW_CUDA(launch_batch(b, b->cur));
-            b->cur = 1 - b->cur;
-          }
-          LBW_CUDA(cudaEventRecord(e0, b->stream));
-          for (int s = 0; s < trial_steps; ++s) {
-            LBW_CUDA(launch_batch(b, b->cur));
-            b->cur = 1 - b->cur;
-          }
-          LBW_CUDA(cudaEventRecord(e1, b->stream));
-          LBW_CUDA(cudaEventSynchronize(e1));
-          float ms = 0.f;
-          LBW_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-          ms /= trial_steps;
-          rep << "by=" << by << " lz=" << lz << " cps=" << cps << " ms=" << ms << "\n";
-          if (best_ms < 0 || ms < best_ms) {
-            best_ms = ms;
-            best = b->shape;
-          }
-        }
-    if (b->res) {  // against the kernel that small members start with
-      b->shape = start;
-      lbw_status st = refresh(b);
-      if (st != LBW_OK) return st;
-      LBW_CUDA(run_resident(b, 2));  // warm-up
+    // ms per step of what `run(n)` launches for n steps, after two warm-up steps
+    auto timed = [&](auto&& run, float* ms) -> lbw_status {
+      LBW_CUDA(run(2));
       LBW_CUDA(cudaEventRecord(e0, b->stream));
-      for (int s = 0; s < trial_steps; s += kResChunk) LBW_CUDA(run_resident(b, std::min(kResChunk, trial_steps - s)));
+      LBW_CUDA(run(trial_steps));
       LBW_CUDA(cudaEventRecord(e1, b->stream));
       LBW_CUDA(cudaEventSynchronize(e1));
+      LBW_CUDA(cudaEventElapsedTime(ms, e0, e1));
+      *ms /= trial_steps;
+      return LBW_OK;
+    };
+    auto try_shape = [&](const Shape& shape) -> lbw_status {
+      b->shape = shape;
+      lbw_status st = refresh(b);
+      if (st != LBW_OK) return st;
       float ms = 0.f;
-      LBW_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      ms /= trial_steps;
+      st = timed(
+          [&](int n) {
+            cudaError_t e = cudaSuccess;
+            for (int s = 0; s < n && e == cudaSuccess; ++s) {
+              e = launch_batch(b, b->cur);
+              b->cur = 1 - b->cur;
+            }
+            return e;
+          },
+          &ms);
+      if (st != LBW_OK) return st;
+      rep << "by=" << shape.by << " lz=" << shape.lz << " cps=" << shape.cps << " ms=" << ms << "\n";
+      if (best_ms < 0 || ms < best_ms) {
+        best_ms = ms;
+        best = shape;
+      }
+      return LBW_OK;
+    };
+    auto try_resident = [&]() -> lbw_status {  // the kernel that small members start with
+      b->shape = start;
+      lbw_status st = refresh(b);
+      float ms = 0.f;
+      if (st == LBW_OK)
+        st = timed(
+            [&](int n) {
+              cudaError_t e = cudaSuccess;
+              for (int s = 0; s < n && e == cudaSuccess; s += kResChunk) e = run_resident(b, std::min(kResChunk, n - s));
+              return e;
+            },
+            &ms);
+      if (st != LBW_OK) return st;
       rep << "resident ms=" << ms << "\n";
       resident = ms < best_ms;
       if (resident) {
         best_ms = ms;
         best = start;
       }
-    }
+      return LBW_OK;
+    };
+    lbw_status st = LBW_OK;
+    for (int by : bys)
+      for (int lz : lzs)
+        for (int cps : cpss) {
+          const int cps_max = b->tma ? tma_cps(b->prec, by) : (b->prec == LBW_F32 ? max_cps<float>() : 2);
+          if (st == LBW_OK && cps <= cps_max) st = try_shape(Shape{by, lz, cps});
+        }
+    if (st == LBW_OK && b->res) st = try_resident();
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    if (st != LBW_OK) {  // back to the shape it had
+      const std::string why = lbw_last_error();
+      b->shape = start;
+      refresh(b, b->res != nullptr);
+      return fail(st, why);
+    }
     if (cache_path) {
       std::ofstream o(cache_path, std::ios::app);
       o << "{\"signature\": \"" << sig << "\", \"by\": " << best.by << ", \"lz\": " << best.lz
@@ -1979,13 +2004,12 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
     }
   }
   b->shape = best;
-  const bool was_resident = b->res != nullptr && !resident;
+  lbw_status st = refresh(b, b->res != nullptr && !resident);
+  if (st != LBW_OK) return st;
   if (!resident) {
     resident_destroy(b->res, b->stream);
     b->res = nullptr;
   }
-  lbw_status st = refresh(b, was_resident);
-  if (st != LBW_OK) return st;
   // trial steps ran on the ensemble's buffers: callers tune before lbw_batch_init
   LBW_CUDA(cudaMemsetAsync(b->counters, 0, 4 * sizeof(unsigned long long), b->stream));
   LBW_CUDA(cudaStreamSynchronize(b->stream));
@@ -2009,17 +2033,17 @@ lbw_status lbw_batch_set_shape(lbw_batch* b, int32_t tile_rows, int32_t seg_plan
   if (ctas_per_sm < 1 || ctas_per_sm > std::max(1, cps_max) || (b->tma && cps_max == 0))
     return fail(LBW_EINVAL, "ctas_per_sm must be in [1, what the kernel keeps resident]");
   const Shape old = b->shape;
-  // a shape chosen by the caller is one of the tiled kernels'
-  const bool was_resident = b->res != nullptr;
-  resident_destroy(b->res, b->stream);
-  b->res = nullptr;
   b->shape = Shape{tile_rows, seg_planes, ctas_per_sm};
-  lbw_status st = refresh(b, was_resident);
+  lbw_status st = refresh(b, b->res != nullptr);
   if (st != LBW_OK) {
+    const std::string why = lbw_last_error();
     b->shape = old;
     refresh(b);
-    return st;
+    return fail(st, why);
   }
+  // a shape chosen by the caller is one of the tiled kernels'
+  resident_destroy(b->res, b->stream);
+  b->res = nullptr;
   LBW_CUDA(cudaStreamSynchronize(b->stream));
   return LBW_OK;
 }

@@ -21,7 +21,7 @@ std::map<uintptr_t, Block> g_blocks;             // freed blocks stay mapped, ma
 std::map<const void*, std::string> g_kernels;    // host stub -> mangled kernel name
 std::map<std::string, int> g_launches;
 std::vector<std::string> g_errors;
-int g_fail_alloc = 0;        // the n-th allocation from now fails
+int g_fail_alloc = 0;         // the n-th allocation from now fails (-n: and all behind it)
 size_t g_largest = SIZE_MAX;  // larger allocations fail
 std::string g_fail_launch;   // launches of kernels whose name holds this fail
 cudaError_t g_last = cudaSuccess;
@@ -89,7 +89,11 @@ const char* fake_errors() {
 }
 
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) {
-  if ((g_fail_alloc > 0 && --g_fail_alloc == 0) || n > g_largest) return g_last = cudaErrorMemoryAllocation;
+  bool fails = false;
+  if (g_fail_alloc > 0) fails = --g_fail_alloc == 0;
+  else if (g_fail_alloc == -1) fails = true;
+  else if (g_fail_alloc < 0) ++g_fail_alloc;
+  if (fails || n > g_largest) return g_last = cudaErrorMemoryAllocation;
   const size_t size = n ? n : 1;
   *p = std::calloc(1, size);
   g_blocks[reinterpret_cast<uintptr_t>(*p)] = Block{size, true};

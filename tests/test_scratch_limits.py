@@ -28,11 +28,11 @@ def _reset(fake):
     L.fake_errors()
 
 
-def _until_it_succeeds(fake, call, after):
-    """`call` with its first, second, ... allocation failing until none is left to fail; `after` runs
-    behind each failure."""
+def _until_it_succeeds(fake, call, after, all_behind=False):
+    """`call` with its first, second, ... allocation failing (and all behind it) until none is left to
+    fail; `after` runs behind each failure."""
     for n in range(1, 50):
-        fake.lib().fake_fail_allocation(n)
+        fake.lib().fake_fail_allocation(-n if all_behind else n)
         try:
             call()
         except fake.LbwError:
@@ -109,5 +109,31 @@ def test_ensemble_probes_after_a_failed_allocation(fake, specs, shape):
         b.set_shape(*shape)
     b.set_probes([[[1, 1, 1]] * 4] * len(specs), 100)
     assert _until_it_succeeds(fake, lambda: b.set_probes([[[2, 2, 2]] * 3] * len(specs), 50), lambda: b.step(3)) > 1
+    b.close()
+    assert fake.lib().fake_errors() == b""
+
+
+@pytest.mark.parametrize("all_behind", [False, True], ids=["one", "all"])
+@pytest.mark.parametrize("call", [lambda b: b.set_shape(7, 16, 2), lambda b: b.set_shape(0, 16, 2),
+                                  lambda b: b.tune(1)], ids=["columns", "rows", "tune"])
+@pytest.mark.parametrize("specs", [[SMALL] * 3, [RAGGED] * 2], ids=["small", "large"])
+def test_ensemble_shapes_after_a_failed_allocation(fake, specs, call, all_behind):
+    """A change of shape that fails leaves the last one, or an ensemble that refuses to step."""
+    b = _batch(fake, specs)
+    b.set_sources([[[1, j, 2] for j in range(30)]] * len(specs), np.ones(len(specs)))
+    before, refused = b.info(), []
+
+    def after():
+        try:
+            b.step(3)
+        except fake.LbwError as e:
+            refused.append(e.status)
+        else:
+            assert refused or fake.lib().fake_launches(b"kernel") > 0
+
+    assert _until_it_succeeds(fake, lambda: call(b), after, all_behind) > 1
+    assert set(refused) <= {fake.LBW_ESTATE}
+    assert before["nodes"] == b.info()["nodes"]
+    b.step(3)  # the change that went through
     b.close()
     assert fake.lib().fake_errors() == b""
