@@ -414,7 +414,7 @@ lbw_status lbw_init(lbw_grid* g, const lbw_pulse* host_pulses, int32_t n_pulses)
     if (!(host_pulses[k].sigma > 0)) return fail(LBW_EINVAL, "pulse sigma must be > 0");
   unsigned char* d_p = nullptr;
   const size_t pb = pulse_bytes(n_pulses);
-  LBW_CUDA(cudaMallocAsync((void**)&d_p, pb + init_scratch_bytes(g->d), g->stream));
+  LBW_CUDA(cudaMallocAsync((void**)&d_p, pb + init_scratch_bytes(*g), g->stream));
   std::vector<unsigned char> hp(pb);
   pack_pulses(host_pulses, n_pulses, hp.data());
   cudaError_t e = cudaMemcpyAsync(d_p, hp.data(), pb, cudaMemcpyHostToDevice, g->stream);

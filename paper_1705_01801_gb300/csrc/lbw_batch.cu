@@ -1723,7 +1723,7 @@ lbw_status lbw_batch_init(lbw_batch* b, const lbw_pulse* host_pulses, const int3
   for (int m = 0; m < b->n; ++m) {
     if (host_counts[m] < 0) return fail(LBW_EINVAL, "negative pulse count");
     total += host_counts[m];
-    scratch = std::max(scratch, init_scratch_bytes(b->views[m].d));  // one member's at a time
+    scratch = std::max(scratch, init_scratch_bytes(b->views[m]));  // one member's at a time
   }
   if (total > 0 && !host_pulses) return fail(LBW_EINVAL, "host_pulses is NULL");
   for (size_t k = 0; k < total; ++k)

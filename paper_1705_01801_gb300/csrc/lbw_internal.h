@@ -152,8 +152,9 @@ bool encode_tiled_map(void* map, int prec, int rank, void* base, const uint64_t*
                       const uint64_t* strides, const uint32_t* box);
 
 // state (lbw_state.cu) -----------------------------------------------------------------------
-// Initial state of buffer g->cur from packed pulses and scratch on the device (enqueued)
-size_t init_scratch_bytes(const lbw_grid_desc& d);
+// Initial state of buffer g->cur from packed pulses and scratch on the device (enqueued); most
+// lattices need no scratch (0), the other population buffer holds it
+size_t init_scratch_bytes(const Grid& g);
 size_t pulse_bytes(int n);
 void pack_pulses(const lbw_pulse* p, int n, void* out);
 cudaError_t launch_init(Grid* g, const void* d_pulses, int npulse, void* d_scratch);

@@ -54,56 +54,115 @@ struct Pulse {
   double x[3], sigma, amp, axis, cut;
 };
 
-// Scratch of one initialisation: cos and sin along q2 (u2 and nothing for Cartesian lattices), per
-// q3 the flare (or cos u3), u3 (or sin u3), one byte per row: some pulse reaches it.
+// Scratch of one initialisation: cos and sin along q2 (unused on Cartesian lattices), per q3
+// the flare (or cos u3), u3 (or sin u3), one byte per row: some pulse reaches it.
 struct InitScratch {
   double *c2, *s2, *a3, *b3;
   unsigned char* near;
 };
 
-__host__ __device__ inline InitScratch carve_init(void* base, int n1, int n2, int n3) {
+inline InitScratch carve_init(void* base, int n2, int n3) {
   InitScratch s;
   s.c2 = static_cast<double*>(base);
   s.s2 = s.c2 + n2;
   s.a3 = s.s2 + n2;
   s.b3 = s.a3 + n3;
   s.near = reinterpret_cast<unsigned char*>(s.b3 + n3);
-  (void)n1;
   return s;
+}
+size_t scratch_bytes(const lbw_grid_desc& d) {
+  return sizeof(double) * 2 * ((size_t)d.n[1] + d.n[2]) + (size_t)d.n[0] * d.n[2];
+}
+size_t scratch_offset(const Grid& g) { return ((size_t)g.nn * (g.elem == 8 ? 8 : 4) + 15) / 16 * 16; }
+
+// Position of row q3's nodes along the axis: the flare (or cos u3), and u3 (or sin u3).
+__device__ __forceinline__ void plane_terms(const InitGeom& G, int q3, double& a, double& b) {
+  const double u3 = G.x0[2] + (q3 + 0.5) * G.h[2];
+  a = 1.0;
+  b = u3;
+  if (G.kind == LBW_TRUMPET) {
+    if (G.profile == 0) a = pow(G.geom[0] - u3, -G.geom[1]);
+    else a = (G.geom[0] + G.geom[1] * exp(G.geom[2] * u3)) / (G.geom[0] + G.geom[1]);
+  } else if (G.kind == LBW_TOROIDAL) {
+    sincos(u3, &b, &a);
+  }
+}
+
+__device__ __forceinline__ void column_terms(const InitGeom& G, int q2, double& c, double& s) {
+  const double u2 = G.x0[1] + (q2 + 0.5) * G.h[1];
+  s = 0.0;
+  c = u2;
+  if (G.kind != LBW_CARTESIAN) sincos(u2, &s, &c);
 }
 
 __global__ void axis_kernel(const InitGeom G, InitScratch t) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < G.n2) {
-    const double u2 = G.x0[1] + (i + 0.5) * G.h[1];
-    if (G.kind == LBW_CARTESIAN) t.c2[i] = u2;
-    else sincos(u2, &t.s2[i], &t.c2[i]);
+    if (G.kind != LBW_CARTESIAN) column_terms(G, i, t.c2[i], t.s2[i]);
   } else if (i < G.n2 + G.n3) {
-    const int q3 = i - G.n2;
-    const double u3 = G.x0[2] + (q3 + 0.5) * G.h[2];
-    double a = 1.0, b = u3;
-    if (G.kind == LBW_TRUMPET) {
-      if (G.profile == 0) a = pow(G.geom[0] - u3, -G.geom[1]);
-      else a = (G.geom[0] + G.geom[1] * exp(G.geom[2] * u3)) / (G.geom[0] + G.geom[1]);
-    } else if (G.kind == LBW_TOROIDAL) {
-      sincos(u3, &b, &a);
-    }
-    t.a3[q3] = a;
-    t.b3[q3] = b;
+    plane_terms(G, i - G.n2, t.a3[i - G.n2], t.b3[i - G.n2]);
   }
 }
 
+// What a warp takes at a time: `rows` whole rows of up to 16 nodes side by side in its lanes, or
+// `cols` columns (a multiple of 32) of one row.  Whole rows repeat the test of the pulses least
+// often, but a lattice of few rows needs their parts to fill the SMs: with a warp per row,
+// one of 1,048,576 nodes took 43 ms, 4 x 4 of 65,536 4.0, and 300,000 of three nodes 0.33; now
+// 121, 111 and 87 us (a thread per node that tests every pulse: 151, 146, 137).
+struct InitUnits {
+  int rows, cols, parts;
+  long long count;
+};
+
+InitUnits init_units(int n1, int n2, int n3) {
+  InitUnits u;
+  const long long rows = (long long)n1 * n3, warps = 152LL * 64;
+  u.rows = n2 <= 16 ? 32 / n2 : 1;
+  u.parts = u.rows > 1 ? 1 : (int)std::max(1LL, std::min<long long>((n2 + 31) / 32, warps / rows));
+  u.cols = (n2 + 32 * u.parts - 1) / (32 * u.parts) * 32;
+  u.parts = (n2 + u.cols - 1) / u.cols;
+  u.count = (rows + u.rows - 1) / u.rows * u.parts;
+  return u;
+}
+
+// A lane's place in a unit: its row (of `rows` from `first` on) and its columns c0, c0 + 32, ... below c1.
+struct InitLane {
+  long long first, row;
+  int rows, sub, c0, c1;
+  __device__ InitLane(const InitUnits& U, long long unit, long long all_rows, int n2) {
+    const int lane = threadIdx.x & 31, part = (int)(unit % U.parts);
+    first = unit / U.parts * U.rows;
+    rows = (int)min((long long)U.rows, all_rows - first);
+    sub = U.rows > 1 ? lane / n2 : 0;
+    const bool in = sub < rows;  // lanes past the unit's last row repeat its first and store nothing
+    if (!in) sub = 0;
+    row = first + sub;
+    c0 = U.rows > 1 ? (in ? lane % n2 : n2) : part * U.cols + lane;
+    c1 = U.rows > 1 ? n2 : min(n2, (part + 1) * U.cols);
+  }
+};
+
+// Adds a pulse's value at (X0, X1, z) to P0.
+__device__ __forceinline__ void add_pulse(const Pulse& p, double X0, double X1, double z, double& P0) {
+  const double d2 = (X0 - p.x[0]) * (X0 - p.x[0]) + (X1 - p.x[1]) * (X1 - p.x[1]) + (z - p.x[2]) * (z - p.x[2]);
+  if (d2 > p.cut) return;
+  const double e = d2 / (2.0 * p.sigma * p.sigma);
+  if (e < 80.0) P0 += p.amp * exp(-e);  // beyond: below 2e-35 of the amplitude
+}
+
 // rho0 = sqrt(g) P0, P0 a sum of Gaussian pulses in the embedding distance (FP64 math), on the rows
-// that a pulse reaches.  One warp per row.
+// that a pulse reaches.
 template <typename R>
-__global__ void init_rho_kernel(const InitGeom G, const InitScratch t, const Pulse* __restrict__ pulses, int npulse,
-                                const R* __restrict__ tab, R* __restrict__ rho0) {
-  const int lane = threadIdx.x & 31;
-  const long long rows = (long long)G.n1 * G.n3, warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long row = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); row < rows; row += warps) {
-    const int q3 = (int)(row / G.n1), q1 = (int)(row - (long long)q3 * G.n1);
+__global__ void init_rho_kernel(const InitGeom G, const InitScratch t, const InitUnits U,
+                                const Pulse* __restrict__ pulses, int npulse, const R* __restrict__ tab,
+                                R* __restrict__ rho0) {
+  const int lane = threadIdx.x & 31, n2 = G.n2;
+  const long long all_rows = (long long)G.n1 * G.n3, warps = (long long)gridDim.x * (blockDim.x >> 5);
+  const bool flat = G.kind == LBW_CARTESIAN;
+  for (long long unit = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); unit < U.count; unit += warps) {
+    const InitLane L(U, unit, all_rows, n2);
+    const int q3 = (int)(L.row / G.n1), q1 = (int)(L.row - (long long)q3 * G.n1);
     const double u1 = G.x0[0] + (q1 + 0.5) * G.h[0];
-    const bool flat = G.kind == LBW_CARTESIAN;
     // the row's nodes sit at (a c2, a s2, z), or (u1, u2, u3) on a Cartesian lattice
     double a = u1, z = t.b3[q3];
     if (G.kind == LBW_TRUMPET) a = u1 * t.a3[q3];
@@ -111,49 +170,95 @@ __global__ void init_rho_kernel(const InitGeom G, const InitScratch t, const Pul
       a = G.geom[0] + u1 * t.a3[q3];
       z = u1 * t.b3[q3];
     }
-    auto reach = [&](int first) -> unsigned {  // which of the pulses first .. first + 31 reach the row
-      bool near = false;
-      if (first + lane < npulse) {
-        const Pulse& p = pulses[first + lane];
-        const double da = flat ? a - p.x[0] : fabs(a) - p.axis, dz = z - p.x[2];
-        near = !(da * da + dz * dz > p.cut);
-      }
-      return __ballot_sync(0xffffffffu, near);
+    auto reaches = [&](const Pulse& p, double as, double zs) -> bool {
+      const double da = flat ? as - p.x[0] : fabs(as) - p.axis, dz = zs - p.x[2];
+      return !(da * da + dz * dz > p.cut);
     };
+    // which of the pulses first .. first + 31 reach row s of the unit (a lane per pulse)
+    auto reach = [&](int first, int s) -> unsigned {
+      const double as = __shfl_sync(0xffffffffu, a, s * n2 & 31), zs = __shfl_sync(0xffffffffu, z, s * n2 & 31);
+      return __ballot_sync(0xffffffffu, first + lane < npulse && reaches(pulses[min(first + lane, npulse - 1)], as, zs));
+    };
+    // fewer pulses than rows: every lane tests its own row instead
+    const bool few = npulse < L.rows;
+    unsigned hit = 0;  // the rows that some pulse reaches
     bool any = false;
-    for (int first = 0; first < npulse && !any; first += 32) any = reach(first) != 0;
-    if (lane == 0) t.near[row] = any;
-    if (!any) continue;
-    const double sg = (double)tab[row * T_SLOTS + T_SG];
-    for (int base = 0; base < G.n2; base += 32) {
-      const int q2 = base + lane;
-      const bool in = q2 < G.n2;
-      const double c2 = in ? t.c2[q2] : 0.0, s2 = in && !flat ? t.s2[q2] : 0.0;
+    if (few) {
+      for (int k = 0; k < npulse; ++k) any |= reaches(pulses[k], a, z);
+      hit = __ballot_sync(0xffffffffu, any);
+    } else {
+      for (int s = 0; s < L.rows; ++s)
+        for (int first = 0; first < npulse && !(hit >> s & 1); first += 32)
+          if (reach(first, s)) hit |= 1u << s;
+      any = hit >> L.sub & 1;
+    }
+    if (L.c0 == 0) t.near[L.row] = any;
+    if (!hit) continue;
+    const double sg = (double)tab[L.row * T_SLOTS + T_SG];
+    const int steps = U.rows > 1 ? 1 : (L.c1 - (L.c0 - lane) + 31) / 32;  // the same for every lane
+    for (int k = 0, q2 = L.c0; k < steps; ++k, q2 += 32) {
+      const bool in = q2 < L.c1 && any;
+      double c2 = 0.0, s2 = 0.0;
+      if (in) {
+        c2 = flat ? G.x0[1] + (q2 + 0.5) * G.h[1] : t.c2[q2];
+        s2 = flat ? 0.0 : t.s2[q2];
+      }
       const double X0 = flat ? a : a * c2, X1 = flat ? c2 : a * s2;
       double P0 = 0.0;
-      for (int first = 0; first < npulse; first += 32)
-        for (unsigned left = reach(first); left; left &= left - 1) {
-          const Pulse& p = pulses[first + __ffs(left) - 1];
-          const double d2 = (X0 - p.x[0]) * (X0 - p.x[0]) + (X1 - p.x[1]) * (X1 - p.x[1]) + (z - p.x[2]) * (z - p.x[2]);
-          if (d2 > p.cut) continue;
-          const double e = d2 / (2.0 * p.sigma * p.sigma);
-          if (e < 80.0) P0 += p.amp * exp(-e);  // beyond: below 2e-35 of the amplitude
+      if (few) {
+        if (in)
+          for (int j = 0; j < npulse; ++j) add_pulse(pulses[j], X0, X1, z, P0);
+      } else {
+        for (int first = 0; first < npulse; first += 32) {
+          unsigned left = 0;
+          for (int s = 0; s < L.rows; ++s) left |= reach(first, s);
+          for (; left; left &= left - 1) add_pulse(pulses[first + __ffs(left) - 1], X0, X1, z, P0);
         }
-      if (in) rho0[row * G.n2 + q2] = (R)(sg * P0);
+      }
+      if (in) rho0[L.row * n2 + q2] = (R)(sg * P0);
     }
   }
 }
 
-// Post-collision state at rest on the rows that a pulse reaches and their neighbours (elsewhere it
-// is zero): f*_i = f_i^eq(rho0, F(rho0) / 2), F from the same table.  One warp per row.
+// The same for small lattices and few pulses: a thread per node tests every pulse and evaluates the
+// terms of its axes itself, which costs less than the launch that tabulates them and the tests of the
+// rows (3000 members of 512 nodes, a launch each: 54 -> 40 ms).
+template <typename R>
+__global__ void init_rho_small_kernel(const InitGeom G, unsigned char* __restrict__ near,
+                                      const Pulse* __restrict__ pulses, int npulse, const R* __restrict__ tab,
+                                      R* __restrict__ rho0) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, row = x / G.n2, q2 = x - row * G.n2;
+  if (row >= G.n1 * G.n3) return;
+  const int q3 = row / G.n1, q1 = row - q3 * G.n1;
+  const double u1 = G.x0[0] + (q1 + 0.5) * G.h[0];
+  double a3, z, c2, s2, a = u1;
+  plane_terms(G, q3, a3, z);
+  column_terms(G, q2, c2, s2);
+  if (G.kind == LBW_TRUMPET) a = u1 * a3;
+  if (G.kind == LBW_TOROIDAL) {
+    a = G.geom[0] + u1 * a3;
+    z = u1 * z;
+  }
+  const bool flat = G.kind == LBW_CARTESIAN;
+  const double X0 = flat ? a : a * c2, X1 = flat ? c2 : a * s2;
+  double P0 = 0.0;
+  for (int k = 0; k < npulse; ++k) add_pulse(pulses[k], X0, X1, z, P0);
+  rho0[x] = (R)((double)tab[(long long)row * T_SLOTS + T_SG] * P0);
+  if (q2 == 0) near[row] = 1;
+}
+
+// Post-collision state at rest, f*_i = f_i^eq(rho0, F(rho0) / 2) with F from the same table, on the
+// rows that a pulse reaches and their neighbours; the others are zero (`all`: written here).
 template <typename S>
-__global__ void init_f_kernel(const StepArgs<S> a, const unsigned char* __restrict__ near,
+__global__ void init_f_kernel(const StepArgs<S> a, const unsigned char* __restrict__ near, const InitUnits U, bool all,
                               const typename Store<S>::R* __restrict__ rho0) {
   using R = typename Store<S>::R;
   const bool p1 = a.bc[0] == LBW_BC_PERIODIC, p2 = a.bc[2] == LBW_BC_PERIODIC, p3 = a.bc[4] == LBW_BC_PERIODIC;
-  const int lane = threadIdx.x & 31, n1 = a.n1, n2 = a.n2;
-  const long long rows = (long long)n1 * a.n3, warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long row = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); row < rows; row += warps) {
+  const int n1 = a.n1, n2 = a.n2;
+  const long long all_rows = (long long)n1 * a.n3, warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long unit = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); unit < U.count; unit += warps) {
+    const InitLane lane(U, unit, all_rows, n2);
+    const long long row = lane.row;
     const int q3 = (int)(row / n1), q1 = (int)(row - (long long)q3 * n1);
     // rho0 of a row, or nullptr where it is zero (or a ghost)
     auto line = [&](int r1, int r3) -> const R* {
@@ -164,10 +269,10 @@ __global__ void init_f_kernel(const StepArgs<S> a, const unsigned char* __restri
       return near[r] ? rho0 + r * n2 : nullptr;
     };
     const R *Lc = line(q1, q3), *Lu = line(q1 + 1, q3), *Ld = line(q1 - 1, q3), *Ln = line(q1, q3 + 1), *Lp = line(q1, q3 - 1);
-    if (!Lc && !Lu && !Ld && !Ln && !Lp) continue;
+    if (!all && !Lc && !Lu && !Ld && !Ln && !Lp) continue;
     auto at = [](const R* l, int q2) -> R { return l ? l[q2] : R(0); };
     const R* c = a.tab + row * T_SLOTS;
-    for (int q2 = lane; q2 < n2; q2 += 32) {
+    for (int q2 = lane.c0; q2 < lane.c1; q2 += 32) {
       const R rho = at(Lc, q2), ru = at(Lu, q2), rd = at(Ld, q2), rn = at(Ln, q2), rp = at(Lp, q2);
       const int ql = q2 == 0 ? n2 - 1 : q2 - 1, qr = q2 == n2 - 1 ? 0 : q2 + 1;
       R rr = at(Lc, qr), rl = at(Lc, ql);
@@ -196,6 +301,11 @@ __global__ void init_f_kernel(const StepArgs<S> a, const unsigned char* __restri
   }
 }
 
+// Lattices of up to kInitAll nodes have every node written by the last kernel instead of a memset
+// before it; those of up to kInitSmall with at most kInitFew pulses take the kernel for them.
+constexpr long long kInitAll = 1 << 20, kInitSmall = 1 << 16;
+constexpr int kInitFew = 16;
+
 template <typename S>
 cudaError_t launch_init_t(Grid* g, const void* d_pulses, int npulse, void* d_scratch) {
   using R = typename Store<S>::R;
@@ -207,18 +317,27 @@ cudaError_t launch_init_t(Grid* g, const void* d_pulses, int npulse, void* d_scr
   G.n3 = g->d.n[2];
   for (int a = 0; a < 3; ++a) { G.h[a] = g->d.h[a]; G.x0[a] = g->d.x0[a]; }
   for (int k = 0; k < 4; ++k) G.geom[k] = g->d.geom[k];
-  const InitScratch t = carve_init(d_scratch, G.n1, G.n2, G.n3);
-  // rho0 goes to the scratch bytes of the other population buffer (>= N values of R)
+  // rho0 goes to the other population buffer (>= N values of R), and the scratch behind it where it fits
   R* rho0 = reinterpret_cast<R*>(g->f[1 - g->cur]);
-  cudaError_t e = cudaMemsetAsync(g->f[g->cur], 0, (size_t)7 * pop_stride(g) * g->elem, g->stream);
+  if (init_scratch_bytes(*g) == 0) d_scratch = static_cast<unsigned char*>(g->f[1 - g->cur]) + scratch_offset(*g);
+  const InitScratch t = carve_init(d_scratch, G.n2, G.n3);
+  const bool all = g->nn <= kInitAll && npulse > 0;
+  cudaError_t e = cudaSuccess;
+  if (!all) e = cudaMemsetAsync(g->f[g->cur], 0, (size_t)7 * pop_stride(g) * g->elem, g->stream);
   if (e != cudaSuccess || npulse == 0) return e;
-  const long long rows = (long long)G.n1 * G.n3;
-  const int blocks = (int)std::min<long long>((rows + 7) / 8, 152LL * 16);
-  axis_kernel<<<(G.n2 + G.n3 + 127) / 128, 128, 0, g->stream>>>(G, t);
-  init_rho_kernel<R><<<blocks, 256, 0, g->stream>>>(G, t, static_cast<const Pulse*>(d_pulses), npulse,
-                                                    reinterpret_cast<const R*>(g->table), rho0);
+  const InitUnits U = init_units(G.n1, G.n2, G.n3);
+  const int warps = U.count < 152 * 16 ? 2 : 8;  // per block: few units spread over the SMs
+  const int blocks = (int)std::min<long long>((U.count + warps - 1) / warps, 152LL * 16);
+  const Pulse* pulses = static_cast<const Pulse*>(d_pulses);
+  const R* tab = reinterpret_cast<const R*>(g->table);
+  if (g->nn <= kInitSmall && npulse <= kInitFew) {
+    init_rho_small_kernel<R><<<(int)(g->nn + 127) / 128, 128, 0, g->stream>>>(G, t.near, pulses, npulse, tab, rho0);
+  } else {
+    axis_kernel<<<(G.n2 + G.n3 + 127) / 128, 128, 0, g->stream>>>(G, t);
+    init_rho_kernel<R><<<blocks, 32 * warps, 0, g->stream>>>(G, t, U, pulses, npulse, tab, rho0);
+  }
   StepArgs<S> a = step_args<S>(*g, 1 - g->cur);  // fout = current buffer
-  init_f_kernel<S><<<blocks, 256, 0, g->stream>>>(a, t.near, rho0);
+  init_f_kernel<S><<<blocks, 32 * warps, 0, g->stream>>>(a, t.near, U, all, rho0);
   return cudaGetLastError();
 }
 
@@ -316,8 +435,8 @@ int planes_per_turn(const Grid* g) {
 
 }  // namespace
 
-size_t init_scratch_bytes(const lbw_grid_desc& d) {
-  return sizeof(double) * 2 * ((size_t)d.n[1] + d.n[2]) + (size_t)d.n[0] * d.n[2];
+size_t init_scratch_bytes(const Grid& g) {
+  return scratch_offset(g) + scratch_bytes(g.d) <= (size_t)7 * pop_stride(&g) * g.elem ? 0 : scratch_bytes(g.d);
 }
 
 size_t pulse_bytes(int n) { return sizeof(Pulse) * std::max(1, n); }
