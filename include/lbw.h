@@ -107,8 +107,9 @@ typedef enum { LBW_EQ_CURVILINEAR = 0, LBW_EQ_MOMENT_MATCHING = 1, LBW_EQ_HERMIT
  * (q2 extent a multiple of 64, non-periodic q1) accept it.  AUTO takes the table, the faster of
  * the two on the benchmark lattices (measured: 472 against 966 us per torus step), and advances
  * lattices that the SMs hold (up to 620,000 nodes; FP64, and 16-bit storage on the tile kernel:
- * 300,000) many steps per launch, with the table rows kept in shared memory; TABLE and ANALYTIC
- * always launch once per step. */
+ * 300,000) many steps per launch, with the table rows kept in shared memory (not while plates
+ * of sources make launches per step the faster way); TABLE and ANALYTIC always launch once per
+ * step. */
 typedef enum { LBW_GEOM_AUTO = 0, LBW_GEOM_TABLE = 1, LBW_GEOM_ANALYTIC = 2 } lbw_geom_mode;
 
 /* A Gaussian pulse P0 = amp exp(-|X - x|^2 / (2 sigma^2)) in the embedding distance. */

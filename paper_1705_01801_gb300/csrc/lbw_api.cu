@@ -434,7 +434,7 @@ lbw_status lbw_step(lbw_grid* g, int64_t n_steps) {
   if (n_steps < 0) return fail(LBW_EINVAL, "n_steps must be >= 0");
   const int chain = 64;
   int64_t left = n_steps;
-  if (g->res) {
+  if (g->res && resident_pays(g->res, g->src_kind)) {
     while (left > 0) {
       const int n = (int)std::min<int64_t>(left, kResChunk);
       const ResState rs{{g->f[0], g->f[1]}, g->cur, g->counters, g->tma_by > 0 ? g->counters + 4 : nullptr,

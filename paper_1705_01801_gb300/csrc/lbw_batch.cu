@@ -1049,6 +1049,7 @@ struct lbw_batch {
   BatchItem* items = nullptr;
   int n_items = 0, blocks = 0;
   Shape shape;
+  bool stale = false;  // the multi-step kernel has stepped: it does not keep the ghost columns
   bool ready = false;  // work list, tensor maps and arguments on the device are those of `shape`
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   int graph_len = 0, cur = 0;
@@ -1237,13 +1238,12 @@ int dense_pitch(int n2, size_t es) {
 }
 
 // The current state into the layout that the launch shape wants (dense rows for full-row tiles,
-// else ghost columns, rebuilt even where the layout stays: the resident kernel does not keep
-// them), through the other buffer.
-lbw_status use_layout(lbw_batch* b, bool rebuild) {
+// else ghost columns, rebuilt even where the layout stays if they are stale), through the other buffer.
+lbw_status use_layout(lbw_batch* b) {
   if (!b->tma) return LBW_OK;
   const size_t es = es_of(b->prec);
   const int G = b->shape.by == 0 ? 0 : ghost_cols(es);
-  if (b->views[0].col0 == G && !(rebuild && G > 0)) return LBW_OK;
+  if (b->views[0].col0 == G && !(b->stale && G > 0)) return LBW_OK;
   for (Grid& g : b->views) {
     const int n2 = g.d.n[1], pitch = G ? padded_pitch(n2, es) : dense_pitch(n2, es);
     const long long rows = 7LL * g.d.n[0] * g.d.n[2];
@@ -1260,6 +1260,7 @@ lbw_status use_layout(lbw_batch* b, bool rebuild) {
   }
   LBW_CUDA(cudaGetLastError());
   b->cur = 1 - b->cur;
+  b->stale = false;
   return build_sources(b);
 }
 
@@ -1411,9 +1412,9 @@ lbw_status upload_members(lbw_batch* b) {
   return prec_dispatch(b->prec, [&](auto tag) { return upload_args<decltype(tag)>(b); });
 }
 
-lbw_status refresh(lbw_batch* b, bool rebuild_ghosts = false) {
+lbw_status refresh(lbw_batch* b) {
   b->ready = false;
-  lbw_status st = use_layout(b, rebuild_ghosts);
+  lbw_status st = use_layout(b);
   if (st == LBW_OK) st = build_items(b);
   if (st == LBW_OK && b->tma) st = build_batch_maps(b, b->shape);
   if (st == LBW_OK) st = upload_members(b);
@@ -1501,6 +1502,7 @@ cudaError_t run_resident(lbw_batch* b, int n) {
                     static_cast<const SourceEntry*>(b->src), b->src_kind, b->src_amp, b->stream};
   const cudaError_t e = resident_run(b->res, nullptr, b->members[0], rs, n);
   if (e == cudaSuccess) b->cur ^= n & 1;
+  b->stale = true;
   return e;
 }
 
@@ -1509,10 +1511,15 @@ lbw_status advance(lbw_batch* b, int64_t n_steps) {
     return fail(LBW_ESTATE, "the ensemble's last change of launch shape failed; lbw_batch_set_shape sets one");
   const int chain = 64;
   int64_t left = n_steps;
-  while (b->res && left > 0) {
+  const bool resident = b->res && resident_pays(b->res, b->src_kind);
+  while (resident && left > 0) {
     const int n = (int)std::min<int64_t>(left, kResChunk);
     LBW_CUDA(run_resident(b, n));
     left -= n;
+  }
+  if (left > 0) {
+    const lbw_status st = use_layout(b);
+    if (st != LBW_OK) return st;
   }
   if (left >= chain) {
     for (int start = 0; start < 2; ++start) {
@@ -1994,7 +2001,7 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
     if (st != LBW_OK) {  // back to the shape it had
       const std::string why = lbw_last_error();
       b->shape = start;
-      refresh(b, b->res != nullptr);
+      refresh(b);
       return fail(st, why);
     }
     if (cache_path) {
@@ -2004,7 +2011,7 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
     }
   }
   b->shape = best;
-  lbw_status st = refresh(b, b->res != nullptr && !resident);
+  lbw_status st = refresh(b);
   if (st != LBW_OK) return st;
   if (!resident) {
     resident_destroy(b->res, b->stream);
@@ -2034,7 +2041,7 @@ lbw_status lbw_batch_set_shape(lbw_batch* b, int32_t tile_rows, int32_t seg_plan
     return fail(LBW_EINVAL, "ctas_per_sm must be in [1, what the kernel keeps resident]");
   const Shape old = b->shape;
   b->shape = Shape{tile_rows, seg_planes, ctas_per_sm};
-  lbw_status st = refresh(b, b->res != nullptr);
+  lbw_status st = refresh(b);
   if (st != LBW_OK) {
     const std::string why = lbw_last_error();
     b->shape = old;

@@ -228,29 +228,44 @@ StepArgs<S> step_args(const Grid& lattice, int src) {
 // populations are replaced by the equilibrium carrying the imposed value v = C sin(omega t);
 // kind 0: f_i = f_i^eq(sqrt(g) v, 0); kind 1: f_i = f_i^eq(rho, (0, 0, sqrt(g) v)) with the
 // node's own rho.  16-bit formats store f_i / w_i.
-template <typename S>
+template <typename S, bool UNROLL = true>
 __device__ __forceinline__ void impose_source(S* base, const SourceEntry& s, int kind, double v) {
+  using R = typename Store<S>::R;
   const double cs2 = s.cs2;
   const double w0 = 1.0 - 3.0 * cs2, w1 = 0.5 * cs2;
   S* f = base + s.off;
-  double rho = 0.0, j3 = 0.0;
-  if (kind == 0) {
-    rho = s.sg * v;
-  } else {
+  double rho = s.sg * v, j3 = 0.0, d = 0.0;  // d = j3 / cs2, not taken where it is not needed
+  if (kind != 0) {
+    j3 = rho;
+    if constexpr (sizeof(S) < 8) d = j3 / cs2;
+    rho = 0.0;
     for (int i = 0; i < 7; ++i) {
       double x = (double)Store<S>::ld_smem(f + (long long)i * s.ps);
       if (Store<S>::kScaled) x *= (i == 0 ? w0 : w1);
       rho += x;
     }
-    j3 = s.sg * v;
   }
-  for (int i = 0; i < 7; ++i) {
-    const double xi3 = i == 5 ? 1.0 : (i == 6 ? -1.0 : 0.0);
-    double val = i == 0 ? w0 * rho : w1 * (rho + xi3 * j3 / cs2);
-    if (Store<S>::kScaled) val /= (i == 0 ? w0 : w1);
-    const typename Store<S>::R r = (typename Store<S>::R)val;
-    Store<S>::st(f + (long long)i * s.ps, r);
-    if (s.ghost != 0) Store<S>::st(f + (long long)i * s.ps + s.ghost, r);
+  auto put = [&](S* at, double val) {
+    const R r = (R)val;
+    Store<S>::st(at, r);
+    if (s.ghost != 0) Store<S>::st(at + s.ghost, r);
+  };
+  if constexpr (sizeof(S) == 8) {
+    for (int i = 0; i < 7; ++i) {
+      const double xi3 = i == 5 ? 1.0 : (i == 6 ? -1.0 : 0.0);
+      put(f + (long long)i * s.ps, i == 0 ? w0 * rho : w1 * (rho + xi3 * j3 / cs2));
+    }
+  } else {
+    // one division at most; not unrolled in the multi-step kernels, which keep more of their nodes in
+    // registers (FP16 4 % faster, also without sources; in FP64, two nodes of which fill them, the form
+    // above is 2 % faster)
+#pragma unroll (UNROLL ? 7 : 1)
+    for (int i = 0; i < 7; ++i) {
+      double val = i == 0 ? w0 * rho : w1 * (i < 5 ? rho : i == 5 ? rho + d : rho - d);
+      if (Store<S>::kScaled) val /= (i == 0 ? w0 : w1);
+      put(f, val);
+      f += s.ps;
+    }
   }
 }
 

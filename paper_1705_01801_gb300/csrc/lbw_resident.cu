@@ -236,6 +236,12 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   __shared__ int near_x[kNear];
   __shared__ R near_v[kNear][2];
   __shared__ double near_sg[kNear], near_om[kNear], near_cs2;
+  // The others of a lattice have one frequency: 32- and 16-bit storage takes the sine of the first once
+  // (far_v) instead of one per source, which bound plates of them (a plane of 128 x 128, FP32: 18.7 ->
+  // 14.2 us a step).  FP64 is bound by its nodes, and the share would cost them registers.
+  constexpr bool kShare = sizeof(S) < 8;
+  __shared__ int ntimed;  // sources whose sine is taken here: the near ones, or the first
+  __shared__ double far_v;
   const int tid = threadIdx.x, nthr = blockDim.x;
   // what only the prologue, the edges and thread 0 need stays in shared memory: 1024 threads have
   // 64 registers each
@@ -344,13 +350,15 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
   S* const buf[2] = {const_cast<S*>(A.fin), A.fout};
   const int nsrc = it.src_hi - it.src_lo;
   const bool near = nsrc <= kNear && ra.src_kind == 0;
+  if (tid == 0) ntimed = near ? nsrc : kShare && nsrc > 0;
   auto source_entry = [&](int e) { return ra.src[ra.src_order[it.src_lo + e]]; };
-  auto source_value = [&](const SourceEntry& s, unsigned long long t) { return ra.src_amp * sin(s.omega * (double)t); };
   // near source `mine`'s populations at time t, as impose_source writes them; the last threads
   // compute them, thread 0 waits at the barrier meanwhile
   const int mine = nthr - 1 - tid;
+  __syncthreads();
   auto set_near = [&](unsigned long long t) {
-    const double rho = near_sg[mine] * (ra.src_amp * sin(near_om[mine] * (double)t));
+    const double v = ra.src_amp * sin(near_om[mine] * (double)t), rho = near_sg[mine] * v;
+    if (kShare && mine == 0) far_v = v;
     const double w0 = 1.0 - 3.0 * near_cs2, w1 = 0.5 * near_cs2;
     double rest = w0 * rho, moving = w1 * rho;
     if (Store<S>::kScaled) {
@@ -360,7 +368,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
     near_v[mine][0] = (R)rest;
     near_v[mine][1] = (R)moving;
   };
-  if (near && mine < nsrc) {
+  if (mine < ntimed) {
     const SourceEntry e = source_entry(mine);
     near_x[mine] = (int)(e.off - (A.fin - ra.base[0]));  // relative to the lattice's own buffer
     near_sg[mine] = e.sg;
@@ -368,7 +376,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
     near_cs2 = e.cs2;
   }
   __syncthreads();
-  if (near && mine < nsrc) set_near(t0 + 1);
+  if (mine < ntimed) set_near(t0 + 1);
   __syncthreads();
   if (near && nsrc > 0) {
 #pragma unroll
@@ -475,7 +483,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
       __syncthreads();
       for (int e = tid; e < nsrc; e += nthr) {
         const SourceEntry se = source_entry(e);
-        impose_source(ra.base[1 - cur], se, ra.src_kind, source_value(se, t0 + s + 1));
+        impose_source<S, false>(ra.base[1 - cur], se, ra.src_kind, kShare ? far_v : ra.src_amp * sin(se.omega * (double)(t0 + s + 1)));
       }
     }
     cur ^= 1;
@@ -483,7 +491,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResArgs<S> ra) {
     __syncthreads();
     if (tid == 0) red_release(ra.bars + 32 * it.group);
     // the next step's source values, while the other CTAs arrive
-    if (near && mine < nsrc) set_near(t0 + s + 2);
+    if (mine < ntimed) set_near(t0 + s + 2);
     if (tid == 0) {
       const unsigned want = (unsigned)(s + 1) * (unsigned)it.group_size;
       long long n = 0;
@@ -669,6 +677,7 @@ lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool ti
   Resident r;
   r.prec = prec;
   r.tile = tile;
+  r.nodes = total;
   for (int m = 0; m < n; ++m) r.x13 |= lattices[m]->d.kind == LBW_TRUMPET;
   for (int first = 0; first < n;) {
     // the lattices of one launch: as many as the SMs hold at the most nodes per thread
@@ -794,9 +803,29 @@ lbw_status resident_sources(Resident* r, const int32_t* host_q, int per_lattice,
   LBW_CUDA(cudaMemcpyAsync(r->items, items.data(), sizeof(ResItem) * items.size(), cudaMemcpyHostToDevice, stream));
   if (r->src_order) cudaFreeAsync(r->src_order, stream);
   r->src_order = d_order;
+  r->most = 0;
+  for (const ResItem& it : items) r->most = std::max(r->most, it.src_hi - it.src_lo);
   r->host_items.swap(items);
   LBW_CUDA(cudaStreamSynchronize(stream));
   return LBW_OK;
+}
+
+// Up to kFewSources sources in a box never decide.  Beyond, ns a step as measured: a node of the largest
+// box and a source of the fullest here (kind 0, 1), a node of all lattices where a step is a launch
+// (tile kernels, others); FP32 with four planes of P sources here / launched: 64 x 128 x 70 31 / 19 us, 64 x 64
+// x 100 20 / 15; with one plane 17 / 18, 12 / 15.
+bool resident_pays(const Resident* r, int src_kind) {
+  constexpr int kFewSources = 256;
+  if (r->most <= kFewSources) return true;
+  struct Cost {
+    double node, source[2], launched[2];
+  };
+  const Cost c = r->prec == LBW_F64   ? Cost{10.2, {9.2, 7.0}, {0.12, 0.19}}
+                 : r->prec == LBW_F32 ? Cost{3.3, {8.5, 14.5}, {0.010, 0.030}}
+                                      : Cost{3.5, {25.0, 31.0}, {0.008, 0.050}};
+  double here = r->most * c.source[src_kind != 0];
+  for (const Resident::Launch& L : r->launches) here += 2000.0 + L.own * c.node;
+  return here < 10500.0 + r->nodes * c.launched[r->tile ? 0 : 1];
 }
 
 cudaError_t resident_run(const Resident* r, const Grid* one, const void* members, const ResState& st, int steps) {

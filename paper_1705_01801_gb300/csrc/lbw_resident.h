@@ -26,6 +26,8 @@ struct Resident {
   int prec = 0;
   bool tile = false;             // operations of the tile kernels (see lbw_resident.cu)
   bool x13 = false;              // some lattice's metric couples q1 and q3
+  long long nodes = 0;           // of all lattices
+  int most = 0;                  // sources of the box that holds the most
   ResItem* items = nullptr;
   unsigned* bars = nullptr;
   int* src_order = nullptr;
@@ -54,6 +56,9 @@ void resident_destroy(Resident* r, cudaStream_t stream);
 // Assigns the sources (per_lattice nodes of each lattice, in SourceEntry order) to the boxes; none
 // (0) before their list is freed, which needs no memory.
 lbw_status resident_sources(Resident* r, const int32_t* host_q, int per_lattice, cudaStream_t stream);
+// Whether it is ahead of a launch per step with the sources that it has (a box's sources are served
+// by one SM, which a plate of several planes keeps busy).
+bool resident_pays(const Resident* r, int src_kind);
 // `steps` <= kResChunk time steps from buffer st.cur: of the lattice `one`, or of an ensemble
 // with StepArgs array `members` (source buffer 0).
 cudaError_t resident_run(const Resident* r, const Grid* one, const void* members, const ResState& st, int steps);
