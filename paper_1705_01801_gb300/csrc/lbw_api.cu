@@ -288,6 +288,7 @@ lbw_status read_counters(Grid* g, unsigned long long* recorded, unsigned long lo
   LBW_CUDA(cudaStreamSynchronize(g->stream));
   if (recorded) *recorded = c[0];
   if (bad) *bad = c[4];
+  if (c[4]) LBW_CUDA(cudaMemsetAsync(g->counters + 5, 0, sizeof(unsigned long long), g->stream));  // told once
   if (c[2]) return fail(LBW_ETIMEOUT, "a time step's bounded wait for staged data ran out; the state is "
                                       "undefined until lbw_init");
   return LBW_OK;
@@ -520,13 +521,15 @@ lbw_status lbw_source(lbw_grid* g, const int32_t* host_q, int32_t n, int32_t kin
   if (n > 0) {
     LBW_CUDA(cudaMallocAsync(&g->src, sizeof(SourceEntry) * n, g->stream));
     LBW_CUDA(cudaMemcpyAsync(g->src, h.data(), sizeof(SourceEntry) * n, cudaMemcpyHostToDevice, g->stream));
-    LBW_CUDA(cudaStreamSynchronize(g->stream));
     g->nsrc = n;
     g->src_kind = kind;
     g->src_amp = amp;
     const lbw_status st = g->res ? resident_sources(g->res, host_q, n, g->stream) : LBW_OK;
-    if (st != LBW_OK) drop();
-    return st;
+    if (st != LBW_OK) {
+      drop();
+      return st;
+    }
+    LBW_CUDA(cudaStreamSynchronize(g->stream));
   }
   return LBW_OK;
 }

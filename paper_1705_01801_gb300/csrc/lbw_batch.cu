@@ -1221,11 +1221,12 @@ lbw_status build_sources(lbw_batch* b) {
   cudaError_t e = cudaMallocAsync(&b->src, sizeof(SourceEntry) * h.size(), b->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->src, h.data(), sizeof(SourceEntry) * h.size(), cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return none(cuda_fail(e, "source list"));
   b->nsrc = (int)h.size();
   const lbw_status st = b->res ? resident_sources(b->res, b->src_q.data(), (int)per, b->stream) : LBW_OK;
-  return st == LBW_OK ? st : none(st);
+  if (st != LBW_OK) return none(st);
+  LBW_CUDA(cudaStreamSynchronize(b->stream));
+  return LBW_OK;
 }
 
 // Rows as the full-row kernel stores them: no ghost columns, n2 rounded up to 16 bytes.  Ghost

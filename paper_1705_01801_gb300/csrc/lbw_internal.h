@@ -159,7 +159,7 @@ size_t pulse_bytes(int n);
 void pack_pulses(const lbw_pulse* p, int n, void* out);
 cudaError_t launch_init(Grid* g, const void* d_pulses, int npulse, void* d_scratch);
 // P and the populations of the current state to host arrays, and back from one (enqueued, through
-// the other population buffer); *d_bad tells whether a value of P is not finite
+// the other population buffer); *d_bad becomes 1 where a value of P is not finite
 cudaError_t read_field(Grid* g, double* host_P, unsigned long long* d_bad);
 cudaError_t read_populations(Grid* g, double* host_f);
 cudaError_t write_populations(Grid* g, const double* host_f);

@@ -806,8 +806,7 @@ lbw_status resident_sources(Resident* r, const int32_t* host_q, int per_lattice,
   r->most = 0;
   for (const ResItem& it : items) r->most = std::max(r->most, it.src_hi - it.src_lo);
   r->host_items.swap(items);
-  LBW_CUDA(cudaStreamSynchronize(stream));
-  return LBW_OK;
+  return LBW_OK;  // pageable copies have left the host arrays; callers synchronise
 }
 
 // Up to kFewSources sources in a box never decide.  Beyond, ns a step as measured: a node of the largest

@@ -10,8 +10,8 @@
 // every pulse's distance at every node: torus 192 x 1024 x 256 8.3 -> 0.45 ms, 48 trumpets with
 // twelve pulses each 33 -> 8.5 ms.
 //
-// Read-out.  The values go through the population buffer that the next step overwrites, so no
-// device memory is allocated; whether they are finite is decided where they are computed (a host
+// Read-out.  The values go through the population buffer that the next step overwrites, so large
+// lattices need no device memory for it; whether they are finite is decided where they are computed (a host
 // loop over the field took 23 of the 39 ms of the torus's snapshot, first touches of the caller's
 // array 13; now 6 ms).
 #include <cuda_bf16.h>
@@ -428,10 +428,36 @@ Pad<I> pad_of(const Grid* g) {
 
 constexpr int kReadThreads = 256, kReadBlocks = 152 * 8;
 
-// populations per turn through the other buffer: as many planes of doubles as it holds
-int planes_per_turn(const Grid* g) {
-  return (int)std::max<long long>(1, std::min<long long>(7, 7 * pop_stride(g) * (long long)g->elem / (8 * g->nn)));
+unsigned read_blocks(const Grid* g) {
+  return (unsigned)std::min<long long>((g->nn + kReadThreads - 1) / kReadThreads, kReadBlocks);
 }
+
+// Room for `per` planes of doubles on the device: the other population buffer, which holds 1 to 7, or
+// for small lattices a temporary of all seven where it can be had, as every turn costs a launch and a
+// copy of its own (64 FP32 nodes 85 -> 42 us, 262,144 557 -> 380).
+struct Planes {
+  Grid* g;
+  double* d;
+  int per;
+  bool own = false;
+  explicit Planes(Grid* grid) : g(grid), d(static_cast<double*>(grid->f[1 - grid->cur])) {
+    constexpr long long kTemporary = 64 << 20;
+    const long long all = 7LL * 8 * g->nn;
+    per = (int)std::max<long long>(1, std::min<long long>(7, 7 * pop_stride(g) * (long long)g->elem / (8 * g->nn)));
+    void* t = nullptr;
+    if (per == 7 || all > kTemporary) return;
+    if (cudaMallocAsync(&t, (size_t)all, g->stream) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    d = static_cast<double*>(t);
+    per = 7;
+    own = true;
+  }
+  ~Planes() {
+    if (own) cudaFreeAsync(d, g->stream);
+  }
+};
 
 }  // namespace
 
@@ -462,6 +488,9 @@ cudaError_t launch_init(Grid* g, const void* d_pulses, int npulse, void* d_scrat
 // faster than the copy that would otherwise take the faults one after the other (403 MB: 13 -> 4 ms).
 void touch_pages(void* p, size_t bytes) {
   const size_t page = (size_t)sysconf(_SC_PAGESIZE), least = (size_t)4 << 20;
+  // smaller arrays come from pages that the allocator keeps mapped as a rule, and asking for the number
+  // of cores alone takes 20 us
+  if (bytes < 8 * least) return;
   const int n = (int)std::min<size_t>({bytes / least, 8, std::max(1u, std::thread::hardware_concurrency())});
   if (n < 2) return;
   std::vector<std::thread> threads;
@@ -480,54 +509,50 @@ void touch_pages(void* p, size_t bytes) {
 
 cudaError_t read_field(Grid* g, double* host_P, unsigned long long* d_bad) {
   double* d = static_cast<double*>(g->f[1 - g->cur]);  // 14 to 56 bytes per node
-  cudaError_t e = cudaMemsetAsync(d_bad, 0, sizeof(*d_bad), g->stream);
-  if (e == cudaSuccess)
-    e = with_types(g, [&](auto tag, auto index) {
-      using S = decltype(tag);
-      using I = decltype(index);
-      field_kernel<S, I><<<kReadBlocks, kReadThreads, 0, g->stream>>>(
-          static_cast<const S*>(g->f[g->cur]), (I)g->nn, pop_stride(g), pad_of<I>(g),
-          static_cast<const typename Store<S>::R*>(g->table), g->w0, g->w1, d, d_bad);
-      return cudaGetLastError();
-    });
+  const cudaError_t e = with_types(g, [&](auto tag, auto index) {
+    using S = decltype(tag);
+    using I = decltype(index);
+    field_kernel<S, I><<<read_blocks(g), kReadThreads, 0, g->stream>>>(
+        static_cast<const S*>(g->f[g->cur]), (I)g->nn, pop_stride(g), pad_of<I>(g),
+        static_cast<const typename Store<S>::R*>(g->table), g->w0, g->w1, d, d_bad);
+    return cudaGetLastError();
+  });
   if (e != cudaSuccess) return e;
   touch_pages(host_P, sizeof(double) * g->nn);
   return cudaMemcpyAsync(host_P, d, sizeof(double) * g->nn, cudaMemcpyDeviceToHost, g->stream);
 }
 
 cudaError_t read_populations(Grid* g, double* host_f) {
-  double* d = static_cast<double*>(g->f[1 - g->cur]);
-  const int per = planes_per_turn(g);
+  const Planes p(g);
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < 7 && e == cudaSuccess; i += per) {
-    const int n = std::min(per, 7 - i);
+  for (int i = 0; i < 7 && e == cudaSuccess; i += p.per) {
+    const int n = std::min(p.per, 7 - i);
     e = with_types(g, [&](auto tag, auto index) {
       using S = decltype(tag);
       using I = decltype(index);
-      to_double_kernel<S, I><<<dim3(kReadBlocks, n), kReadThreads, 0, g->stream>>>(
-          static_cast<const S*>(g->f[g->cur]), i, (I)g->nn, pop_stride(g), pad_of<I>(g), g->w0, g->w1, d);
+      to_double_kernel<S, I><<<dim3(read_blocks(g), n), kReadThreads, 0, g->stream>>>(
+          static_cast<const S*>(g->f[g->cur]), i, (I)g->nn, pop_stride(g), pad_of<I>(g), g->w0, g->w1, p.d);
       return cudaGetLastError();
     });
     if (i == 0) touch_pages(host_f, sizeof(double) * 7 * g->nn);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(host_f + (size_t)i * g->nn, d, sizeof(double) * n * g->nn, cudaMemcpyDeviceToHost, g->stream);
+      e = cudaMemcpyAsync(host_f + (size_t)i * g->nn, p.d, sizeof(double) * n * g->nn, cudaMemcpyDeviceToHost, g->stream);
   }
   return e;
 }
 
 cudaError_t write_populations(Grid* g, const double* host_f) {
-  double* d = static_cast<double*>(g->f[1 - g->cur]);
-  const int per = planes_per_turn(g);
+  const Planes p(g);
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < 7 && e == cudaSuccess; i += per) {
-    const int n = std::min(per, 7 - i);
-    e = cudaMemcpyAsync(d, host_f + (size_t)i * g->nn, sizeof(double) * n * g->nn, cudaMemcpyHostToDevice, g->stream);
+  for (int i = 0; i < 7 && e == cudaSuccess; i += p.per) {
+    const int n = std::min(p.per, 7 - i);
+    e = cudaMemcpyAsync(p.d, host_f + (size_t)i * g->nn, sizeof(double) * n * g->nn, cudaMemcpyHostToDevice, g->stream);
     if (e != cudaSuccess) break;
     e = with_types(g, [&](auto tag, auto index) {
       using S = decltype(tag);
       using I = decltype(index);
-      from_double_kernel<S, I><<<dim3(kReadBlocks, n), kReadThreads, 0, g->stream>>>(
-          d, i, (I)g->nn, pop_stride(g), pad_of<I>(g), g->d.bc[2] == LBW_BC_PERIODIC, g->w0, g->w1,
+      from_double_kernel<S, I><<<dim3(read_blocks(g), n), kReadThreads, 0, g->stream>>>(
+          p.d, i, (I)g->nn, pop_stride(g), pad_of<I>(g), g->d.bc[2] == LBW_BC_PERIODIC, g->w0, g->w1,
           static_cast<S*>(g->f[g->cur]));
       return cudaGetLastError();
     });

@@ -1,0 +1,42 @@
+"""Populations of small lattices go through a temporary in one turn, those of large ones through the
+other population buffer in up to seven: written values come back exactly on both sides of the line
+(1,198,372 nodes), and a small lattice's read-out takes as long in 16-bit storage, whose other buffer
+holds one plane of doubles, as in FP64, whose holds all."""
+import time
+
+import numpy as np
+import pytest
+
+import lbw_workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec", [W.PREC_F64, W.PREC_F32, W.PREC_F16S, W.PREC_BF16S])
+@pytest.mark.parametrize("n", [(4, 4, 4), (100, 100, 119), (100, 100, 120), (64, 128, 150)])
+def test_written_populations_come_back(n, prec):
+    from paper_1705_01801_gb300 import lbw
+    g = lbw.Grid(W.cylinder(*n).with_(prec=prec))
+    rng = np.random.default_rng(sum(n))
+    f = rng.integers(-127, 128, size=(7, n[2], n[0], n[1])) / 64.0  # exact in every format
+    g.set_f(f)
+    np.testing.assert_array_equal(g.get_f(), f)
+    assert np.isfinite(g.get_P()).all()
+    g.close()
+
+
+def test_storage_does_not_set_the_time_of_a_small_read_out():
+    """One copy for each of seven turns takes 2.5 times as long."""
+    from paper_1705_01801_gb300 import lbw
+    took = []
+    for prec in (W.PREC_F16S, W.PREC_F64):
+        g = lbw.Grid(W.GridSpec(kind=W.KIND_CARTESIAN, n=(4, 4, 4), h=(1, 1, 1), x0=(0, 0, 0), c=0.4, bc=(0,) * 6, prec=prec))
+        g.init(np.zeros((0, 5)))
+        best = 1e9
+        for _ in range(30):
+            t = time.perf_counter()
+            g.get_f()
+            best = min(best, time.perf_counter() - t)
+        took.append(best)
+        g.close()
+    assert took[0] < 1.5 * took[1], took
