@@ -742,11 +742,13 @@ lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool ti
   r.host_items = items;
   Resident* p = new (std::nothrow) Resident(r);
   if (!p) return fail(LBW_ENOMEM, "host allocation failed");
-  cudaError_t e = cudaMallocAsync((void**)&p->items, sizeof(ResItem) * items.size(), stream);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&p->bars, sizeof(unsigned) * 32 * groups, stream);
-  if (e == cudaSuccess)
+  // one allocation: the barriers, then the boxes
+  const size_t bars = sizeof(unsigned) * 32 * groups;
+  cudaError_t e = cudaMallocAsync((void**)&p->bars, bars + sizeof(ResItem) * items.size(), stream);
+  if (e == cudaSuccess) {
+    p->items = reinterpret_cast<ResItem*>(reinterpret_cast<unsigned char*>(p->bars) + bars);
     e = cudaMemcpyAsync(p->items, items.data(), sizeof(ResItem) * items.size(), cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  }
   if (e != cudaSuccess) {
     resident_destroy(p, stream);
     return cuda_fail(e, "resident step kernel: upload");
@@ -757,7 +759,6 @@ lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool ti
 
 void resident_destroy(Resident* r, cudaStream_t stream) {
   if (!r) return;
-  if (r->items) cudaFreeAsync(r->items, stream);
   if (r->bars) cudaFreeAsync(r->bars, stream);
   if (r->src_order) cudaFreeAsync(r->src_order, stream);
   delete r;
