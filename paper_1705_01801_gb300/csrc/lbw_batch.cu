@@ -2110,6 +2110,12 @@ bool ragged_fits(const lbw_grid_desc& d) {
   // FP32 and FP64 only: 16-bit storage would round in another order than the kernel it has had;
   // smaller lattices run many steps per launch
   if ((d.prec != LBW_F32 && d.prec != LBW_F64) || nn <= (d.prec == LBW_F32 ? 640000 : 320000)) return false;
+  // two or three rows leave most of a tile's FP64 work to its halo: 2 x 200 x 3193 243 us a step, 326
+  // here, 3 x 120 x 1483 72 / 88; full-row tiles of many planes are ahead (2 x 100 x 19560 693 / 603)
+  if (d.prec == LBW_F64 && d.n[0] <= 3) {
+    const bool rows = row_tile_rows<9>(d.n[1], es) > 0;
+    if (d.n[0] < 3 ? !rows || nn < 1200000 : !rows && nn < 560000) return false;
+  }
   if (d.n[1] % kTmaBatchBX == 0 || d.bc[2] != LBW_BC_PERIODIC || d.bc[0] == LBW_BC_PERIODIC || d.n[0] < 2 ||
       d.n[1] < 2 * ghost_cols(es) || 7LL * d.n[0] * d.n[2] * padded_pitch(d.n[1], es) >= (1LL << 31))
     return false;
