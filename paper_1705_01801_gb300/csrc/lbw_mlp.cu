@@ -645,6 +645,23 @@ cudaError_t launch_forward(lbw_mlp* q, const FwdArgs& a, const WB* wt) {
   return cudaGetLastError();
 }
 
+template <typename WB>
+cudaError_t launch_forward_rows(lbw_mlp* q, const FwdArgs& a, const WB* wt) {
+  int widest = 0, units = 0;
+  for (int l = 0; l <= a.depth; ++l) widest = std::max(widest, a.dims[l]);
+  for (int l = 1; l <= a.depth; ++l) units = std::max(units, fwd_pad(a.dims[l]));
+  // a thread per unit; too few blocks to fill the SMs split the rows further
+  const int threads = a.n >= 8 * 152 * kFwdRows ? units : std::max(units, std::min(256, 4 * units));
+  bool splits = false;
+  for (int l = 0; l < a.depth; ++l) splits |= fwd_splits(a.dims[l], a.dims[l + 1], threads);
+  const size_t smem = sizeof(float) * kFwdRows * (2 * widest + (splits ? kFwdThreads : 0));
+  const cudaError_t e =
+      cudaFuncSetAttribute(forward_rows_kernel<WB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  forward_rows_kernel<WB><<<(a.n + kFwdRows - 1) / kFwdRows, threads, smem, q->stream>>>(a, wt);
+  return cudaGetLastError();
+}
+
 bool fits_forward(const lbw_mlp* q) {
   for (int w : q->dims)
     if (w > kFwdMaxWidth) return false;
@@ -684,9 +701,9 @@ lbw_status forward_fused(lbw_mlp* q, const float* host_x, int n, float* host_y, 
     valid = true;
   }
   // rows per CTA: more rows share a read of the weights, fewer fill the SMs
-  const cudaError_t e = n <= 4 * 152 ? launch_forward<WB, 4>(q, a, wt)
+  const cudaError_t e = n <= 4 * 152       ? launch_forward<WB, 4>(q, a, wt)
                         : n <= 8 * 2 * 152 ? launch_forward<WB, 8>(q, a, wt)
-                        : n <= 16 * 4 * 152 ? launch_forward<WB, 16>(q, a, wt) : launch_forward<WB, 32>(q, a, wt);
+                                           : launch_forward_rows<WB>(q, a, wt);
   if (e != cudaSuccess) return cuda_fail(e, "mlp forward");
   LBW_CUDA(cudaMemcpyAsync(host_y, a.y, sizeof(float) * ny, cudaMemcpyDeviceToHost, q->stream));
   LBW_CUDA(cudaStreamSynchronize(q->stream));

@@ -36,3 +36,17 @@ def _kernels(fake, spec):
 ])
 def test_kernel_of_a_lattice(fake, prec, n, kernel):
     assert _kernels(fake, W.GridSpec(n=n, prec=prec, **CART)) == {kernel}
+
+
+@pytest.mark.parametrize("rows,kernel", [(1, b"14forward_kernel"), (2432, b"14forward_kernel"),
+                                         (2433, b"19forward_rows_kernel"), (50000, b"19forward_rows_kernel")])
+def test_kernel_of_a_forward_pass(fake, rows, kernel):
+    """Splitting every layer's inputs over 512 threads made narrow networks of many rows 1.6 times
+    slower than a product per layer."""
+    import numpy as np
+    L = fake.lib()
+    net = fake.MLP(7, 16, 4, 8)
+    before = L.fake_launches(kernel), L.fake_launches(b"forward")
+    net.forward(np.zeros((rows, 7), np.float32))
+    assert (L.fake_launches(kernel) - before[0], L.fake_launches(b"forward") - before[1]) == (1, 1)
+    net.close()
