@@ -698,6 +698,7 @@ lbw_status forward_fused(lbw_mlp* q, const float* host_x, int n, float* host_y, 
     for (int l = 0; l < q->depth; ++l)
       pack_kernel<WB><<<dim3((a.dims[l] + 31) / 32, fwd_pad(a.dims[l + 1]) / 32), dim3(32, 8), 0, q->stream>>>(
           q->p + q->woff[l], a.dims[l], a.dims[l + 1], wt + a.woff[l]);
+    LBW_CUDA(cudaGetLastError());
     valid = true;
   }
   // rows per CTA: more rows share a read of the weights, fewer fill the SMs

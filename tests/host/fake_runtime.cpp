@@ -72,6 +72,11 @@ void fake_fail_allocation(int n) { g_fail_alloc = n; }
 void fake_largest_allocation(size_t bytes) { g_largest = bytes; }
 void fake_fail_launch(const char* part) { g_fail_launch = part; }
 void fake_elapsed(float (*f)()) { g_elapsed = f; }
+int fake_live() {
+  int n = 0;
+  for (const auto& b : g_blocks) n += b.second.live;
+  return n;
+}
 float fake_adam_correction() { return g_adam_correction; }
 int fake_launches(const char* part) {
   int n = 0;

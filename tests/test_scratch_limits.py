@@ -137,3 +137,19 @@ def test_ensemble_shapes_after_a_failed_allocation(fake, specs, call, all_behind
     b.step(3)  # the change that went through
     b.close()
     assert fake.lib().fake_errors() == b""
+
+
+def test_weights_are_packed_again_after_a_failed_launch(fake):
+    L = fake.lib()
+    net = fake.MLP(7, 16, 4, 8)
+    x = np.zeros((5, 7), np.float32)
+    L.fake_fail_launch(b"pack_kernel")
+    with pytest.raises(fake.LbwError):
+        net.forward(x)
+    L.fake_fail_launch(b"")
+    before = L.fake_launches(b"pack_kernel")
+    net.forward(x)
+    assert L.fake_launches(b"pack_kernel") - before == 4
+    net.forward(x)  # still those of the last change of the parameters
+    assert L.fake_launches(b"pack_kernel") - before == 4
+    net.close()
