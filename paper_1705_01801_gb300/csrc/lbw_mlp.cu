@@ -769,7 +769,20 @@ TrainPlan train_plan(const lbw_mlp* q, int rows) {
   return t;
 }
 
-// n_steps Adam steps on train_kernel; order, corrections and the loss curve on the device.
+// Device memory of one call, given back on every way out.
+struct Temporary {
+  void* p = nullptr;
+  cudaStream_t stream;
+  explicit Temporary(cudaStream_t s) : stream(s) {}
+  Temporary(const Temporary&) = delete;
+  ~Temporary() {
+    if (p) cudaFreeAsync(p, stream);
+  }
+  template <typename T> T* as() const { return static_cast<T*>(p); }
+};
+
+// n_steps Adam steps on train_kernel; order, corrections and the loss curve on the device.  adam_t counts
+// the steps launched.
 lbw_status train_fused(lbw_mlp* q, const TrainPlan& t, const int* d_order, const float2* d_corr, int n_steps, int rows,
                        float lr, float* d_curve) {
   const size_t layer = (size_t)rows * q->hidden, need = layer * (2 * (q->depth - 1) + q->depth);
@@ -824,6 +837,8 @@ lbw_status train_fused(lbw_mlp* q, const TrainPlan& t, const int* d_order, const
     cfg.numAttrs = 1;
     LBW_CUDA(with_train_kernel(t.npc, q->hidden, [&](auto kern) { return cudaLaunchKernelEx(&cfg, kern, a); }));
     if (a.steps & 1) std::swap(q->p, q->p2);
+    q->adam_t += a.steps;
+    params_changed(q);
   }
   return LBW_OK;
 }
@@ -1005,41 +1020,37 @@ lbw_status lbw_mlp_train(lbw_mlp* q, const float* host_x, const float* host_t, i
   if (q->data_n != n) {
     if (q->data_x) cudaFreeAsync(q->data_x, q->stream);
     if (q->data_t) cudaFreeAsync(q->data_t, q->stream);
+    q->data_x = q->data_t = nullptr;
+    q->data_n = 0;
     LBW_CUDA(cudaMallocAsync((void**)&q->data_x, sizeof(float) * n * q->in, q->stream));
     LBW_CUDA(cudaMallocAsync((void**)&q->data_t, sizeof(float) * n * q->out, q->stream));
     q->data_n = n;
   }
   LBW_CUDA(cudaMemcpyAsync(q->data_x, host_x, sizeof(float) * n * q->in, cudaMemcpyHostToDevice, q->stream));
   LBW_CUDA(cudaMemcpyAsync(q->data_t, host_t, sizeof(float) * n * q->out, cudaMemcpyHostToDevice, q->stream));
-  int* d_order = nullptr;
-  LBW_CUDA(cudaMallocAsync((void**)&d_order, sizeof(int) * (size_t)n_steps * batch, q->stream));
-  LBW_CUDA(cudaMemcpyAsync(d_order, host_order, sizeof(int) * (size_t)n_steps * batch, cudaMemcpyHostToDevice,
+  Temporary order(q->stream), curve(q->stream);
+  LBW_CUDA(cudaMallocAsync(&order.p, sizeof(int) * (size_t)n_steps * batch, q->stream));
+  LBW_CUDA(cudaMemcpyAsync(order.p, host_order, sizeof(int) * (size_t)n_steps * batch, cudaMemcpyHostToDevice,
                            q->stream));
-  float* d_curve = nullptr;
-  LBW_CUDA(cudaMallocAsync((void**)&d_curve, sizeof(float) * std::max(1, n_steps), q->stream));
+  LBW_CUDA(cudaMallocAsync(&curve.p, sizeof(float) * std::max(1, n_steps), q->stream));
+  const int* const d_order = order.as<int>();
+  float* const d_curve = curve.as<float>();
   if (plan.npc) {
     std::vector<float2> corr(std::max(1, n_steps));
     for (int s = 0; s < n_steps; ++s) {
-      ++q->adam_t;
-      corr[s] = make_float2((float)(1.0 - std::pow(0.9, (double)q->adam_t)), (float)(1.0 - std::pow(0.999, (double)q->adam_t)));
+      const double t = (double)(q->adam_t + s + 1);
+      corr[s] = make_float2((float)(1.0 - std::pow(0.9, t)), (float)(1.0 - std::pow(0.999, t)));
     }
-    float2* d_corr = nullptr;
+    Temporary d_corr(q->stream);
     int err = 0;
-    LBW_CUDA(cudaMallocAsync((void**)&d_corr, sizeof(float2) * corr.size(), q->stream));
-    LBW_CUDA(cudaMemcpyAsync(d_corr, corr.data(), sizeof(float2) * corr.size(), cudaMemcpyHostToDevice, q->stream));
-    st = train_fused(q, plan, d_order, d_corr, n_steps, batch, lr, d_curve);
-    cudaFreeAsync(d_corr, q->stream);
-    cudaError_t e = st == LBW_OK ? cudaGetLastError() : cudaSuccess;
-    if (st == LBW_OK && e == cudaSuccess)
-      e = cudaMemcpyAsync(&err, q->sync + 1, sizeof(int), cudaMemcpyDeviceToHost, q->stream);
-    if (st == LBW_OK && e == cudaSuccess && host_loss && n_steps > 0)
-      e = cudaMemcpyAsync(host_loss, d_curve, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, q->stream);
-    cudaFreeAsync(d_order, q->stream);
-    cudaFreeAsync(d_curve, q->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(q->stream);
-    params_changed(q);
+    LBW_CUDA(cudaMallocAsync(&d_corr.p, sizeof(float2) * corr.size(), q->stream));
+    LBW_CUDA(cudaMemcpyAsync(d_corr.p, corr.data(), sizeof(float2) * corr.size(), cudaMemcpyHostToDevice, q->stream));
+    st = train_fused(q, plan, d_order, d_corr.as<float2>(), n_steps, batch, lr, d_curve);
     if (st != LBW_OK) return st;
-    if (e != cudaSuccess) return cuda_fail(e, "mlp train");
+    LBW_CUDA(cudaMemcpyAsync(&err, q->sync + 1, sizeof(int), cudaMemcpyDeviceToHost, q->stream));
+    if (host_loss && n_steps > 0)
+      LBW_CUDA(cudaMemcpyAsync(host_loss, d_curve, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, q->stream));
+    LBW_CUDA(cudaStreamSynchronize(q->stream));
     if (err) return fail(LBW_ETIMEOUT, "a training step's bounded wait ran out; the parameters are undefined until "
                                        "lbw_mlp_set_params");
     return LBW_OK;
@@ -1056,14 +1067,12 @@ lbw_status lbw_mlp_train(lbw_mlp* q, const float* host_x, const float* host_t, i
                                                  (float)(1.0 - std::pow(0.9, (double)q->adam_t)),
                                                  (float)(1.0 - std::pow(0.999, (double)q->adam_t)));
   }
+  params_changed(q);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && host_loss && n_steps > 0)
     e = cudaMemcpyAsync(host_loss, d_curve, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, q->stream);
-  cudaFreeAsync(d_order, q->stream);
-  cudaFreeAsync(d_curve, q->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(q->stream);
   if (e != cudaSuccess) return cuda_fail(e, "mlp train");
-  params_changed(q);
   return LBW_OK;
 }
 

@@ -153,3 +153,46 @@ def test_weights_are_packed_again_after_a_failed_launch(fake):
     net.forward(x)  # still those of the last change of the parameters
     assert L.fake_launches(b"pack_kernel") - before == 4
     net.close()
+
+
+@pytest.mark.parametrize("hidden", [16, 18], ids=["one launch", "layer by layer"])
+def test_training_after_a_failed_allocation(fake, hidden):
+    """A call that could not train leaves the count of Adam's steps, frees what it took and names no
+    sample that it has freed."""
+    L = fake.lib()
+    x, t = np.zeros((20, 7), np.float32), np.zeros((20, 8), np.float32)
+    order = np.zeros((3, 8), np.int32)
+    grads = []
+    for n in range(1, 40):
+        net = fake.MLP(7, hidden, 4, 8)
+        net.train(x[:10], t[:10], order, 8, 1e-3)
+        net.set_params(net.get_params())  # counts from 0
+        L.fake_fail_allocation(n)
+        try:
+            net.train(x, t, order, 8, 1e-3)
+            done = 3
+        except fake.LbwError:
+            done = 0
+        L.fake_fail_allocation(0)
+        if not done:
+            net.train(x[:10], t[:10], order, 8, 1e-3)
+            done = 3
+        net.adam_step(np.zeros(net.nparam, np.float32), 1e-3)
+        grads.append(L.fake_adam_correction())
+        net.close()
+        assert L.fake_errors() == b"", n
+        assert abs(grads[-1] - (1 - 0.9 ** (done + 1))) < 1e-6, n
+
+
+def test_a_failed_training_call_frees_what_it_took(fake):
+    L = fake.lib()
+    net = fake.MLP(7, 16, 4, 8)
+    x, t, order = np.zeros((20, 7), np.float32), np.zeros((20, 8), np.float32), np.zeros((3, 8), np.int32)
+    net.train(x, t, order, 8, 1e-3)
+    live = L.fake_live()
+    for n in (1, 2, 3):
+        L.fake_fail_allocation(n)
+        with pytest.raises(fake.LbwError):
+            net.train(x, t, order, 8, 1e-3)
+        assert L.fake_live() == live, n
+    net.close()
