@@ -525,10 +525,14 @@ lbw_status spectrum_device(const double* d_x, int64_t T, int32_t count, int64_t 
                            int32_t* h_n, bool lowest, double rel_power) {
   size_t M = 1;
   while (M < 4 * (size_t)T) M <<= 1;
-  // as many estimates per pass as fit in 256 MB of workspace
-  const int per = (int)std::max<size_t>(1, std::min<size_t>(std::min(count, 4096), (256u << 20) / workspace_bytes(M, (size_t)T, 1, k)));
+  // as many estimates per pass as fit in 256 MB of workspace, or in what there is
+  int per = (int)std::max<size_t>(1, std::min<size_t>(std::min(count, 4096), (256u << 20) / workspace_bytes(M, (size_t)T, 1, k)));
   unsigned char* base = nullptr;
-  LBW_CUDA(cudaMallocAsync((void**)&base, workspace_bytes(M, (size_t)T, per, k), s));
+  while (cudaMallocAsync((void**)&base, workspace_bytes(M, (size_t)T, per, k), s) != cudaSuccess) {
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation || per == 1) return cuda_fail(e, "spectrum workspace");
+    per = (per + 1) / 2;
+  }
   const Work w = carve(base, M, (size_t)T, per, k);
   std::vector<double> res;
   cudaError_t e = cudaSuccess;

@@ -196,3 +196,14 @@ def test_a_failed_training_call_frees_what_it_took(fake):
             net.train(x, t, order, 8, 1e-3)
         assert L.fake_live() == live, n
     net.close()
+
+
+@pytest.mark.parametrize("n", [1, 16, 200])
+def test_spectra_in_smaller_passes_where_memory_is_short(fake, n):
+    """The estimates of a call share a workspace, but need no more memory than one after the other."""
+    T = 4096
+    fake.lib().fake_largest_allocation(max(8 * T * n, 5 * 10 ** 6))  # the series, or four estimates' workspace
+    assert len(fake.lbw_spectrum_series(np.zeros((n, T)), 4)) == n
+    fake.lib().fake_largest_allocation(8 * T * n - 1)
+    with pytest.raises(fake.LbwError):
+        fake.lbw_spectrum_series(np.zeros((n, T)), 4)
