@@ -337,21 +337,40 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
     lbw_destroy(g);
     return s;
   };
+  size_t fbytes = 0;
+  auto allocate = [&]() -> cudaError_t {  // both population buffers, or neither
+    fbytes = (size_t)7 * pop_stride(g) * g->elem;
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMallocAsync(&g->f[k], fbytes, g->stream);
+    if (e != cudaSuccess) cudaGetLastError();
+    for (int k = 0; k < 2 && e != cudaSuccess; ++k) {
+      if (g->f[k]) cudaFreeAsync(g->f[k], g->stream);
+      g->f[k] = nullptr;
+    }
+    return e;
+  };
+  // dense rows, for the kernels that need no memory of their own
+  auto forget_ragged = [&]() {
+    ragged_destroy(g);
+    g->pitch = g->col0 = 0;
+    for (void*& f : g->f) {
+      if (f) cudaFreeAsync(f, g->stream);
+      f = nullptr;
+    }
+  };
   if (d.geom_mode != LBW_GEOM_ANALYTIC && ragged_fits(d)) {
     st = ragged_plan(g);
     if (st != LBW_OK) return cleanup(st);
   }
-  const size_t fbytes = (size_t)7 * pop_stride(g) * g->elem;
-  for (int k = 0; k < 2; ++k) {
-    cudaError_t e = cudaMallocAsync(&g->f[k], fbytes, g->stream);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return cleanup(fail(LBW_ENOMEM, std::string("population buffers: ") + cudaGetErrorString(e)));
-    }
+  cudaError_t e = allocate();
+  if (e != cudaSuccess && g->ragged) {  // no room for the longer rows
+    forget_ragged();
+    e = allocate();
   }
+  if (e != cudaSuccess) return cleanup(fail(LBW_ENOMEM, std::string("population buffers: ") + cudaGetErrorString(e)));
   const size_t rs = real_size(d.prec);
   const size_t tbytes = tab.size() * rs;
-  cudaError_t e = cudaMallocAsync(&g->table, tbytes, g->stream);
+  e = cudaMallocAsync(&g->table, tbytes, g->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&g->counters, 6 * sizeof(unsigned long long), g->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -368,12 +387,13 @@ lbw_status lbw_create_grid(const lbw_grid_desc* desc, void* stream, lbw_grid** o
   if (e == cudaSuccess) e = cudaMemsetAsync(g->f[0], 0, fbytes, g->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "create: upload"));
-  if (g->ragged) {
-    st = ragged_refresh(g);
-    if (st != LBW_OK) return cleanup(st);
-  } else {
-    step_launch_shape(g);
+  if (g->ragged && ragged_refresh(g) != LBW_OK) {  // no room for its work list or maps
+    forget_ragged();
+    e = allocate();
+    if (e == cudaSuccess) e = cudaMemsetAsync(g->f[0], 0, fbytes, g->stream);
+    if (e != cudaSuccess) return cleanup(fail(LBW_ENOMEM, std::string("population buffers: ") + cudaGetErrorString(e)));
   }
+  if (!g->ragged) step_launch_shape(g);
   if (d.geom_mode == LBW_GEOM_ANALYTIC && g->tma_by == 0)
     return cleanup(fail(LBW_EINVAL, "geom_mode ANALYTIC needs the tile kernel: q2 extent a multiple of "
                                     "the tile width (64, or 128 for 16-bit storage) and non-periodic q1"));

@@ -751,7 +751,9 @@ lbw_status resident_create(const Grid* const* lattices, int n, int prec, bool ti
   }
   if (e != cudaSuccess) {
     resident_destroy(p, stream);
-    return cuda_fail(e, "resident step kernel: upload");
+    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "resident step kernel: upload");
+    cudaGetLastError();
+    return LBW_OK;  // a launch per step needs no memory of its own
   }
   *out = p;
   return LBW_OK;

@@ -207,3 +207,40 @@ def test_spectra_in_smaller_passes_where_memory_is_short(fake, n):
     fake.lib().fake_largest_allocation(8 * T * n - 1)
     with pytest.raises(fake.LbwError):
         fake.lbw_spectrum_series(np.zeros((n, T)), 4)
+
+
+@pytest.mark.parametrize("failing", range(1, 9))
+@pytest.mark.parametrize("spec", [SMALL, RAGGED, TILED], ids=["small", "ragged", "tiled"])
+def test_creation_needs_no_more_memory_than_the_lattice(fake, spec, failing):
+    """Of a lattice's allocations only its populations, table and counters have to succeed: without the
+    rest (or the longer rows of the ensemble kernels) it runs on the kernels that need none of it."""
+    L = fake.lib()
+    L.fake_fail_allocation(failing)
+    try:
+        g = fake.Grid(spec)
+    except fake.LbwError:
+        assert failing <= 4  # f, f, table, counters
+        return
+    finally:
+        L.fake_fail_allocation(0)
+    g.init(W.pulses(spec, 1, 1, margin=0))
+    g.set_probes([[1, 1, 1]], 100)
+    g.step(3)
+    g.close()
+    assert L.fake_errors() == b""
+
+
+def test_ragged_lattice_without_room_for_its_padding(fake):
+    """350 columns are stored in rows of 360 with ghost columns; where only the lattice itself fits it is
+    stored densely."""
+    L = fake.lib()
+    spec = W.cylinder(40, 350, 60)
+    L.fake_largest_allocation(7 * 4 * spec.nodes)
+    g = fake.Grid(spec)
+    L.fake_largest_allocation(2 ** 63)
+    g.init(W.pulses(spec, 1, 1, margin=0))
+    before = L.fake_launches(b"11step_kernel")
+    g.step(3)
+    assert L.fake_launches(b"11step_kernel") == before + 3
+    g.close()
+    assert L.fake_errors() == b""
