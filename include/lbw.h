@@ -298,7 +298,8 @@ lbw_status lbw_batch_get_populations(lbw_batch* b, int32_t member, double* host_
  * (tile rows 4 or 7 of 64 columns, or 0: full-row tiles, each member's whole rows with a
  * height that follows its row length, offered when every member fits one and the storage
  * is 32- or 64-bit; CTAs per SM 1/2); others the register-pipelined kernel (rows 4/8/16,
- * CTAs per SM 1/2/4); planes per q3 segment 16/32/64 for both.  With a cache_path (JSON
+ * CTAs per SM 1/2/4); planes per q3 segment 16/32/64 for both; and the shape that the ensemble
+ * has (and the multi-step kernel where it has that).  With a cache_path (JSON
  * lines), a shape stored for the same ensemble signature is reused without timing and a new
  * choice is appended.  The trial steps run on the ensemble's buffers: call it before
  * lbw_batch_init.  A text report of the timings goes to report (may be NULL). */

@@ -1954,7 +1954,7 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
   if (!cached) {
     // register-pipelined kernel: rows {4, 8, 16} x CTAs per SM {1, 2, 4}; TMA-staged kernel:
     // rows {4, 7} and full-row tiles (by = 0, where every member fits one) x CTAs per SM
-    // {1, 2}; both x segment planes {16, 32, 64}
+    // {1, 2}; both x segment planes {16, 32, 64}; and the shape that the ensemble has
     std::vector<int> bys = b->tma ? std::vector<int>{4, 7} : std::vector<int>{4, 8, 16};
     if (b->rowk) bys.push_back(0);
     std::vector<int> cpss = b->tma ? std::vector<int>{1, 2} : std::vector<int>{1, 2, 4};
@@ -2017,10 +2017,11 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
       }
       return LBW_OK;
     };
-    lbw_status st = LBW_OK;
+    lbw_status st = try_shape(start);
     for (int by : bys)
       for (int lz : lzs)
         for (int cps : cpss) {
+          if (by == start.by && lz == start.lz && cps == start.cps) continue;
           const int cps_max = b->tma ? tma_cps(b->prec, by) : (b->prec == LBW_F32 ? max_cps<float>() : 2);
           if (st == LBW_OK && cps <= cps_max) st = try_shape(Shape{by, lz, cps});
         }
