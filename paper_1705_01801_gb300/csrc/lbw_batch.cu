@@ -1060,6 +1060,7 @@ struct lbw_batch {
   bool rowk = false;             // ... and every member fits a full-row tile (shape.by == 0)
   void* maps = nullptr;          // device: per member tensor maps (buffer 0, buffer 1, table)
   Resident* res = nullptr;       // small members: many steps per launch (nullptr: a launch per step)
+  bool small = false;            // it had one when it was created
   // harmonic sources of all members (offsets from the buffer base), applied after each step
   int nsrc = 0, src_kind = 0;
   double src_amp = 0.0;
@@ -1581,7 +1582,10 @@ lbw_status batch_counters(lbw_batch* b, unsigned long long* recorded) {
   return LBW_OK;
 }
 
+// Names what a tuned shape depends on: members, storage, the kernels (kForms counts their forms, as a
+// shape stands for another kernel when they change) and whether the multi-step kernel is among them.
 std::string signature(const lbw_batch* b) {
+  constexpr int kForms = 2;
   unsigned long long h = 1469598103934665603ULL;  // FNV-1a over the members' sizes
   for (const Grid& g : b->views)
     for (int a = 0; a < 3; ++a) {
@@ -1590,7 +1594,7 @@ std::string signature(const lbw_batch* b) {
     }
   std::ostringstream s;
   s << "n" << b->n << "-p" << b->prec << (b->tma ? "-tma" : "-reg") << "-nodes" << b->total_nodes << "-h"
-    << std::hex << h;
+    << std::hex << h << "-k" << std::dec << kForms << (b->small ? "-many" : "");
   return s.str();
 }
 
@@ -1728,6 +1732,7 @@ lbw_status lbw_batch_create(const lbw_grid_desc* descs, int32_t n, void* stream,
   st = resident_create(lattices.data(), n, b->prec, b->tma,
                        !b->tma || b->prec == LBW_F64 ? 1LL << 40 : (wide ? 640000 : 300000), b->stream, &b->res);
   if (st != LBW_OK) return cleanup(st);
+  b->small = b->res != nullptr;
   LBW_CUDA(cudaStreamSynchronize(b->stream));
   *out = b;
   return LBW_OK;
@@ -1940,11 +1945,12 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
     while (in && std::getline(in, line)) {
       if (line.find("\"" + sig + "\"") == std::string::npos) continue;
       Shape s;
-      resident = line.find("\"resident\": 1") != std::string::npos;
-      if (sscanf(line.c_str() + line.find("\"by\""), "\"by\": %d, \"lz\": %d, \"cps\": %d", &s.by, &s.lz,
-                 &s.cps) == 3) {
+      const size_t at = line.find("\"by\"");
+      if (at != std::string::npos &&
+          sscanf(line.c_str() + at, "\"by\": %d, \"lz\": %d, \"cps\": %d", &s.by, &s.lz, &s.cps) == 3) {
         best = s;
         cached = true;
+        resident = b->res && line.find("\"resident\": 1") != std::string::npos;
       }
     }
   }

@@ -51,3 +51,25 @@ def test_the_shape_it_starts_with_is_among_those_timed(fake):
         _tune(fake, b, lambda info, resident: 1.0 if info == start else 2.0)
         assert b.info() == start
         b.close()
+
+
+def test_cache_lines_of_other_kernels_are_not_taken(fake, tmp_path):
+    """A line of the same sizes written before there was a multi-step kernel (no field for it, another
+    signature), or for an ensemble that does not offer it, says nothing about this one."""
+    cache = tmp_path / "tune.jsonl"
+    table = fake.Batch([s.with_(geom_mode=W.GEOM_TABLE) for s in SMALL])
+    _tune(fake, table, lambda info, resident: 1.0, cache_path=str(cache))
+    line = json.loads(cache.read_text())
+    old = dict(line, signature=line["signature"].split("-k")[0])
+    cache.write_text(json.dumps(old) + "\n" + json.dumps(line) + "\n")
+    table.close()
+    b = fake.Batch(SMALL)
+    report = _tune(fake, b, lambda info, resident: 0.1 if resident else 1.0, cache_path=str(cache))
+    assert "cached" not in report and "resident" in report
+    assert _steps_on(fake, b, b"15resident_kernel")
+    b.close()
+    b = fake.Batch(SMALL)  # its own line is
+    assert "cached resident" in _tune(fake, b, lambda info, resident: 1.0, cache_path=str(cache))
+    assert _steps_on(fake, b, b"15resident_kernel")
+    b.close()
+    assert fake.lib().fake_errors() == b""
