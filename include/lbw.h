@@ -219,13 +219,15 @@ lbw_status lbw_set_populations(lbw_grid* g, const double* host_f);
 lbw_status lbw_step_count(lbw_grid* g, int64_t* out);
 
 /* Failure injection for tests of the timeout path; the paper has no counterpart.  From the
- * next time step on, the step kernel's consumer warps wait on a barrier that no copy ever
- * completes.  The bounded wait runs out after a few hundred tries (under a millisecond), the
- * step raises its timeout flag, and every CTA leaves once the copies it issued have landed,
- * exactly as after a lost copy, with no device fault and no hang.  Calls that synchronise
- * then return LBW_ETIMEOUT; lbw_init clears the request and the flag.  LBW_ESTATE before
- * lbw_init; LBW_EINVAL on lattices that run the register-pipelined kernel (q2 extent not a
- * multiple of the tile width, or periodic q1), which has no device waits. */
+ * next time step on, the tile kernel's consumer warps wait on a barrier that no copy ever
+ * completes (the multi-step kernel's blocks: on an arrival that never comes).  The bounded wait
+ * runs out after a few hundred tries (under a millisecond), the step raises its timeout flag, and
+ * every CTA leaves once the copies it issued have landed, exactly as after a lost copy, with no
+ * device fault and no hang.  Calls that synchronise then return LBW_ETIMEOUT; lbw_init clears the
+ * request and the flag.  LBW_ESTATE before lbw_init; LBW_EINVAL on lattices that are not of the
+ * tile kernel's shape (q2 extent not a multiple of the tile width, or periodic q1): the
+ * register-pipelined kernel has no device waits, and the injection is not built into the
+ * ensemble kernels that step large ragged lattices. */
 lbw_status lbw_inject_wait_timeout(lbw_grid* g);
 
 /* Frees the grid's device memory (stream-ordered) and graphs; NULL is allowed. */
@@ -313,7 +315,8 @@ lbw_status lbw_batch_tune(lbw_batch* b, int32_t trial_steps, const char* cache_p
  * gives the same numbers). */
 lbw_status lbw_batch_set_shape(lbw_batch* b, int32_t tile_rows, int32_t seg_planes, int32_t ctas_per_sm);
 
-/* Total nodes and the launch shape in use (any pointer may be NULL). */
+/* Total nodes and the launch shape (any pointer may be NULL): the one in use, or where the
+ * multi-step kernel advances the ensemble, which has none, the one that launches per step take. */
 lbw_status lbw_batch_info(lbw_batch* b, int64_t* total_nodes, int32_t* tile_rows, int32_t* seg_planes,
                           int32_t* ctas_per_sm);
 
@@ -348,9 +351,11 @@ lbw_status lbw_mlp_grad(lbw_mlp* q, const float* host_x, const float* host_t, in
 lbw_status lbw_mlp_adam_step(lbw_mlp* q, const float* host_grad, float lr);
 /* n_steps Adam steps on minibatches of `batch` rows of the n samples: step s uses rows
  * host_order[s * batch .. s * batch + batch - 1] (the caller draws the order).  host_loss
- * (may be NULL) receives the minibatch loss before each step.  Hidden widths that are multiples of
- * 4 up to 512 with at most 64 inputs, 16 outputs and 512 rows train in one cooperative launch per
- * 1024 steps, whose bounded waits return LBW_ETIMEOUT when one runs out. */
+ * (may be NULL) receives the minibatch loss before each step.  Networks of two
+ * layers and more whose hidden width is a multiple of 4 up to 512, with at most 64 inputs, 16 outputs
+ * (and a CTA for each) and 512 rows, train in one cooperative launch per 1024 steps where a CTA's
+ * share of weights and rows fits its shared memory; its bounded waits return LBW_ETIMEOUT when one
+ * runs out.  Others take a sequence of launches per step. */
 lbw_status lbw_mlp_train(lbw_mlp* q, const float* host_x, const float* host_t, int32_t n,
                          const int32_t* host_order, int32_t n_steps, int32_t batch, float lr, float* host_loss);
 void lbw_mlp_destroy(lbw_mlp* q);

@@ -491,7 +491,8 @@ lbw_status lbw_inject_wait_timeout(lbw_grid* g) {
   if (!g) return fail(LBW_EINVAL, "grid is NULL");
   if (!g->initialised) return fail(LBW_ESTATE, "lbw_inject_wait_timeout before lbw_init");
   if (g->tma_by == 0)
-    return fail(LBW_EINVAL, "this lattice runs the register-pipelined step kernel, which has no device waits");
+    return fail(LBW_EINVAL, "the injected timeout is built for lattices of the tile kernel's shape: q2 extent a "
+                            "multiple of the tile width, walls in q1");
   // any non-zero value requests the injected timeout; lbw_init clears it
   LBW_CUDA(cudaMemsetAsync(g->counters + 4, 0xff, sizeof(unsigned long long), g->stream));
   LBW_CUDA(cudaStreamSynchronize(g->stream));

@@ -5,7 +5,8 @@
 // whole ensemble is one launch of a persistent kernel whose CTAs walk a work list of
 // (member, q2 tile, q1 tile, q3 segment) items and run the same register-pipelined tile march
 // as the single-lattice kernel (lbw_march.cuh), so a member's numbers do not depend on the
-// batching.  Steps are captured in CUDA-graph chains.  lbw_batch_tune times candidate tile
+// batching; members that wrap in q2 run on the TMA-staged kernels below, small ones on the multi-step
+// kernel (lbw_resident.cu).  Steps are captured in CUDA-graph chains.  lbw_batch_tune times candidate tile
 // shapes (rows per tile, planes per q3 segment, CTAs per SM) on the ensemble and keeps the
 // fastest, optionally persisting it in a JSON-lines cache keyed by the ensemble's signature.
 #include <cuda_runtime.h>
@@ -2114,8 +2115,9 @@ namespace lbw {
 bool ragged_fits(const lbw_grid_desc& d) {
   const size_t es = es_of(d.prec);
   const long long nn = (long long)d.n[0] * d.n[1] * d.n[2];
-  // FP32 and FP64 only: 16-bit storage would round in another order than the kernel it has had;
-  // smaller lattices run many steps per launch
+  // FP32 and FP64 only: 16-bit storage would round in another order than the kernel it has had.  Most
+  // smaller lattices run many steps per launch; those that find no boxes near its capacity (100 x 100 x
+  // 61 FP32) and those of geom_mode TABLE stay on the register-pipelined kernel.
   if ((d.prec != LBW_F32 && d.prec != LBW_F64) || nn <= (d.prec == LBW_F32 ? 640000 : 320000)) return false;
   // two or three rows leave most of a tile's FP64 work to its halo: 2 x 200 x 3193 243 us a step, 326
   // here, 3 x 120 x 1483 72 / 88; full-row tiles of many planes are ahead (2 x 100 x 19560 693 / 603)

@@ -20,7 +20,8 @@
 // point, a radix-16 pass about 20 and does the work of four; golden section on the sums takes
 // 81 x 8 a sample and peak, the moments about 40, spread over all SMs instead of one CTA per peak.
 // Measured, 16 host series of 20,000 samples with 8 peaks each, one after the other -> here:
-// 62.2 -> 0.86 ms (moments 0.30, four FFT passes 0.17, search 0.10, selection 0.08, power 0.06);
+// 62.2 -> 1.07 ms a call (0.86 in the kernels: moments 0.30, four FFT passes 0.17, search 0.10,
+// selection 0.08, power 0.06);
 // one series of 20,000: 4.1 -> 0.46 ms, of 256: 0.97 -> 0.41 ms.
 #include <cuda.h>
 #include <cuda_runtime.h>

@@ -50,3 +50,14 @@ def test_kernel_of_a_forward_pass(fake, rows, kernel):
     net.forward(np.zeros((rows, 7), np.float32))
     assert (L.fake_launches(kernel) - before[0], L.fake_launches(b"forward") - before[1]) == (1, 1)
     net.close()
+
+
+def test_the_injected_timeout_says_where_it_is_built(fake):
+    """It is refused on ragged lattices, but not because their kernels had no waits."""
+    for n in ((20, 33, 10), (100, 100, 70)):
+        g = fake.Grid(W.cylinder(*n))
+        g.init(W.pulses(g.spec, 1, 1, margin=0))
+        with pytest.raises(fake.LbwError) as e:
+            fake.lbw_inject_wait_timeout(g.handle)
+        assert e.value.status == fake.LBW_EINVAL and "tile width" in str(e.value) and "no device waits" not in str(e.value)
+        g.close()
