@@ -433,19 +433,20 @@ unsigned read_blocks(const Grid* g) {
 }
 
 // Room for `per` planes of doubles on the device: the other population buffer, which holds 1 to 7, or
-// for small lattices a temporary of all seven where it can be had, as every turn costs a launch and a
-// copy of its own (64 FP32 nodes 85 -> 42 us, 262,144 557 -> 380).
+// a temporary of all seven (up to `limit` bytes, where it can be had), as every turn costs a launch and
+// a copy of its own and a large temporary is slow to map.  FP32, through the buffer / a temporary: read
+// 64 nodes 68 / 31 us, 262,144 488 / 375, 512,000 930 / 815, 1e6 2320 / 2560; written 28 / 19, 133 / 115,
+// 210 / 305, 390 / 545.
 struct Planes {
   Grid* g;
   double* d;
   int per;
   bool own = false;
-  explicit Planes(Grid* grid) : g(grid), d(static_cast<double*>(grid->f[1 - grid->cur])) {
-    constexpr long long kTemporary = 64 << 20;
+  Planes(Grid* grid, long long limit) : g(grid), d(static_cast<double*>(grid->f[1 - grid->cur])) {
     const long long all = 7LL * 8 * g->nn;
     per = (int)std::max<long long>(1, std::min<long long>(7, 7 * pop_stride(g) * (long long)g->elem / (8 * g->nn)));
     void* t = nullptr;
-    if (per == 7 || all > kTemporary) return;
+    if (per == 7 || all > limit) return;
     if (cudaMallocAsync(&t, (size_t)all, g->stream) != cudaSuccess) {
       cudaGetLastError();
       return;
@@ -523,7 +524,7 @@ cudaError_t read_field(Grid* g, double* host_P, unsigned long long* d_bad) {
 }
 
 cudaError_t read_populations(Grid* g, double* host_f) {
-  const Planes p(g);
+  const Planes p(g, 32 << 20);
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 7 && e == cudaSuccess; i += p.per) {
     const int n = std::min(p.per, 7 - i);
@@ -542,7 +543,7 @@ cudaError_t read_populations(Grid* g, double* host_f) {
 }
 
 cudaError_t write_populations(Grid* g, const double* host_f) {
-  const Planes p(g);
+  const Planes p(g, 16 << 20);
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 7 && e == cudaSuccess; i += p.per) {
     const int n = std::min(p.per, 7 - i);
