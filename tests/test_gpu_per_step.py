@@ -170,3 +170,26 @@ def test_injected_wait_timeout_per_step(spec):
     g.step(80)
     np.testing.assert_array_equal(g.get_f(), want)
     g.close()
+
+
+@pytest.mark.parametrize("prec,tol", [(W.PREC_F64, 1e-11), (W.PREC_F32, 2e-5)], ids=["f64", "f32"])
+@pytest.mark.parametrize("spec", [
+    W.disk(1000, 701), W.disk(2700, 250),
+    W.GridSpec(kind=W.KIND_CARTESIAN, n=(900, 801, 1), h=(1, 1, 1), x0=(0, 0, 0), c=0.4, bc=(1, 2, 0, 0, 1, 3)),
+    W.GridSpec(kind=W.KIND_CARTESIAN, n=(130, 2601, 2), h=(1, 1, 1), x0=(0, 0, 0), c=0.4, bc=(3, 1, 0, 0, 2, 1)),
+    W.GridSpec(kind=W.KIND_CARTESIAN, n=(2, 300, 1200), h=(1, 1, 1), x0=(0, 0, 0), c=0.4, bc=(3, 1, 0, 0, 0, 0))],
+    ids=["disk", "disk rows", "plane", "two planes", "two rows"])
+def test_large_thin_ragged_lattices_match_oracle(spec, prec, tol):
+    """Ragged lattices of one or two planes (or rows) beyond the multi-step kernel's capacity."""
+    from paper_1705_01801_gb300 import lbw
+    spec = spec.with_(prec=prec)
+    pl, pr = W.pulses(spec, 7, 6, sigma=9.0, random_phase=True, margin=0), W.probes(spec, 7, 5, margin=0)
+    g, o = lbw.Grid(spec), oracle.OracleGrid(spec)
+    for s in (g, o):
+        s.init(pl)
+        s.set_probes(pr, 25)
+        s.step(25)
+    fo, so = o.get_f(), o.read_probes()
+    np.testing.assert_allclose(g.get_f(), fo, rtol=0, atol=tol * np.abs(fo).max())
+    np.testing.assert_allclose(g.read_probes(), so, rtol=0, atol=10 * tol * np.abs(fo).max())
+    g.close()
